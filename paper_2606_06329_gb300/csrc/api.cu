@@ -560,7 +560,7 @@ mecuco_status run_curvature(mecuco_t h, char *ws, const void *X, mecuco_dtype dt
             LAUNCH(h, MECUCO_STAGE_GRAM, s, launch_gram_tc(dt, sg, nullptr, 0, np, haar, h->wait_limit, h->ctr, s));
             LAUNCH(h, MECUCO_STAGE_JACOBI, s,
                    launch_jacobi_seg(sg, nullptr, 0, k, np, fp64, h->jacobi_max_sweeps, h->ctr, s, kJacobiPreLoose,
-                                 h->jacobi_warp));
+                                     h->jacobi_warp, true));
             if (fp64 == 1 || fp64 == 3) ++h->launches;  // the refinement is a second kernel
             LAUNCH(h, MECUCO_STAGE_ROTATE, s,
                    launch_rotate_tc(dt, sg, nullptr, 0, np, b.Y, rot_ld(m), h->wait_limit, h->ctr, s));
@@ -574,7 +574,7 @@ mecuco_status run_curvature(mecuco_t h, char *ws, const void *X, mecuco_dtype dt
             LAUNCH(h, MECUCO_STAGE_GRAM, s,
                    launch_patch_gram(X, dt, N, m, ld, nb, k, 0, np, nullptr, b.G, b.R, nullptr, h->ctr, s));
             LAUNCH(h, MECUCO_STAGE_JACOBI, s, launch_jacobi(b.G, k, np, 1, h->jacobi_max_sweeps, b.sig, b.U0, h->ctr, s,
-                                 kJacobiPreTight, h->jacobi_warp));
+                                 kJacobiPreTight, h->jacobi_warp, true));
             ++h->launches;
             LAUNCH(h, MECUCO_STAGE_GRAM, s,
                    launch_patch_gram(X, dt, N, m, ld, nb, k, 0, np, b.U0, b.G, b.R, var == MECUCO_FAST_HAAR ? b.Q : nullptr,
@@ -708,6 +708,7 @@ struct BatchChunk {
     int kmax;
     int64_t ldy;   // leading dimension of the rotated patches (BF16 elements)
     uint16_t *Y;
+    int64_t jwarps;  // warps of the register-resident eigensolve
 };
 
 struct BatchPlan {
@@ -807,7 +808,7 @@ mecuco_status plan_batch(mecuco_t h, const mecuco_dataset *sets, int nsets, mecu
     // estimator chunks: greedy over the points in table order
     const int64_t pt_cap = h->chunk_points > 0 ? h->chunk_points : ((int64_t)1 << 24);
     size_t est_end = after_idx;
-    BatchChunk cur{0, 0, 0, 0, 0, nullptr};
+    BatchChunk cur{0, 0, 0, 0, 0, nullptr, 0};
     auto close = [&]() {
         if (cur.np == 0) return;
         Carver e(base, after_idx);
@@ -826,7 +827,7 @@ mecuco_status plan_batch(mecuco_t h, const mecuco_dataset *sets, int nsets, mecu
             g.U = b.U + f * kk * kk;
         }
         p.chunks.push_back(cur);
-        cur = BatchChunk{0, (int)p.segs.size(), 0, 0, 0, nullptr};
+        cur = BatchChunk{0, (int)p.segs.size(), 0, 0, 0, nullptr, 0};
     };
     for (int t = 0; t < nsets; ++t) {
         const mecuco_dataset &d = sets[p.order[t]];
@@ -845,6 +846,9 @@ mecuco_status plan_batch(mecuco_t h, const mecuco_dataset *sets, int nsets, mecu
             g.ld = d.ld;
             g.k = d.k;
             g.first = (int)cur.np;
+            g.npts = (int)take;
+            g.jfirst = (int)cur.jwarps;
+            cur.jwarps += jacobi_reg_warps(d.k, take);
             g.rowtab = h->tttab[d.k];
             p.segs.push_back(g);
             p.refs.push_back(SegRef{t, 0, a});
@@ -943,7 +947,7 @@ mecuco_status run_batched_persistent(mecuco_t h, const mecuco_dataset *sets, int
         LAUNCH(h, MECUCO_STAGE_GRAM, s, launch_gram_tc(dt, none, tab, ch.nseg, ch.np, haar, h->wait_limit, h->ctr, s));
         LAUNCH(h, MECUCO_STAGE_JACOBI, s,
                launch_jacobi_seg(none, tab, ch.nseg, ch.kmax, ch.np, fp64, h->jacobi_max_sweeps, h->ctr, s,
-                                 kJacobiPreLoose, h->jacobi_warp));
+                                 kJacobiPreLoose, h->jacobi_warp, true, ch.jwarps));
         if (fp64 == 1 || fp64 == 3) ++h->launches;
         LAUNCH(h, MECUCO_STAGE_ROTATE, s,
                launch_rotate_tc(dt, none, tab, ch.nseg, ch.np, ch.Y, ch.ldy, h->wait_limit, h->ctr, s));

@@ -38,6 +38,8 @@ struct PatchSeg {
     int64_t N, m, ld;
     int k;
     int first;                // first point (block) of the launch in this segment
+    int npts;                 // points of the segment
+    int jfirst;               // first warp of the segment in the register-resident eigensolve
     const int32_t *idx;       // neighbour lists (k per point)
     const int32_t *rowtab;    // third-moment pass: row table for this k
     float *G, *R, *Q;         // k x k, k, k x k per point

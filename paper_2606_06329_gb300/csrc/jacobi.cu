@@ -603,7 +603,8 @@ size_t jacobi_smem_bytes(int k, int fp64) {
 }
 
 cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t np, int fp64,
-                              int max_sweeps, DevCounters *ctr, cudaStream_t s, float pre_eps, int warp_form) {
+                              int max_sweeps, DevCounters *ctr, cudaStream_t s, float pre_eps, int warp_form,
+                              bool refined_only, int64_t reg_warps) {
     if (np <= 0) return cudaSuccess;
     if (kmax > 64 || kmax < 1) return cudaErrorInvalidValue;
     cudaError_t e;
@@ -619,7 +620,19 @@ cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab
     };
     if (fp64 == 1 || fp64 == 3) {
         // FP32 sweeps, then one refinement step (3: relative cluster test)
-        e = sweeps32(pre_eps);
+        if (refined_only && fp64 == 1 && warp_form == 2) {
+            // |cos| of the last sweep: the step after it squares what is left
+            const float stop = pre_eps >= kJacobiPreLoose ? 9.765625e-04f : 1.220703125e-04f;  // 2^-10, 2^-13
+            PatchSeg seg = one;
+            if (ntab == 0) {
+                seg.npts = (int)np;
+                seg.jfirst = 0;
+                reg_warps = jacobi_reg_warps(one.k, np);
+            }
+            e = launch_jacobi_reg(seg, tab, ntab, kmax, reg_warps, max_sweeps, stop, ctr, s);
+        } else {
+            e = sweeps32(pre_eps);
+        }
         if (e != cudaSuccess) return e;
         // threads per patch: 64 (k <= 16), 128 (k <= 32) or 256, so that small
         // patches are not limited to 8 per SM by idle threads
@@ -645,13 +658,13 @@ cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab
 }
 
 cudaError_t launch_jacobi(const float *G, int k, int64_t np, int fp64, int max_sweeps, float *sigma, float *U,
-                          DevCounters *ctr, cudaStream_t s, float pre_eps, int warp_form) {
+                          DevCounters *ctr, cudaStream_t s, float pre_eps, int warp_form, bool refined_only) {
     PatchSeg one{};
     one.k = k;
     one.G = const_cast<float *>(G);
     one.sig = sigma;
     one.U = U;
-    return launch_jacobi_seg(one, nullptr, 0, k, np, fp64, max_sweeps, ctr, s, pre_eps, warp_form);
+    return launch_jacobi_seg(one, nullptr, 0, k, np, fp64, max_sweeps, ctr, s, pre_eps, warp_form, refined_only);
 }
 
 }  // namespace mecuco

@@ -223,16 +223,29 @@ cudaError_t launch_tthird_tc(const PatchSeg &one, const PatchSeg *tab, int ntab,
 // rotated Gram must come out nearly diagonal, take kJacobiPreTight.
 constexpr float kJacobiPreTight = 2.384185791015625e-07f;  // 2^-22
 constexpr float kJacobiPreLoose = 6.103515625e-05f;        // 2^-14
+// refined_only: the caller needs the eigenpairs after the refinement step
+// (fp64 = 1) only to its accuracy, so the FP32 sweeps may be the
+// register-resident one-sided form (jacobi_reg.cu), taken with warp_form = 2
+// (the default): 4 to 9 times faster than the fused two-sided form at every k
+// measured (jacobi_reg.cu).  Callers whose results follow the eigenvectors of
+// near-degenerate pairs (Exact mode, the adjoint) keep the two-sided sweeps.
 // warp_form != 0: the FP32 sweeps run one warp per patch (fused 2 x 2 block
 // updates, no block barriers); 0: one CTA of 128 threads per patch.  FP64
 // sweeps (fp64 = 2) always take the CTA form.
 cudaError_t launch_jacobi(const float *G, int k, int64_t np, int fp64, int max_sweeps,
                           float *sigma, float *U, DevCounters *ctr, cudaStream_t s,
-                          float pre_eps = kJacobiPreTight, int warp_form = 1);
+                          float pre_eps = kJacobiPreTight, int warp_form = 1, bool refined_only = false);
 // The same over a segment table (PatchSeg: G, k, sig, U of each segment);
 // kmax bounds every segment's k.
 cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t np, int fp64,
-                              int max_sweeps, DevCounters *ctr, cudaStream_t s, float pre_eps, int warp_form = 1);
+                              int max_sweeps, DevCounters *ctr, cudaStream_t s, float pre_eps, int warp_form = 1,
+                              bool refined_only = false, int64_t reg_warps = 0);
+// Register-resident one-sided sweeps: nwarps warps in all, each on
+// jacobi_reg_warps()'s share of one segment's patches (PatchSeg: k, npts,
+// jfirst, G, sig, U); stop_cos bounds |cos| between columns in the last sweep.
+int64_t jacobi_reg_warps(int k, int64_t np);
+cudaError_t launch_jacobi_reg(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t nwarps,
+                              int max_sweeps, float stop_cos, DevCounters *ctr, cudaStream_t s);
 
 // ---- Step 4: k-space estimator ----------------------------------------------
 // sigma/U from launch_jacobi, M pair-major from launch_patch_m3, R and Q from
