@@ -138,15 +138,15 @@ typedef enum {
                                         dataset group, as the FP32 form always does.  Results identical */
     MECUCO_OPT_JACOBI_WARP = 16,     /* FP32 Jacobi sweeps.  2 (default): the register-resident one-sided form
                                         (Cholesky factor, one patch per 8 to 32 lanes) where only the refined
-                                        eigenpairs are used (BF16-mixed forward, the plain form's rotation), two
+                                        eigenpairs are used (BF16-mixed forward with m >= 128, plain rotation), two
                                         warps per patch in the fused form elsewhere; 1, 4: that many warps per
                                         patch in the fused form (a round's rotations applied in one pass over 2 x 2 blocks of A
                                         and U, two barriers per round, none with 1 warp); 0: one CTA of 128
                                         threads per patch in three passes (row, column and eigenvector
                                         updates, three barriers per round).  The fused and the CTA form apply the
                                         same rotations and thresholds; all forms agree to rounding.  Measured per
-                                        100k patches (k = 64): 230 ms (0), 221 (1), 192 (4); default 78 with the
-                                        refinement, of which 29 the register-resident sweeps */
+                                        100k patches (k = 64), with the refinement: 230 ms (0), 221 (1), 192 (4),
+                                        default 40 */
     MECUCO_OPT_KNN_SPLIT_BF16 = 17   /* BF16-mixed kNN of FP32 rows: 1 (default) the tensor-core search runs on
                                         the three-term split of each row (h = bf16(x), l = bf16(x - h); one GEMM
                                         over [h|h|l] . [h|l|h], three times the K of one rounding) and the

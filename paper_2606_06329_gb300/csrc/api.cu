@@ -320,18 +320,10 @@ mecuco_status run_knn(mecuco_t h, char *ws, const void *X, mecuco_dtype dt, int6
     KnnBufs b;
     knn_scratch(c, p, N, &b);
     if (b.maxima) CK(cudaMemsetAsync(b.maxima, 0, 3 * sizeof(float), s));
-    LAUNCH(h, MECUCO_STAGE_ROWNORM, s, launch_rownorm(X, dt, N, m, ld, b.norms, s, b.resid, b.maxima, p.quant));
-    const void *Xa = X, *Xb = X;
-    if (p.quant == KNN_QUANT_SPLIT) {
-        CK(launch_to_bf16_split(static_cast<const float *>(X), N, m, ld, b.xb, b.xb2, split_segment(m), p.ldb, s));
-        ++h->launches;
-        Xa = b.xb;
-        Xb = b.xb2;
-    } else if (p.bf16_copy) {
-        CK(launch_to_bf16(X, dt, N, m, ld, b.xb, p.ldb, s));
-        ++h->launches;
-        Xa = Xb = b.xb;
-    }
+    LAUNCH(h, MECUCO_STAGE_ROWNORM, s,
+           launch_row_prep(X, dt, N, m, ld, b.norms, s, b.resid, b.maxima, p.quant, b.xb, b.xb2, split_segment(m),
+                           p.ldb));
+    const void *Xa = b.xb ? b.xb : X, *Xb = b.xb2 ? b.xb2 : Xa;
     for (int64_t q0 = rb; q0 < re; q0 += p.qchunk) {
         int64_t nq = std::min(p.qchunk, re - q0);
         int32_t *io = idx_out + (q0 - rb) * k;
@@ -560,7 +552,7 @@ mecuco_status run_curvature(mecuco_t h, char *ws, const void *X, mecuco_dtype dt
             LAUNCH(h, MECUCO_STAGE_GRAM, s, launch_gram_tc(dt, sg, nullptr, 0, np, haar, h->wait_limit, h->ctr, s));
             LAUNCH(h, MECUCO_STAGE_JACOBI, s,
                    launch_jacobi_seg(sg, nullptr, 0, k, np, fp64, h->jacobi_max_sweeps, h->ctr, s, kJacobiPreLoose,
-                                     h->jacobi_warp, true));
+                                     h->jacobi_warp, m >= JACOBI_REG_MIN_M ? jacobi_reg_all(k, np) : JacobiReg()));
             if (fp64 == 1 || fp64 == 3) ++h->launches;  // the refinement is a second kernel
             LAUNCH(h, MECUCO_STAGE_ROTATE, s,
                    launch_rotate_tc(dt, sg, nullptr, 0, np, b.Y, rot_ld(m), h->wait_limit, h->ctr, s));
@@ -708,7 +700,7 @@ struct BatchChunk {
     int kmax;
     int64_t ldy;   // leading dimension of the rotated patches (BF16 elements)
     uint16_t *Y;
-    int64_t jwarps;  // warps of the register-resident eigensolve
+    JacobiReg reg;  // its points in the register-resident eigensolve (m descends, so they lead)
 };
 
 struct BatchPlan {
@@ -720,7 +712,6 @@ struct BatchPlan {
     std::vector<BatchOut> outs;   // this call's outputs, table order
     int64_t nrows = 0, nitems = 0;
     int kcmax = 0, lmax = 0, kmax = 0;
-    bool any_copy = false;
     float *maxima = nullptr;      // 2 per dataset (FP32 rows), zeroed before the row norms
     size_t bytes = 0;             // workspace bytes
 };
@@ -791,7 +782,6 @@ mecuco_status plan_batch(mecuco_t h, const mecuco_dataset *sets, int nsets, mecu
         p.kcmax = std::max(p.kcmax, e.kcl);
         p.lmax = std::max(p.lmax, e.kcl * e.lists);
         p.kmax = std::max(p.kmax, d.k);
-        p.any_copy = p.any_copy || !direct;
     }
     // the datasets' rounding maxima, contiguous (one memset per call)
     p.maxima = dt == MECUCO_F32 ? c.take<float>((size_t)3 * nsets) : nullptr;
@@ -808,7 +798,7 @@ mecuco_status plan_batch(mecuco_t h, const mecuco_dataset *sets, int nsets, mecu
     // estimator chunks: greedy over the points in table order
     const int64_t pt_cap = h->chunk_points > 0 ? h->chunk_points : ((int64_t)1 << 24);
     size_t est_end = after_idx;
-    BatchChunk cur{0, 0, 0, 0, 0, nullptr, 0};
+    BatchChunk cur{0, 0, 0, 0, 0, nullptr, JacobiReg()};
     auto close = [&]() {
         if (cur.np == 0) return;
         Carver e(base, after_idx);
@@ -827,7 +817,7 @@ mecuco_status plan_batch(mecuco_t h, const mecuco_dataset *sets, int nsets, mecu
             g.U = b.U + f * kk * kk;
         }
         p.chunks.push_back(cur);
-        cur = BatchChunk{0, (int)p.segs.size(), 0, 0, 0, nullptr, 0};
+        cur = BatchChunk{0, (int)p.segs.size(), 0, 0, 0, nullptr, JacobiReg()};
     };
     for (int t = 0; t < nsets; ++t) {
         const mecuco_dataset &d = sets[p.order[t]];
@@ -847,8 +837,15 @@ mecuco_status plan_batch(mecuco_t h, const mecuco_dataset *sets, int nsets, mecu
             g.k = d.k;
             g.first = (int)cur.np;
             g.npts = (int)take;
-            g.jfirst = (int)cur.jwarps;
-            cur.jwarps += jacobi_reg_warps(d.k, take);
+            g.jfirst = (int)cur.reg.warps;
+            if (d.m >= JACOBI_REG_MIN_M) {
+                cur.reg.np += take;
+                cur.reg.warps += jacobi_reg_warps(d.k, take);
+                ++cur.reg.nseg;
+                cur.reg.kmax = std::max(cur.reg.kmax, d.k);
+            } else {
+                cur.reg.kmax_rest = std::max(cur.reg.kmax_rest, d.k);
+            }
             g.rowtab = h->tttab[d.k];
             p.segs.push_back(g);
             p.refs.push_back(SegRef{t, 0, a});
@@ -928,11 +925,7 @@ mecuco_status run_batched_persistent(mecuco_t h, const mecuco_dataset *sets, int
     h->launches += (nsets + BATCH_PATCH_SETS - 1) / BATCH_PATCH_SETS;
     // kNN of every row of every dataset: one launch per stage
     if (p.maxima) CK(cudaMemsetAsync(p.maxima, 0, 3 * sizeof(float) * nsets, s));
-    LAUNCH(h, MECUCO_STAGE_ROWNORM, s, launch_rownorm_batch(kt, nsets, p.nrows, dt, s));
-    if (p.any_copy) {
-        CK(launch_to_bf16_batch(kt, nsets, p.nrows, dt, s));
-        ++h->launches;
-    }
+    LAUNCH(h, MECUCO_STAGE_ROWNORM, s, launch_row_prep_batch(kt, nsets, p.nrows, dt, s));
     LAUNCH(h, MECUCO_STAGE_KNN_SEARCH, s,
            launch_knn_tc_batch(kt, nsets, p.nitems, p.kcmax, tn.knn_pair, h->wait_limit, h->ctr, s));
     LAUNCH(h, MECUCO_STAGE_KNN_RERANK, s, launch_knn_rerank_batch(kt, nsets, p.nrows, p.lmax, dt, h->ctr, s));
@@ -947,8 +940,9 @@ mecuco_status run_batched_persistent(mecuco_t h, const mecuco_dataset *sets, int
         LAUNCH(h, MECUCO_STAGE_GRAM, s, launch_gram_tc(dt, none, tab, ch.nseg, ch.np, haar, h->wait_limit, h->ctr, s));
         LAUNCH(h, MECUCO_STAGE_JACOBI, s,
                launch_jacobi_seg(none, tab, ch.nseg, ch.kmax, ch.np, fp64, h->jacobi_max_sweeps, h->ctr, s,
-                                 kJacobiPreLoose, h->jacobi_warp, true, ch.jwarps));
+                                 kJacobiPreLoose, h->jacobi_warp, ch.reg));
         if (fp64 == 1 || fp64 == 3) ++h->launches;
+        if (fp64 == 1 && h->jacobi_warp == 2 && ch.reg.np > 0 && ch.reg.np < ch.np) ++h->launches;  // both sweep forms
         LAUNCH(h, MECUCO_STAGE_ROTATE, s,
                launch_rotate_tc(dt, none, tab, ch.nseg, ch.np, ch.Y, ch.ldy, h->wait_limit, h->ctr, s));
         LAUNCH(h, MECUCO_STAGE_MOMENTS, s,

@@ -25,6 +25,8 @@
 // eigenpairs - it never traps.  Real = float (plain form) or double.
 #include <math.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -55,11 +57,11 @@ struct alignas(2 * sizeof(Real) + 2 * sizeof(int) > 16 ? 32 : 16) JRot {
 
 template <typename Real>
 __global__ void __launch_bounds__(JT)
-jacobi_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restrict__ tab, int ntab, int max_sweeps,
-              Real eps, DevCounters *ctr) {
+jacobi_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restrict__ tab, int ntab, int blk0,
+              int max_sweeps, Real eps, DevCounters *ctr) {
     extern __shared__ __align__(16) unsigned char jsm[];
     int local;
-    const PatchSeg &seg = find_seg(one, tab, ntab, (int)blockIdx.x, local);
+    const PatchSeg &seg = find_seg(one, tab, ntab, blk0 + (int)blockIdx.x, local);
     const int k = seg.k;
     const float *G = seg.G;
     float *sigma = seg.sig, *U = seg.U;
@@ -225,13 +227,13 @@ __device__ __forceinline__ void jw_sync() {
 
 template <int NW>
 __global__ void __launch_bounds__(NW * 32)
-jacobi_warp_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restrict__ tab, int ntab, int max_sweeps,
-                   float eps, DevCounters *ctr) {
+jacobi_warp_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restrict__ tab, int ntab, int blk0,
+                   int max_sweeps, float eps, DevCounters *ctr) {
     extern __shared__ __align__(16) float jw_sm[];
     __shared__ unsigned ctl_mask;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int local;
-    const PatchSeg &seg = find_seg(one, tab, ntab, (int)blockIdx.x, local);
+    const PatchSeg &seg = find_seg(one, tab, ntab, blk0 + (int)blockIdx.x, local);
     const int k = seg.k;
     const int kp = (k + 1) & ~1;
     const int h = kp / 2;
@@ -389,23 +391,24 @@ jacobi_warp_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restr
 }
 
 namespace {
+// blk0: launch point of the first block (the points before it are solved elsewhere)
 template <int NW>
-cudaError_t launch_jw(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t np, int max_sweeps,
-                      float eps, DevCounters *ctr, cudaStream_t s) {
+cudaError_t launch_jw(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t np, int blk0,
+                      int max_sweeps, float eps, DevCounters *ctr, cudaStream_t s) {
     const size_t smem = jw_smem_bytes(kmax);
     cudaError_t e = cudaFuncSetAttribute(jacobi_warp_kernel<NW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem);
     if (e != cudaSuccess) return e;
-    jacobi_warp_kernel<NW><<<(unsigned)np, NW * 32, smem, s>>>(one, tab, ntab, max_sweeps, eps, ctr);
+    jacobi_warp_kernel<NW><<<(unsigned)np, NW * 32, smem, s>>>(one, tab, ntab, blk0, max_sweeps, eps, ctr);
     return cudaGetLastError();
 }
 
 // warps per patch of the fused form (1, 2 or 4)
-cudaError_t launch_jacobi_warp(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t np,
+cudaError_t launch_jacobi_warp(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t np, int blk0,
                                int max_sweeps, float eps, DevCounters *ctr, cudaStream_t s, int nw) {
-    if (nw == 4) return launch_jw<4>(one, tab, ntab, kmax, np, max_sweeps, eps, ctr, s);
-    if (nw == 2) return launch_jw<2>(one, tab, ntab, kmax, np, max_sweeps, eps, ctr, s);
-    return launch_jw<1>(one, tab, ntab, kmax, np, max_sweeps, eps, ctr, s);
+    if (nw == 4) return launch_jw<4>(one, tab, ntab, kmax, np, blk0, max_sweeps, eps, ctr, s);
+    if (nw == 2) return launch_jw<2>(one, tab, ntab, kmax, np, blk0, max_sweeps, eps, ctr, s);
+    return launch_jw<1>(one, tab, ntab, kmax, np, blk0, max_sweeps, eps, ctr, s);
 }
 }  // namespace
 
@@ -457,11 +460,7 @@ __device__ __forceinline__ int tri(int a, int b, int k) { return a * k - (a * (a
 constexpr int FT_REFINE = 256;
 
 template <int NT>
-__global__ void __launch_bounds__(NT, 512 / NT)
-jacobi_refine_ff_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restrict__ tab, int ntab, int rel) {
-    extern __shared__ __align__(16) unsigned char fsm[];
-    int local;
-    const PatchSeg &seg = find_seg(one, tab, ntab, (int)blockIdx.x, local);
+__device__ __forceinline__ void refine_ff_patch(const PatchSeg &seg, int local, int rel, unsigned char *fsm) {
     const int k = seg.k;
     const float *G = seg.G;
     float *sigma = seg.sig, *U = seg.U;
@@ -589,11 +588,255 @@ jacobi_refine_ff_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__
     }
 }
 
+template <int NT>
+__global__ void __launch_bounds__(NT, 512 / NT)
+jacobi_refine_ff_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restrict__ tab, int ntab, int rel) {
+    extern __shared__ __align__(16) unsigned char fsm[];
+    int local;
+    const PatchSeg &seg = find_seg(one, tab, ntab, (int)blockIdx.x, local);
+    refine_ff_patch<NT>(seg, local, rel, fsm);
+}
+
 size_t refine_ff_smem_bytes(int k) {
     return (size_t)4 * k * (k + 1) * sizeof(float) + (size_t)2 * k * (k + 1) * sizeof(float) + 16 +
            (size_t)k * sizeof(double);
 }
 
+
+// ---------------------------------------------------------------------------
+// The same refinement step through the residual T = A X - X diag(l), l the
+// sweeps' eigenvalues, for callers that use only the refined eigenpairs:
+//   N = X^T T = S + R diag(l) - diag(l)      (R = I - X^T X, S = X^T A X),
+// so N_ij is the numerator of E_ij for i != j, and lam_i = l_i + N_ii / (1 -
+// R_ii).  Only T needs more than FP32: it is small (the sweeps' residual, 1e-6
+// to 1e-4 of lam_1), so N from FP32 products carries 2^-24 of a small matrix,
+// which is a relative error of the correction E, not of the eigenvectors.  R is
+// formed (two-term) only where E uses it alone: the diagonal and pairs inside
+// a cluster.  A product a x is added to a two-term sum in four operations: hi
+// carries an offset of 1.5 2^e that every partial sum stays below a third of
+// (|A X| <= lam_1 by Cauchy, so 2^e >= 4 lam_1; 2^e = 4 for the sums of R), so
+// hi never leaves its binade, d = fma(a, x, hi) - hi is exact and fma(a, x, -d)
+// is what the sum lost, to 2^-24 of one unit in the last place of the offset:
+// about 2^-41 lam_1 over 64 terms.
+// One k^3 two-term product and two FP32 ones, no FP64, against two and a half
+// two-term products at ten operations a term, one FP32 product and k^2 FP64
+// divisions (GB300 has 1/64 of the FP32 rate in FP64).
+// Measured on GB300 per 100k patches: k = 64 9.4 ms (two-term products: 52),
+// k = 37 3.3 (12), k = 32 1.6 (6.7); U^T U - I and the off-diagonals of U^T A U
+// as with the two-term products (5e-7, 1.3e-8 lam_1).  FMA-issue bound.
+// Every thread forms 4 x 4 blocks from 16-byte shared loads, two columns per
+// packed FP32 instruction.
+// ---------------------------------------------------------------------------
+namespace {
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pack2(float lo, float hi) {
+    f2 v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ float2 unpack2(f2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+// (hi, lo) += a x, two independent sums with the offset in hi; minus = (-1, -1)
+__device__ __forceinline__ void off_mac2(f2 &hi, f2 &lo, f2 a, f2 x, f2 minus) {
+    const f2 h = fma2(a, x, hi);
+    lo = add2(lo, fma2(a, x, fma2(h, minus, hi)));
+    hi = h;
+}
+// sum of a_r b_r - base over r < k (|sum| <= 1 or so), rounded once
+__device__ __forceinline__ float off_dot(const float *a, const float *b, int stride, int k, float base) {
+    float hi = 6.f, lo = 0.f;
+    for (int r = 0; r < k; ++r) {
+        const float h = __fmaf_rn(a[r * stride], b[r * stride], hi);
+        lo = __fadd_rn(lo, __fmaf_rn(a[r * stride], b[r * stride], __fsub_rn(hi, h)));
+        hi = h;
+    }
+    return __fadd_rn(__fsub_rn(hi, 6.f + base), lo);
+}
+__host__ __device__ inline int rr_ld(int k) { return (k + 3) / 4 * 4 + 4; }
+__host__ __device__ inline size_t refine_res_smem_bytes(int k) {
+    const int k4 = (k + 3) / 4 * 4;
+    return ((size_t)3 * k4 * rr_ld(k) + 4 * k4) * sizeof(float);
+}
+}  // namespace
+
+template <int NT>
+__device__ __forceinline__ void refine_res_patch(const PatchSeg &seg, int local, float *rsm) {
+    const int k = seg.k;
+    const int k4 = (k + 3) / 4 * 4, ld = rr_ld(k), nt = k4 / 4;
+    float *A = rsm;            // [k4][ld] G, later X^T
+    float *X = A + k4 * ld;    // [k4][ld]
+    float *T = X + k4 * ld;    // [k4][ld] A X - X diag(l), later E
+    float *l0 = T + k4 * ld;   // [k4] the sweeps' eigenvalues
+    float *dl = l0 + k4;       // [k4] lam - l0
+    float *rd = dl + k4;       // [k4] R_ii
+    float *lam = rd + k4;      // [k4]
+    const int tid = threadIdx.x;
+    const int64_t pt = local;
+    const float *g = seg.G + pt * (int64_t)k * k;
+    float *u = seg.U + pt * (int64_t)k * k;
+    float *sg = seg.sig + pt * (int64_t)k;
+    for (int r = tid / 32; r < k4; r += NT / 32)
+        for (int c = tid & 31; c < k4; c += 32) {
+            const bool in = r < k && c < k;
+            A[r * ld + c] = in ? g[r * k + c] : 0.f;
+            X[r * ld + c] = in ? u[r * k + c] : 0.f;
+        }
+    if (tid < k4) l0[tid] = tid < k ? sg[tid] : 0.f;
+    __syncthreads();
+    const f2 minus = pack2(-1.f, -1.f);
+    // T = A X - X diag(l): A's rows stand for its columns (symmetric)
+    const bool mine = tid < nt * nt;  // one 4 x 4 block per thread (nt^2 <= NT)
+    const int i0 = tid / nt * 4, c0 = tid % nt * 4;
+    if (mine) {
+        float l1 = 9.4039548e-38f;
+        for (int j = 0; j < k; ++j) l1 = fmaxf(l1, fabsf(l0[j]));
+        // 1.5 2^e, 4 l1 <= 2^e < 8 l1 (the largest binade at the end of the range)
+        const float off = 1.5f * __uint_as_float(min((__float_as_uint(l1) >> 23) + 3u, 253u) << 23);
+        const f2 off2 = pack2(off, off), noff2 = pack2(-off, -off);
+        f2 hi[4][2], lo[4][2] = {};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) hi[i][0] = hi[i][1] = off2;
+        for (int j = 0; j < k; ++j) {
+            const float4 a = *reinterpret_cast<const float4 *>(A + j * ld + i0);
+            const float4 x = *reinterpret_cast<const float4 *>(X + j * ld + c0);
+            const f2 x0 = pack2(x.x, x.y), x1 = pack2(x.z, x.w);
+            const float av[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const f2 a2 = pack2(av[i], av[i]);
+                off_mac2(hi[i][0], lo[i][0], a2, x0, minus);
+                off_mac2(hi[i][1], lo[i][1], a2, x1, minus);
+            }
+        }
+        const float4 l = *reinterpret_cast<const float4 *>(l0 + c0);
+        const f2 n0 = pack2(-l.x, -l.y), n1 = pack2(-l.z, -l.w);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float4 x = *reinterpret_cast<const float4 *>(X + (i0 + i) * ld + c0);
+            off_mac2(hi[i][0], lo[i][0], n0, pack2(x.x, x.y), minus);
+            off_mac2(hi[i][1], lo[i][1], n1, pack2(x.z, x.w), minus);
+            const float2 p = unpack2(add2(add2(hi[i][0], noff2), lo[i][0])),
+                         q = unpack2(add2(add2(hi[i][1], noff2), lo[i][1]));
+            *reinterpret_cast<float4 *>(T + (i0 + i) * ld + c0) = make_float4(p.x, p.y, q.x, q.y);
+        }
+    }
+    // R_ii
+    if (tid < k4) rd[tid] = -off_dot(X + tid, X + tid, ld, k, 1.f);
+    __syncthreads();
+    // N = X^T T, kept in registers
+    f2 n[4][2] = {};
+    if (mine) {
+        for (int r = 0; r < k; ++r) {
+            const float4 x = *reinterpret_cast<const float4 *>(X + r * ld + i0);
+            const float4 v = *reinterpret_cast<const float4 *>(T + r * ld + c0);
+            const f2 v0 = pack2(v.x, v.y), v1 = pack2(v.z, v.w);
+            const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const f2 x2 = pack2(xv[i], xv[i]);
+                n[i][0] = fma2(x2, v0, n[i][0]);
+                n[i][1] = fma2(x2, v1, n[i][1]);
+            }
+        }
+        if (i0 == c0) {
+            const float d[4] = {unpack2(n[0][0]).x, unpack2(n[1][0]).y, unpack2(n[2][1]).x, unpack2(n[3][1]).y};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                dl[i0 + i] = d[i] / (1.f - rd[i0 + i]);
+                lam[i0 + i] = l0[i0 + i] + dl[i0 + i];
+            }
+        }
+    }
+    // X^T over A
+    for (int r = tid / 32; r < k4; r += NT / 32)
+        for (int c = tid & 31; c < k4; c += 32) A[c * ld + r] = X[r * ld + c];
+    __syncthreads();
+    float lmax = 0.f;
+    for (int i = 0; i < k; ++i) lmax = fmaxf(lmax, fabsf(lam[i]));
+    const float delta = 3.814697265625e-06f * lmax;  // 2^-18 max|lam|
+    // E over T (every thread is past its reads of T)
+    if (mine) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 p = unpack2(n[i][0]), q = unpack2(n[i][1]);
+            float v[4] = {p.x, p.y, q.x, q.y};
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+                const int ii = i0 + i, jj = c0 + c;
+                const float d = (l0[jj] - l0[ii]) + (dl[jj] - dl[ii]);
+                if (ii == jj) {
+                    v[c] = 0.5f * rd[ii];
+                } else if (!(fabsf(d) > delta)) {
+                    v[c] = ii < k && jj < k ? -0.5f * off_dot(X + ii, X + jj, ld, k, 0.f) : 0.f;
+                } else {
+                    v[c] = v[c] / d;
+                }
+            }
+            *reinterpret_cast<float4 *>(T + (i0 + i) * ld + c0) = make_float4(v[0], v[1], v[2], v[3]);
+        }
+    }
+    __syncthreads();
+    // X' = X + X E
+    if (mine) {
+        f2 acc[4][2] = {};
+        for (int j = 0; j < k; ++j) {
+            const float4 x = *reinterpret_cast<const float4 *>(A + j * ld + i0);
+            const float4 e = *reinterpret_cast<const float4 *>(T + j * ld + c0);
+            const f2 e0 = pack2(e.x, e.y), e1 = pack2(e.z, e.w);
+            const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const f2 x2 = pack2(xv[i], xv[i]);
+                acc[i][0] = fma2(x2, e0, acc[i][0]);
+                acc[i][1] = fma2(x2, e1, acc[i][1]);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            float4 *xr = reinterpret_cast<float4 *>(X + (i0 + i) * ld + c0);
+            const float4 x = *xr;
+            const float2 p = unpack2(add2(acc[i][0], pack2(x.x, x.y))), q = unpack2(add2(acc[i][1], pack2(x.z, x.w)));
+            *xr = make_float4(p.x, p.y, q.x, q.y);
+        }
+    }
+    // ranks (descending, lowest index first on ties), over dl
+    int *rk = reinterpret_cast<int *>(dl);
+    if (tid < k) {
+        const float li = lam[tid];
+        int rank = 0;
+        for (int j = 0; j < k; ++j) rank += (lam[j] > li) || (lam[j] == li && j < tid);
+        sg[rank] = li;
+        rk[tid] = rank;
+    }
+    __syncthreads();
+    for (int r = tid / 32; r < k; r += NT / 32)
+        for (int c = tid & 31; c < k; c += 32) u[r * k + rk[c]] = X[r * ld + c];
+}
+
+// nres: segments (of a table; they lead) refined through the residual, the rest
+// by the two-term products
+template <int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB)
+jacobi_refine_res_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restrict__ tab, int ntab, int nres) {
+    extern __shared__ __align__(16) float rsm[];
+    int local;
+    const PatchSeg &seg = find_seg(one, tab, ntab, (int)blockIdx.x, local);
+    if (ntab == 0 || (int)(&seg - tab) < nres) refine_res_patch<NT>(seg, local, rsm);
+    else refine_ff_patch<NT>(seg, local, 0, reinterpret_cast<unsigned char *>(rsm));
+}
 
 size_t jacobi_smem_bytes(int k, int fp64) {
     const int kp = (k + 1) & ~1;
@@ -604,36 +847,52 @@ size_t jacobi_smem_bytes(int k, int fp64) {
 
 cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t np, int fp64,
                               int max_sweeps, DevCounters *ctr, cudaStream_t s, float pre_eps, int warp_form,
-                              bool refined_only, int64_t reg_warps) {
+                              const JacobiReg &reg) {
     if (np <= 0) return cudaSuccess;
     if (kmax > 64 || kmax < 1) return cudaErrorInvalidValue;
     cudaError_t e;
-    // FP32 sweeps: one warp per patch, or one CTA per patch
-    auto sweeps32 = [&](float eps) -> cudaError_t {
-        if (warp_form) return launch_jacobi_warp(one, tab, ntab, kmax, np, max_sweeps, eps, ctr, s, warp_form);
-        const size_t smem = jacobi_smem_bytes(kmax, 0);
+    // FP32 sweeps: one or more warps per patch, or one CTA per patch
+    auto sweeps32 = [&](const PatchSeg *t, int nt, int kb, int64_t n, int64_t blk0, float eps) -> cudaError_t {
+        if (n <= 0) return cudaSuccess;
+        if (warp_form) return launch_jacobi_warp(one, t, nt, kb, n, (int)blk0, max_sweeps, eps, ctr, s, warp_form);
+        const size_t smem = jacobi_smem_bytes(kb, 0);
         cudaError_t r = cudaFuncSetAttribute(jacobi_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
         if (r != cudaSuccess) return r;
-        jacobi_kernel<float><<<(unsigned)np, JT, smem, s>>>(one, tab, ntab, max_sweeps, eps, ctr);
+        jacobi_kernel<float><<<(unsigned)n, JT, smem, s>>>(one, t, nt, (int)blk0, max_sweeps, eps, ctr);
         return cudaGetLastError();
     };
     if (fp64 == 1 || fp64 == 3) {
         // FP32 sweeps, then one refinement step (3: relative cluster test)
-        if (refined_only && fp64 == 1 && warp_form == 2) {
+        const bool fast = reg.np > 0 && fp64 == 1 && warp_form == 2;
+        if (fast) {
             // |cos| of the last sweep: the step after it squares what is left
             const float stop = pre_eps >= kJacobiPreLoose ? 9.765625e-04f : 1.220703125e-04f;  // 2^-10, 2^-13
             PatchSeg seg = one;
-            if (ntab == 0) {
-                seg.npts = (int)np;
-                seg.jfirst = 0;
-                reg_warps = jacobi_reg_warps(one.k, np);
-            }
-            e = launch_jacobi_reg(seg, tab, ntab, kmax, reg_warps, max_sweeps, stop, ctr, s);
+            seg.npts = (int)np;
+            seg.jfirst = 0;
+            e = launch_jacobi_reg(seg, tab, ntab ? reg.nseg : 0, reg.kmax, reg.warps, max_sweeps, stop, ctr, s);
+            if (e != cudaSuccess) return e;
+            e = sweeps32(tab + reg.nseg, ntab - reg.nseg, reg.kmax_rest, np - reg.np, reg.np, pre_eps);
         } else {
-            e = sweeps32(pre_eps);
+            e = sweeps32(tab, ntab, kmax, np, 0, pre_eps);
         }
         if (e != cudaSuccess) return e;
+        if (fast) {
+            // threads per patch: one 4 x 4 block each; one launch, which takes the
+            // two-term products for the points solved by the two-sided sweeps
+            const bool rest = reg.np < np;
+            const size_t rs = std::max(refine_res_smem_bytes(reg.kmax), rest ? refine_ff_smem_bytes(reg.kmax_rest) : 0);
+            auto refine = [&](auto kern, int nt) -> cudaError_t {
+                cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
+                if (r != cudaSuccess) return r;
+                kern<<<(unsigned)np, nt, rs, s>>>(one, tab, ntab, reg.nseg);
+                return cudaGetLastError();
+            };
+            if (kmax <= 32) return refine(jacobi_refine_res_kernel<64, 12>, 64);
+            if (kmax <= 44) return refine(jacobi_refine_res_kernel<128, 6>, 128);
+            return refine(jacobi_refine_res_kernel<256, 3>, 256);
+        }
         // threads per patch: 64 (k <= 16), 128 (k <= 32) or 256, so that small
         // patches are not limited to 8 per SM by idle threads
         const size_t rs = refine_ff_smem_bytes(kmax);
@@ -651,20 +910,21 @@ cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab
         const size_t smem = jacobi_smem_bytes(kmax, fp64);
         e = cudaFuncSetAttribute(jacobi_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        jacobi_kernel<double><<<(unsigned)np, JT, smem, s>>>(one, tab, ntab, max_sweeps, JacobiEps<double>::rel(), ctr);
+        jacobi_kernel<double><<<(unsigned)np, JT, smem, s>>>(one, tab, ntab, 0, max_sweeps, JacobiEps<double>::rel(), ctr);
         return cudaGetLastError();
     }
-    return sweeps32(JacobiEps<float>::rel());
+    return sweeps32(tab, ntab, kmax, np, 0, JacobiEps<float>::rel());
 }
 
 cudaError_t launch_jacobi(const float *G, int k, int64_t np, int fp64, int max_sweeps, float *sigma, float *U,
-                          DevCounters *ctr, cudaStream_t s, float pre_eps, int warp_form, bool refined_only) {
+                          DevCounters *ctr, cudaStream_t s, float pre_eps, int warp_form, bool reg) {
     PatchSeg one{};
     one.k = k;
     one.G = const_cast<float *>(G);
     one.sig = sigma;
     one.U = U;
-    return launch_jacobi_seg(one, nullptr, 0, k, np, fp64, max_sweeps, ctr, s, pre_eps, warp_form, refined_only);
+    return launch_jacobi_seg(one, nullptr, 0, k, np, fp64, max_sweeps, ctr, s, pre_eps, warp_form,
+                             reg ? jacobi_reg_all(k, np) : JacobiReg());
 }
 
 }  // namespace mecuco

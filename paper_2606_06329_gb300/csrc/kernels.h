@@ -20,16 +20,21 @@ void set_error_text(const char *msg);
 // ---- Step 1: kNN -----------------------------------------------------------
 // How the tensor-core search sees FP32 rows (KNN_QUANT_*): not at all (BF16
 // rows, or the CUDA-core search), as one BF16 rounding h = bf16(x), or as the
-// three-term split (h, l = bf16(x - h)) of launch_to_bf16_split.
+// three-term split (h, l = bf16(x - h)) of launch_row_prep.
 enum { KNN_QUANT_NONE = 0, KNN_QUANT_SINGLE = 1, KNN_QUANT_SPLIT = 2 };
-// Squared row norms |x_i|^2 (compensated sum, rounded once), i in [0, N).
+// Squared row norms |x_i|^2 (compensated sum, rounded once), i in [0, N), and in
+// the same pass the search's BF16 operand rows (leading dimension ldb): ya =
+// bf16(x), or with yb the three-term split in segments of ms >= m columns (ms %
+// 8 == 0), query copy ya = [h | h | l], candidate copy yb = [h | l | h]; zero
+// past the data; NULL: none.
 // With quant != KNN_QUANT_NONE (FP32 rows only), resid[2 i .. 2 i + 1] gets the
 // row's rounding terms, rounded up: single rounding |x - h| and 0; split
 // |l| and |x - h - l|; maxima[0..2] (zeroed by the caller) receives the
 // dataset's largest |x|^2 and the largest of each term.
-cudaError_t launch_rownorm(const void *X, mecuco_dtype dt, int64_t N, int64_t m, int64_t ld,
-                           float *norms, cudaStream_t s, float *resid = nullptr, float *maxima = nullptr,
-                           int quant = KNN_QUANT_NONE);
+cudaError_t launch_row_prep(const void *X, mecuco_dtype dt, int64_t N, int64_t m, int64_t ld, float *norms,
+                            cudaStream_t s, float *resid = nullptr, float *maxima = nullptr,
+                            int quant = KNN_QUANT_NONE, void *ya = nullptr, void *yb = nullptr, int64_t ms = 0,
+                            int64_t ldb = 0);
 
 // Candidate search, plain FP32 on the CUDA cores.  Queries [q0, q0 + nq) against
 // all N rows, candidate range split in `nsplit` parts; per (query, split) the
@@ -44,7 +49,7 @@ cudaError_t launch_knn_simt(const void *X, mecuco_dtype dt, int64_t N, int64_t m
 // knn_tc_halves() lists of capacity kc per row and split.  Xa (query operand)
 // and Xb (candidate operand) are BF16 row-major with K = m columns, ldb % 8 ==
 // 0 and 16-byte aligned bases: both X itself when it is stored that way, both
-// the copy of launch_to_bf16, or the two copies of launch_to_bf16_split (then
+// the copy of launch_row_prep, or its two copies of the split (then
 // m is their K = 3 ms).  kc <= 64.
 // pair != 0 (and nq >= 256): CTA pairs sharing 256 x 256 cta_group::2 MMAs;
 // the lists are the same.  wait_limit: clock cycles after which a wait of the
@@ -74,7 +79,7 @@ struct KnnSet {  // aligned as CUtensorMap (the device table needs 64-byte align
     int32_t *cand_i;
     int32_t *flags;    // N
     int32_t *idx;      // N x k, the neighbour lists
-    float *resid;      // 2 N: the rows' rounding terms (launch_rownorm), or NULL
+    float *resid;      // 2 N: the rows' rounding terms (launch_row_prep), or NULL
     float *maxima;     // 3: their maxima and the largest |x|^2 (with resid)
     int k, kc, kcl, nsplit, lists, include_self;
     int quant;         // KNN_QUANT_*
@@ -107,30 +112,20 @@ struct SegRef {
 constexpr int BATCH_PATCH_SETS = 1024;
 cudaError_t launch_batch_patch(KnnSet *sets, int nsets, PatchSeg *segs, const SegRef *refs, int nsegs,
                                const BatchOut *outs, cudaStream_t s);
-// Row norms, BF16 copies, exact re-rank and fallback over every row of a
+// Row norms and BF16 copies, exact re-rank and fallback over every row of a
 // batch (table rows sorted by row_begin, nrows rows in all); the re-rank's
 // shared memory is sized for lmax = the largest kcl * lists.
-cudaError_t launch_rownorm_batch(const KnnSet *sets, int nsets, int64_t nrows, mecuco_dtype dt, cudaStream_t s);
-cudaError_t launch_to_bf16_batch(const KnnSet *sets, int nsets, int64_t nrows, mecuco_dtype dt, cudaStream_t s);
+cudaError_t launch_row_prep_batch(const KnnSet *sets, int nsets, int64_t nrows, mecuco_dtype dt, cudaStream_t s);
 cudaError_t launch_knn_rerank_batch(const KnnSet *sets, int nsets, int64_t nrows, int lmax, mecuco_dtype dt,
                                     DevCounters *ctr, cudaStream_t s);
 cudaError_t launch_knn_fallback_batch(const KnnSet *sets, int nsets, int64_t nrows, int kmax, mecuco_dtype dt,
                                       DevCounters *ctr, cudaStream_t s);
 
-// The three-term split of FP32 rows: query copy Ya = [h | h | l], candidate
-// copy Yb = [h | l | h] in segments of ms >= m columns (ms % 8 == 0, zero past
-// m), leading dimension ldb >= 3 ms.
-cudaError_t launch_to_bf16_split(const float *X, int64_t N, int64_t m, int64_t ld, void *Ya, void *Yb, int64_t ms,
-                                 int64_t ldb, cudaStream_t s);
-// BF16 copy of X (round to nearest even) with leading dimension ldb >= m.
-cudaError_t launch_to_bf16(const void *X, mecuco_dtype dt, int64_t N, int64_t m, int64_t ld, void *Y,
-                           int64_t ldb, cudaStream_t s);
-
 // Exact re-rank of the L = kc * nsplit candidates of each query by a
 // compensated (float-float) sum of (x_a - y_a)^2, top-k by (distance, index),
 // and the certification test; uncertified rows get flags[q - q0] = 1.
 // idx_out / dist_out point at query q0's row (row q - q0 is written).
-// resid / maxima (from launch_rownorm): the search ran on BF16 roundings of
+// resid / maxima (from launch_row_prep): the search ran on BF16 roundings of
 // FP32 rows; the certification then also covers the rounding's a-priori
 // bound on every candidate's distance error.
 cudaError_t launch_knn_rerank(const void *X, mecuco_dtype dt, int64_t N, int64_t m, int64_t ld,
@@ -223,27 +218,47 @@ cudaError_t launch_tthird_tc(const PatchSeg &one, const PatchSeg *tab, int ntab,
 // rotated Gram must come out nearly diagonal, take kJacobiPreTight.
 constexpr float kJacobiPreTight = 2.384185791015625e-07f;  // 2^-22
 constexpr float kJacobiPreLoose = 6.103515625e-05f;        // 2^-14
-// refined_only: the caller needs the eigenpairs after the refinement step
-// (fp64 = 1) only to its accuracy, so the FP32 sweeps may be the
-// register-resident one-sided form (jacobi_reg.cu), taken with warp_form = 2
-// (the default): 4 to 9 times faster than the fused two-sided form at every k
-// measured (jacobi_reg.cu).  Callers whose results follow the eigenvectors of
-// near-degenerate pairs (Exact mode, the adjoint) keep the two-sided sweeps.
+// reg: the leading points solved, with fp64 = 1 and warp_form = 2 (the default),
+// by the register-resident one-sided sweeps (jacobi_reg.cu; 4 to 9 times faster
+// than the fused two-sided form at every k measured) and the refinement through
+// the residual (5 times faster at k = 64).  Callers whose results follow the
+// eigenvectors of near-degenerate pairs (Exact mode, the adjoint) keep the
+// two-sided sweeps and the two-term products.
+struct JacobiReg {
+    int64_t np = 0;             // leading points of the launch in the register form
+    int64_t warps = 0;          // their warps (a table's segments: the sum of jacobi_reg_warps)
+    int nseg = 0;               // their segments (tables)
+    int kmax = 0, kmax_rest = 0;  // bounds of k on either side
+};
+// The BF16-mixed form takes it for m >= JACOBI_REG_MIN_M.  Below, the null-space
+// term divides by a small m - p and the BF16 rounding of the rotated patch turns
+// the last bits of the eigenvectors into 1e-5 of kappa and more: the curvatures
+// of the two solvers, both as accurate against FP64, differ by up to 2.5e-5 at
+// m = 64, k = 52, against 5e-6 at m = 128 and 3e-6 from m = 192 up, and such
+// narrow sets keep the values they had.
+constexpr int64_t JACOBI_REG_MIN_M = 128;
 // warp_form != 0: the FP32 sweeps run one warp per patch (fused 2 x 2 block
 // updates, no block barriers); 0: one CTA of 128 threads per patch.  FP64
 // sweeps (fp64 = 2) always take the CTA form.
 cudaError_t launch_jacobi(const float *G, int k, int64_t np, int fp64, int max_sweeps,
                           float *sigma, float *U, DevCounters *ctr, cudaStream_t s,
-                          float pre_eps = kJacobiPreTight, int warp_form = 1, bool refined_only = false);
+                          float pre_eps = kJacobiPreTight, int warp_form = 1, bool reg = false);
 // The same over a segment table (PatchSeg: G, k, sig, U of each segment);
 // kmax bounds every segment's k.
 cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t np, int fp64,
                               int max_sweeps, DevCounters *ctr, cudaStream_t s, float pre_eps, int warp_form = 1,
-                              bool refined_only = false, int64_t reg_warps = 0);
+                              const JacobiReg &reg = JacobiReg());
 // Register-resident one-sided sweeps: nwarps warps in all, each on
 // jacobi_reg_warps()'s share of one segment's patches (PatchSeg: k, npts,
 // jfirst, G, sig, U); stop_cos bounds |cos| between columns in the last sweep.
 int64_t jacobi_reg_warps(int k, int64_t np);
+inline JacobiReg jacobi_reg_all(int k, int64_t np) {  // every point of a single segment
+    JacobiReg r;
+    r.np = np;
+    r.warps = jacobi_reg_warps(k, np);
+    r.kmax = k;
+    return r;
+}
 cudaError_t launch_jacobi_reg(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t nwarps,
                               int max_sweeps, float stop_cos, DevCounters *ctr, cudaStream_t s);
 

@@ -26,32 +26,57 @@ __device__ __forceinline__ const KnnSet &find_set_row(const KnnSet *sets, int ns
     return sets[lo];
 }
 
-// One warp: |x|^2 of a row as a compensated sum (hi + lo rounded once, so
-// within a few FP32 units of the exact value) and, for quant != NONE, the
-// norms of the row's BF16 rounding terms (rounded up) into resid[0..1]:
-// single rounding h = bf16(x): |x - h| and 0; three-term split, l = bf16(x - h):
-// |l| and |x - h - l| (both differences exact in FP32).  The dataset's largest
-// |x|^2 and terms go to maxima[0..2] (non-negative floats, so their bit
-// patterns order as integers).
+// One warp, one read of a row: |x|^2 as a compensated sum (hi + lo rounded once,
+// so within a few FP32 units of the exact value), the BF16 operand rows of the
+// tensor-core search (ya, and yb for the three-term split; NULL: none), and, for
+// quant != NONE, the norms of the row's BF16 rounding terms (rounded up) into
+// resid[0..1]: single rounding h = bf16(x): |x - h| and 0; three-term split,
+// l = bf16(x - h): |l| and |x - h - l| (both differences exact in FP32).  The
+// dataset's largest |x|^2 and terms go to maxima[0..2] (non-negative floats, so
+// their bit patterns order as integers).
+// Operand rows (leading dimension ldb, zero past the data): one rounding, y = h;
+// the three-term split, in segments of ms columns, query copy [h | h | l] and
+// candidate copy [h | l | h], so that one GEMM over K = 3 ms gives h.h' + h.l' +
+// l.h', the FP32 product up to l.l' and the remainders past two terms.
 template <typename T>
-__device__ __forceinline__ void row_norm_warp(const T *__restrict__ x, int64_t m, int lane, float *norm_out,
-                                              float *resid_out, float *maxima, int quant) {
+__device__ __forceinline__ void row_prep_warp(const T *__restrict__ x, int64_t m, int lane, float *norm_out,
+                                              float *resid_out, float *maxima, int quant,
+                                              __nv_bfloat16 *__restrict__ ya, __nv_bfloat16 *__restrict__ yb,
+                                              int64_t ms, int64_t ldb) {
     ff acc{0.f, 0.f};
     float a1 = 0.f, a2 = 0.f;
     for (int64_t a = lane; a < m; a += 32) {
         const float v = load_elem(x + a);
         ff_acc_sqdiff(acc, v, 0.f);
-        if (quant != KNN_QUANT_NONE) {
-            const float r = v - __bfloat162float(__float2bfloat16_rn(v));
-            if (quant == KNN_QUANT_SINGLE) {
-                a1 = fmaf(r, r, a1);
-            } else {
-                const float l = __bfloat162float(__float2bfloat16_rn(r));
-                const float r2 = r - l;
-                a1 = fmaf(l, l, a1);
-                a2 = fmaf(r2, r2, a2);
-            }
+        const __nv_bfloat16 h = __float2bfloat16_rn(v);
+        const float r = v - __bfloat162float(h);
+        const __nv_bfloat16 lb = __float2bfloat16_rn(r);
+        if (quant == KNN_QUANT_SINGLE) {
+            a1 = fmaf(r, r, a1);
+        } else if (quant == KNN_QUANT_SPLIT) {
+            const float l = __bfloat162float(lb);
+            const float r2 = r - l;
+            a1 = fmaf(l, l, a1);
+            a2 = fmaf(r2, r2, a2);
         }
+        if (yb) {
+            ya[a] = h;
+            ya[ms + a] = h;
+            ya[2 * ms + a] = lb;
+            yb[a] = h;
+            yb[ms + a] = lb;
+            yb[2 * ms + a] = h;
+        } else if (ya) {
+            ya[a] = h;
+        }
+    }
+    const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
+    if (yb) {
+        for (int64_t a = m + lane; a < ms; a += 32)
+            ya[a] = ya[ms + a] = ya[2 * ms + a] = yb[a] = yb[ms + a] = yb[2 * ms + a] = zero;
+        for (int64_t a = 3 * ms + lane; a < ldb; a += 32) ya[a] = yb[a] = zero;
+    } else if (ya) {
+        for (int64_t a = m + lane; a < ldb; a += 32) ya[a] = zero;
     }
     acc = ff_warp_sum(acc);
     const float n = acc.hi + acc.lo;
@@ -74,81 +99,52 @@ __device__ __forceinline__ void row_norm_warp(const T *__restrict__ x, int64_t m
 }
 
 template <typename T>
-__global__ void rownorm_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld, float *__restrict__ out,
-                               float *__restrict__ resid, float *__restrict__ maxima, int quant) {
+__global__ void row_prep_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld, float *__restrict__ out,
+                                float *__restrict__ resid, float *__restrict__ maxima, int quant,
+                                __nv_bfloat16 *__restrict__ ya, __nv_bfloat16 *__restrict__ yb, int64_t ms,
+                                int64_t ldb) {
     int64_t row = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     int lane = threadIdx.x & 31;
     if (row >= N) return;
-    row_norm_warp(X + row * ld, m, lane, out + row, quant ? resid + 2 * row : nullptr, maxima, quant);
+    row_prep_warp(X + row * ld, m, lane, out + row, quant ? resid + 2 * row : nullptr, maxima, quant,
+                  ya ? ya + row * ldb : nullptr, yb ? yb + row * ldb : nullptr, ms, ldb);
 }
 
-cudaError_t launch_rownorm(const void *X, mecuco_dtype dt, int64_t N, int64_t m, int64_t ld,
-                           float *norms, cudaStream_t s, float *resid, float *maxima, int quant) {
+cudaError_t launch_row_prep(const void *X, mecuco_dtype dt, int64_t N, int64_t m, int64_t ld, float *norms,
+                            cudaStream_t s, float *resid, float *maxima, int quant, void *ya, void *yb, int64_t ms,
+                            int64_t ldb) {
     if (N <= 0) return cudaSuccess;
     if (dt == MECUCO_BF16 || !resid || !maxima) quant = KNN_QUANT_NONE;
     dim3 block(256), grid((unsigned)((N + 7) / 8));
+    __nv_bfloat16 *a = (__nv_bfloat16 *)ya, *b = (__nv_bfloat16 *)yb;
     if (dt == MECUCO_BF16)
-        rownorm_kernel<<<grid, block, 0, s>>>((const __nv_bfloat16 *)X, N, m, ld, norms, nullptr, nullptr, quant);
+        row_prep_kernel<<<grid, block, 0, s>>>((const __nv_bfloat16 *)X, N, m, ld, norms, nullptr, nullptr, quant, a,
+                                               b, ms, ldb);
     else
-        rownorm_kernel<<<grid, block, 0, s>>>((const float *)X, N, m, ld, norms, resid, maxima, quant);
+        row_prep_kernel<<<grid, block, 0, s>>>((const float *)X, N, m, ld, norms, resid, maxima, quant, a, b, ms, ldb);
     return cudaGetLastError();
 }
 
-// Row norms of every row of a batch: one warp per row, each row's dataset from
-// the table.
+// The same for every row of a batch: one warp per row, each row's dataset from
+// the table (xb, xb2 its operand rows where it has them).
 template <typename T>
-__global__ void rownorm_batch_kernel(const KnnSet *__restrict__ sets, int nsets, int64_t nrows) {
+__global__ void row_prep_batch_kernel(const KnnSet *__restrict__ sets, int nsets, int64_t nrows) {
     const int64_t gr = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
     const int lane = threadIdx.x & 31;
     if (gr >= nrows) return;
     const KnnSet &d = find_set_row(sets, nsets, gr);
     const int64_t row = gr - d.row_begin;
-    row_norm_warp(static_cast<const T *>(d.X) + row * d.ld, d.m, lane, d.norms + row,
-                  d.quant ? d.resid + 2 * row : nullptr, d.maxima, d.quant);
+    __nv_bfloat16 *ya = static_cast<__nv_bfloat16 *>(d.xb), *yb = static_cast<__nv_bfloat16 *>(d.xb2);
+    row_prep_warp(static_cast<const T *>(d.X) + row * d.ld, d.m, lane, d.norms + row,
+                  d.quant ? d.resid + 2 * row : nullptr, d.maxima, d.quant, ya ? ya + row * d.ldb : nullptr,
+                  yb ? yb + row * d.ldb : nullptr, d.mk / 3, d.ldb);
 }
 
-cudaError_t launch_rownorm_batch(const KnnSet *sets, int nsets, int64_t nrows, mecuco_dtype dt, cudaStream_t s) {
+cudaError_t launch_row_prep_batch(const KnnSet *sets, int nsets, int64_t nrows, mecuco_dtype dt, cudaStream_t s) {
     if (nrows <= 0) return cudaSuccess;
     dim3 block(256), grid((unsigned)((nrows + 7) / 8));
-    if (dt == MECUCO_BF16) rownorm_batch_kernel<__nv_bfloat16><<<grid, block, 0, s>>>(sets, nsets, nrows);
-    else rownorm_batch_kernel<float><<<grid, block, 0, s>>>(sets, nsets, nrows);
-    return cudaGetLastError();
-}
-
-// BF16 copies (round to nearest even, zero past m) of the rows of every
-// dataset that has one (xb): one warp per row, coalesced along the row.
-template <typename T>
-__global__ void to_bf16_batch_kernel(const KnnSet *__restrict__ sets, int nsets, int64_t nrows) {
-    const int64_t gr = (int64_t)blockIdx.x * (blockDim.x / 32) + threadIdx.x / 32;
-    const int lane = threadIdx.x & 31;
-    if (gr >= nrows) return;
-    const KnnSet &d = find_set_row(sets, nsets, gr);
-    if (!d.xb) return;
-    const int64_t row = gr - d.row_begin;
-    const T *x = static_cast<const T *>(d.X) + row * d.ld;
-    __nv_bfloat16 *y = static_cast<__nv_bfloat16 *>(d.xb) + row * d.ldb;
-    if (!d.xb2) {
-        for (int64_t a = lane; a < d.ldb; a += 32) y[a] = __float2bfloat16_rn(a < d.m ? load_elem(x + a) : 0.f);
-        return;
-    }
-    // three-term split (as launch_to_bf16_split): query [h | h | l], candidate [h | l | h]
-    __nv_bfloat16 *yb = static_cast<__nv_bfloat16 *>(d.xb2) + row * d.ldb;
-    const int64_t ms = d.mk / 3;
-    for (int64_t a = lane; a < d.ldb; a += 32) {
-        const int64_t seg = a / ms, c = a - seg * ms;
-        const float v = (seg < 3 && c < d.m) ? load_elem(x + c) : 0.f;
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
-        y[a] = seg == 2 ? l : h;
-        yb[a] = seg == 1 ? l : h;
-    }
-}
-
-cudaError_t launch_to_bf16_batch(const KnnSet *sets, int nsets, int64_t nrows, mecuco_dtype dt, cudaStream_t s) {
-    if (nrows <= 0) return cudaSuccess;
-    dim3 block(256), grid((unsigned)((nrows + 7) / 8));
-    if (dt == MECUCO_BF16) to_bf16_batch_kernel<__nv_bfloat16><<<grid, block, 0, s>>>(sets, nsets, nrows);
-    else to_bf16_batch_kernel<float><<<grid, block, 0, s>>>(sets, nsets, nrows);
+    if (dt == MECUCO_BF16) row_prep_batch_kernel<__nv_bfloat16><<<grid, block, 0, s>>>(sets, nsets, nrows);
+    else row_prep_batch_kernel<float><<<grid, block, 0, s>>>(sets, nsets, nrows);
     return cudaGetLastError();
 }
 

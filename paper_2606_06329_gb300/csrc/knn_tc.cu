@@ -701,50 +701,4 @@ cudaError_t launch_knn_tc_batch(const KnnSet *sets, int nsets, int64_t nitems, i
     return cudaGetLastError();
 }
 
-// FP32 -> BF16 copy (round to nearest even) with a padded leading dimension.
-__global__ void to_bf16_kernel(const float *__restrict__ X, int64_t N, int64_t m, int64_t ld,
-                               __nv_bfloat16 *__restrict__ Y, int64_t ldb) {
-    const int64_t row = blockIdx.x;
-    for (int64_t a = threadIdx.x; a < ldb; a += blockDim.x)
-        Y[row * ldb + a] = __float2bfloat16_rn(a < m ? X[row * ld + a] : 0.f);
-}
-
-// The three-term split of FP32 rows for the search: with h = bf16(x) and
-// l = bf16(x - h), the query copy holds [h | h | l] and the candidate copy
-// [h | l | h] along K (segments of ms columns, zero past m), so that one GEMM
-// over K = 3 ms gives h.h' + h.l' + l.h', the FP32 product up to l.l' and the
-// remainders past two terms.
-__global__ void to_bf16_split_kernel(const float *__restrict__ X, int64_t m, int64_t ld, __nv_bfloat16 *__restrict__ Ya,
-                                     __nv_bfloat16 *__restrict__ Yb, int64_t ms, int64_t ldb) {
-    const int64_t row = blockIdx.x;
-    const float *x = X + row * ld;
-    __nv_bfloat16 *ya = Ya + row * ldb, *yb = Yb + row * ldb;
-    for (int64_t a = threadIdx.x; a < ldb; a += blockDim.x) {
-        const int64_t seg = a / ms, c = a - seg * ms;
-        const float v = (seg < 3 && c < m) ? x[c] : 0.f;
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        const __nv_bfloat16 l = __float2bfloat16_rn(v - __bfloat162float(h));
-        ya[a] = seg == 2 ? l : h;
-        yb[a] = seg == 1 ? l : h;
-    }
-}
-
-cudaError_t launch_to_bf16_split(const float *X, int64_t N, int64_t m, int64_t ld, void *Ya, void *Yb, int64_t ms,
-                                 int64_t ldb, cudaStream_t s) {
-    if (N <= 0) return cudaSuccess;
-    to_bf16_split_kernel<<<(unsigned)N, 256, 0, s>>>(X, m, ld, (__nv_bfloat16 *)Ya, (__nv_bfloat16 *)Yb, ms, ldb);
-    return cudaGetLastError();
-}
-
-cudaError_t launch_to_bf16(const void *X, mecuco_dtype dt, int64_t N, int64_t m, int64_t ld, void *Y, int64_t ldb,
-                           cudaStream_t s) {
-    if (N <= 0) return cudaSuccess;
-    if (dt == MECUCO_BF16) {
-        return cudaMemcpy2DAsync(Y, (size_t)ldb * 2, X, (size_t)ld * 2, (size_t)m * 2, (size_t)N,
-                                 cudaMemcpyDeviceToDevice, s);
-    }
-    to_bf16_kernel<<<(unsigned)N, 256, 0, s>>>((const float *)X, N, m, ld, (__nv_bfloat16 *)Y, ldb);
-    return cudaGetLastError();
-}
-
 }  // namespace mecuco

@@ -151,7 +151,7 @@ extern "C" MECUCO_API mecuco_status mecuco_knn_noalloc(const void *X, mecuco_dty
     int32_t *cand_i = reinterpret_cast<int32_t *>(p);
 
     if (cudaMemsetAsync(ctr, 0, sizeof(DevCounters), s) != cudaSuccess) return MECUCO_ERR_CUDA;
-    if (launch_rownorm(X, dt, N, m, ld, norms, s) != cudaSuccess) return MECUCO_ERR_CUDA;
+    if (launch_row_prep(X, dt, N, m, ld, norms, s) != cudaSuccess) return MECUCO_ERR_CUDA;
     for (int64_t q0 = 0; q0 < N; q0 += qchunk) {
         const int64_t nq = std::min(qchunk, N - q0);
         int32_t *io = idx_out + q0 * k;
