@@ -65,7 +65,7 @@ struct mecuco_ctx {
     int32_t *rowtab[65] = {};    // per k: row codes of the tensor-core moment kernel
     int32_t *tttab[65] = {};     // per k: row codes of the third-moment pass (pairs only)
     int knn_splits = 0;
-    int knn_pair = -1;  // -1: CTA pairs for N >= KNN_PAIR_MIN_N
+    int knn_pair = -1;  // -1: CTA pairs for operand rows of KNN_PAIR_MIN_K columns or more
     int knn_split_bf16 = 1;  // FP32 rows: three-term BF16 split in the tensor-core search
     int chunk_share = 1;  // concurrent lanes sharing the chunk budget (batched calls)
     int tc_slots = 4;
@@ -226,13 +226,33 @@ int candidate_capacity(mecuco_t h, int k) {
     return (int)kc;
 }
 
-constexpr int64_t KNN_PAIR_MIN_N = 200000;
+// CTA pairs (256 x 256 two-SM MMAs, two thirds of the operand bytes per MMA) from
+// this row length of the BF16 operands on: single / pair search time 1.10 at K =
+// 4096, 1.17 at 2352, 0.97 at 2048, 0.92 at 1024, 0.87 at 512 (100,000 points;
+// 0.92 at 200,000 x 1024, 1.05 at 20,000 x 4096).
+constexpr int64_t KNN_PAIR_MIN_K = 2200;
 
 struct KnnPlan {
-    int kc, nsplit;
-    int lists;      // candidate lists per query row (splits x the tensor-core kernel's column halves)
+    struct Piece {
+        int64_t rows;  // query rows of one search launch
+        int nsplit;    // candidate-range splits; nsplit x halves lists per row
+    };
+    std::vector<Piece> pieces;
+    int kc;
+    int halves;     // lists per row and split (the tensor-core kernel's column halves)
     int kcl;        // capacity of each list
+    int cap;        // largest number of splits (1024 candidates per row)
     int64_t qchunk;
+    int64_t max_rows() const {
+        int64_t r = 0;
+        for (const Piece &q : pieces) r = std::max(r, q.rows);
+        return r;
+    }
+    int64_t max_slots() const {
+        int64_t r = 0;
+        for (const Piece &q : pieces) r = std::max(r, q.rows * q.nsplit * halves * kcl);
+        return r;
+    }
     bool tc;        // candidate search on the tensor cores (BF16 operands)
     bool pair;      // tensor-core search as CTA pairs sharing two-SM MMAs
     bool bf16_copy; // the tensor-core path needs a BF16 copy of X
@@ -249,11 +269,6 @@ KnnPlan plan_knn(mecuco_t h, const void *X, mecuco_dtype dt, int64_t N, int64_t 
     KnnPlan p;
     p.kc = candidate_capacity(h, k);
     p.tc = prec == MECUCO_PREC_BF16_MIXED;
-    // CTA pairs (256 x 256 two-SM MMAs, half the candidate bytes per SM) pay
-    // from a few hundred thousand candidates up: measured at m = 4096, k = 64,
-    // 1M points 7.53 s against 7.93 s per search, 300k 0.683 against 0.716 s,
-    // but 100k 88.5 against 85.4 ms
-    p.pair = p.tc && (h->knn_pair > 0 || (h->knn_pair < 0 && N >= KNN_PAIR_MIN_N));
     const bool direct = dt == MECUCO_BF16 && ld % 8 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
     p.bf16_copy = p.tc && !direct;
     // FP32 rows: the three-term split (a search three times as long in K whose
@@ -263,31 +278,60 @@ KnnPlan plan_knn(mecuco_t h, const void *X, mecuco_dtype dt, int64_t N, int64_t 
     p.quant = !(p.tc && dt == MECUCO_F32) ? KNN_QUANT_NONE : (h->knn_split_bf16 ? KNN_QUANT_SPLIT : KNN_QUANT_SINGLE);
     p.mk = p.quant == KNN_QUANT_SPLIT ? 3 * split_segment(m) : m;
     p.ldb = direct ? ld : (p.mk + 7) / 8 * 8;
+    p.pair = p.tc && (h->knn_pair > 0 || (h->knn_pair < 0 && p.mk >= KNN_PAIR_MIN_K));
     p.qchunk = h->knn_qchunk > 0 ? h->knn_qchunk : (int64_t)1 << 18;
-    if (p.tc && h->knn_qchunk <= 0) {
-        // whole waves of the persistent search per launch: a multiple of the
-        // query rows one wave of CTAs (pairs) covers, so that only the last
-        // launch ends on a partial wave (1M points: 52 instead of 53 waves)
-        const int64_t wave = p.pair ? (int64_t)(h->num_sms / 2) * 256 : (int64_t)h->num_sms * 128;
-        if (p.qchunk > wave) p.qchunk = p.qchunk / wave * wave;
-    }
+    // query rows that one wave of the persistent search covers (tensor-core form)
+    const int64_t wave = p.pair ? (int64_t)(h->num_sms / 2) * 256 : (int64_t)h->num_sms * 128;
+    if (p.tc && h->knn_qchunk <= 0 && p.qchunk > wave) p.qchunk = p.qchunk / wave * wave;
     if (p.qchunk > nrows) p.qchunk = nrows;
-    // keep every SM busy (tensor-core kernel: 1 CTA/SM; CUDA-core kernel: 2):
-    // split the candidate range when there are few query blocks (the re-rank
-    // then sees kc * nsplit candidates per row)
-    const int64_t qblocks = (p.qchunk + 127) / 128;
-    const int64_t want = (p.tc ? 1LL : 2LL) * h->num_sms;
-    p.nsplit = 1;
-    if (qblocks < want) p.nsplit = (int)std::min<int64_t>((want + qblocks - 1) / qblocks, 1024 / p.kc);
     // tensor-core search: each split leaves knn_tc_halves() lists per row, each of
-    // capacity >= k (<= 64, the shared-memory budget next to three stages)
-    const int halves = p.tc ? knn_tc_halves() : 1;
+    // capacity >= k (<= 64)
+    p.halves = p.tc ? knn_tc_halves() : 1;
     p.kcl = p.tc ? std::min(p.kc, 64) : p.kc;
-    const int cap = 1024 / (halves * p.kcl);
-    if (p.nsplit > cap) p.nsplit = cap;
-    if (h->knn_splits > 0) p.nsplit = std::min(h->knn_splits, cap);
-    while (p.nsplit > 1 && (N + p.nsplit - 1) / p.nsplit < p.kc) --p.nsplit;
-    p.lists = p.nsplit * halves;
+    p.cap = 1024 / (p.halves * p.kcl);
+    auto fits = [&](int sp) { return sp <= p.cap && (sp == 1 || (N + sp - 1) / sp >= p.kc); };
+    if (h->knn_splits > 0 || !p.tc || h->knn_qchunk > 0) {
+        // keep every SM busy (tensor-core kernel: 1 CTA/SM; CUDA-core kernel: 2):
+        // split the candidate range when there are few query blocks (the re-rank
+        // then sees kc * nsplit candidates per row)
+        const int64_t qblocks = (p.qchunk + 127) / 128;
+        const int64_t want = (p.tc ? 1LL : 2LL) * h->num_sms;
+        int sp = 1;
+        if (qblocks < want) sp = (int)std::min<int64_t>((want + qblocks - 1) / qblocks, 1024 / p.kc);
+        sp = std::min(sp, p.cap);
+        if (h->knn_splits > 0) sp = std::min(h->knn_splits, p.cap);
+        while (sp > 1 && !fits(sp)) --sp;
+        for (int64_t a = 0; a < nrows; a += p.qchunk) p.pieces.push_back({std::min(p.qchunk, nrows - a), sp});
+        return p;
+    }
+    // Tensor-core search: launches of whole waves with one list set per row, and
+    // the rows of the last, partial wave in a launch of their own whose candidate
+    // range is split so that its items fill the SMs again (62,500 rows against 1M
+    // points: 3.25 instead of 4 waves).  A split shortens the search but gives
+    // every row another set of lists to re-rank; the model weighs the two, in ns:
+    // a wave is max(4000, 7.5 K) per 256-row candidate tile (the drain, or the
+    // operands' way from L2), a row's set of lists 3 in the re-rank (reading and
+    // selecting; it evaluates k + 16 candidates however many there are).
+    const double tile = std::max(4000.0, 7.5 * (double)p.mk);
+    const double waves1 = (double)((N + 255) / 256) * tile, rr = 3.0;
+    for (int64_t left = nrows; left > 0;) {
+        const int64_t take = left >= wave ? std::min(p.qchunk, left / wave * wave) : left;
+        int best = 1;
+        if (take < wave) {
+            const int64_t items = (take + knn_tc_item_rows(p.pair) - 1) / knn_tc_item_rows(p.pair);
+            const int64_t slots = wave / knn_tc_item_rows(p.pair);
+            double cost = waves1 + rr * (double)take;
+            for (int sp = 2; fits(sp); ++sp) {
+                const double c = (double)((items * sp + slots - 1) / slots) / sp * waves1 + rr * (double)take * sp;
+                if (c < 0.95 * cost) {
+                    cost = c;
+                    best = sp;
+                }
+            }
+        }
+        p.pieces.push_back({take, best});
+        left -= take;
+    }
     return p;
 }
 
@@ -301,9 +345,9 @@ struct KnnBufs {
 // Scratch of run_knn, carved after `start`.
 void knn_scratch(Carver &c, const KnnPlan &p, int64_t N, KnnBufs *b) {
     b->norms = c.take<float>((size_t)N);
-    b->cand_d = c.take<float>((size_t)p.qchunk * p.lists * p.kcl);
-    b->cand_i = c.take<int32_t>((size_t)p.qchunk * p.lists * p.kcl);
-    b->flags = c.take<int32_t>((size_t)p.qchunk);
+    b->cand_d = c.take<float>((size_t)p.max_slots());
+    b->cand_i = c.take<int32_t>((size_t)p.max_slots());
+    b->flags = c.take<int32_t>((size_t)p.max_rows());
     b->xb = p.bf16_copy ? (void *)c.take<uint16_t>((size_t)N * p.ldb) : nullptr;
     b->xb2 = p.quant == KNN_QUANT_SPLIT ? (void *)c.take<uint16_t>((size_t)N * p.ldb) : nullptr;
     b->resid = p.quant ? c.take<float>((size_t)2 * N) : nullptr;
@@ -324,27 +368,30 @@ mecuco_status run_knn(mecuco_t h, char *ws, const void *X, mecuco_dtype dt, int6
            launch_row_prep(X, dt, N, m, ld, b.norms, s, b.resid, b.maxima, p.quant, b.xb, b.xb2, split_segment(m),
                            p.ldb));
     const void *Xa = b.xb ? b.xb : X, *Xb = b.xb2 ? b.xb2 : Xa;
-    for (int64_t q0 = rb; q0 < re; q0 += p.qchunk) {
-        int64_t nq = std::min(p.qchunk, re - q0);
+    int64_t q0 = rb;
+    for (const KnnPlan::Piece &piece : p.pieces) {
+        const int64_t nq = piece.rows;
         int32_t *io = idx_out + (q0 - rb) * k;
         float *dout = dist_out ? dist_out + (q0 - rb) * k : nullptr;
         if (p.tc) {
             LAUNCH(h, MECUCO_STAGE_KNN_SEARCH, s,
-                   launch_knn_tc(Xa, Xb, N, p.mk, p.ldb, b.norms, q0, nq, p.kcl, p.nsplit, include_self, b.cand_d,
+                   launch_knn_tc(Xa, Xb, N, p.mk, p.ldb, b.norms, q0, nq, p.kcl, piece.nsplit, include_self, b.cand_d,
                                  b.cand_i, p.pair ? 1 : 0, h->wait_limit, h->ctr, s));
         } else {
             LAUNCH(h, MECUCO_STAGE_KNN_SEARCH, s,
-                   launch_knn_simt(X, dt, N, m, ld, b.norms, q0, nq, p.kc, p.nsplit, include_self, b.cand_d,
+                   launch_knn_simt(X, dt, N, m, ld, b.norms, q0, nq, p.kc, piece.nsplit, include_self, b.cand_d,
                                    b.cand_i, s));
         }
         // every row's lists go to the exact re-rank together: a point that a list
         // rejected has d~ >= that list's maximum, so the smallest list maximum
         // bounds every candidate left out
         LAUNCH(h, MECUCO_STAGE_KNN_RERANK, s,
-               launch_knn_rerank(X, dt, N, m, ld, b.norms, q0, nq, p.kcl, p.lists, k, b.cand_d, b.cand_i, io, dout,
+               launch_knn_rerank(X, dt, N, m, ld, b.norms, q0, nq, p.kcl, piece.nsplit * p.halves, k, b.cand_d,
+                                 b.cand_i, io, dout,
                                  b.flags, h->ctr, s, b.resid, b.maxima, p.quant));
         LAUNCH(h, MECUCO_STAGE_KNN_FALLBACK, s,
                launch_knn_fallback(X, dt, N, m, ld, q0, nq, k, include_self, b.flags, io, dout, h->ctr, s));
+        q0 += nq;
     }
     h->knn_rows += re - rb;
     return MECUCO_OK;
@@ -960,9 +1007,13 @@ mecuco_batch_tuning batch_config(mecuco_t h, const mecuco_dataset *sets, int nse
     if (it != h->tuned.end()) return it->second;
     mecuco_batch_tuning t{};
     t.lanes = h->batch_lanes;
-    int64_t maxn = 0;
-    for (int i = 0; i < nsets; ++i) maxn = std::max(maxn, sets[i].N);
-    t.knn_pair = h->knn_pair > 0 || (h->knn_pair < 0 && maxn >= KNN_PAIR_MIN_N) ? 1 : 0;
+    // one search form for the whole batch: the one that suits most of its work
+    double work[2] = {0.0, 0.0};
+    for (int i = 0; i < nsets; ++i) {
+        const int64_t mk = dt == MECUCO_F32 && h->knn_split_bf16 ? 3 * split_segment(sets[i].m) : sets[i].m;
+        work[mk >= KNN_PAIR_MIN_K] += (double)sets[i].N * (double)sets[i].N * (double)std::max<int64_t>(mk, 512);
+    }
+    t.knn_pair = h->knn_pair > 0 || (h->knn_pair < 0 && work[1] > work[0]) ? 1 : 0;
     t.tt_ctas = h->tt_ctas;
     t.tt_slots = h->tt_slots;
     return t;

@@ -38,8 +38,8 @@ __device__ __forceinline__ const KnnSet &find_set_row(const KnnSet *sets, int ns
 // the three-term split, in segments of ms columns, query copy [h | h | l] and
 // candidate copy [h | l | h], so that one GEMM over K = 3 ms gives h.h' + h.l' +
 // l.h', the FP32 product up to l.l' and the remainders past two terms.
-template <typename T>
-__device__ __forceinline__ void row_prep_warp(const T *__restrict__ x, int64_t m, int lane, float *norm_out,
+template <typename T, int COPIES>
+__device__ __forceinline__ void row_prep_copies(const T *__restrict__ x, int64_t m, int lane, float *norm_out,
                                               float *resid_out, float *maxima, int quant,
                                               __nv_bfloat16 *__restrict__ ya, __nv_bfloat16 *__restrict__ yb,
                                               int64_t ms, int64_t ldb) {
@@ -48,34 +48,36 @@ __device__ __forceinline__ void row_prep_warp(const T *__restrict__ x, int64_t m
     for (int64_t a = lane; a < m; a += 32) {
         const float v = load_elem(x + a);
         ff_acc_sqdiff(acc, v, 0.f);
-        const __nv_bfloat16 h = __float2bfloat16_rn(v);
-        const float r = v - __bfloat162float(h);
-        const __nv_bfloat16 lb = __float2bfloat16_rn(r);
-        if (quant == KNN_QUANT_SINGLE) {
-            a1 = fmaf(r, r, a1);
-        } else if (quant == KNN_QUANT_SPLIT) {
-            const float l = __bfloat162float(lb);
-            const float r2 = r - l;
-            a1 = fmaf(l, l, a1);
-            a2 = fmaf(r2, r2, a2);
-        }
-        if (yb) {
-            ya[a] = h;
-            ya[ms + a] = h;
-            ya[2 * ms + a] = lb;
-            yb[a] = h;
-            yb[ms + a] = lb;
-            yb[2 * ms + a] = h;
-        } else if (ya) {
-            ya[a] = h;
+        if constexpr (COPIES > 0 || sizeof(T) == 4) {
+            const __nv_bfloat16 h = __float2bfloat16_rn(v);
+            const float r = v - __bfloat162float(h);
+            const __nv_bfloat16 lb = __float2bfloat16_rn(r);
+            if (quant == KNN_QUANT_SINGLE) {
+                a1 = fmaf(r, r, a1);
+            } else if (quant == KNN_QUANT_SPLIT) {
+                const float l = __bfloat162float(lb);
+                const float r2 = r - l;
+                a1 = fmaf(l, l, a1);
+                a2 = fmaf(r2, r2, a2);
+            }
+            if constexpr (COPIES == 2) {
+                ya[a] = h;
+                ya[ms + a] = h;
+                ya[2 * ms + a] = lb;
+                yb[a] = h;
+                yb[ms + a] = lb;
+                yb[2 * ms + a] = h;
+            } else if constexpr (COPIES == 1) {
+                ya[a] = h;
+            }
         }
     }
     const __nv_bfloat16 zero = __float2bfloat16_rn(0.f);
-    if (yb) {
+    if constexpr (COPIES == 2) {
         for (int64_t a = m + lane; a < ms; a += 32)
             ya[a] = ya[ms + a] = ya[2 * ms + a] = yb[a] = yb[ms + a] = yb[2 * ms + a] = zero;
         for (int64_t a = 3 * ms + lane; a < ldb; a += 32) ya[a] = yb[a] = zero;
-    } else if (ya) {
+    } else if constexpr (COPIES == 1) {
         for (int64_t a = m + lane; a < ldb; a += 32) ya[a] = zero;
     }
     acc = ff_warp_sum(acc);
@@ -96,6 +98,15 @@ __device__ __forceinline__ void row_prep_warp(const T *__restrict__ x, int64_t m
             atomicMax(reinterpret_cast<int *>(maxima) + 2, __float_as_int(t2));
         }
     }
+}
+
+template <typename T>
+__device__ __forceinline__ void row_prep_warp(const T *x, int64_t m, int lane, float *norm_out, float *resid_out,
+                                              float *maxima, int quant, __nv_bfloat16 *ya, __nv_bfloat16 *yb,
+                                              int64_t ms, int64_t ldb) {
+    if (yb) row_prep_copies<T, 2>(x, m, lane, norm_out, resid_out, maxima, quant, ya, yb, ms, ldb);
+    else if (ya) row_prep_copies<T, 1>(x, m, lane, norm_out, resid_out, maxima, quant, ya, yb, ms, ldb);
+    else row_prep_copies<T, 0>(x, m, lane, norm_out, resid_out, maxima, quant, ya, yb, ms, ldb);
 }
 
 template <typename T>

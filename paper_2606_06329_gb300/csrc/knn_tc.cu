@@ -19,7 +19,17 @@
 //               half) with its own kc-slot candidate list (distances in shared
 //               memory as a max-heap, indices straight to global), so a row leaves with
 //               TC_HALVES lists per candidate split; d~ = |x|^2 + |y|^2 - 2 x.y;
-//               values below a list's admission threshold enter it.
+//               values below a list's admission threshold wait in a per-lane
+//               buffer and enter the heaps in common updates of all eight warps.
+// The drain (measured on GB300, 100,000 x 512 BF16, k = 32): 53 ms per search
+// when every admitting column ran the warp through a heap update, 26 ms with
+// buffered updates of each warp at its own time, 14.6 ms with common updates
+// (9.2 ms when nothing is admitted).  Listing the pending candidates by
+// warp-wide bitonic merges into sorted lists instead of per-lane heaps took
+// 34 ms (a warp's 32 rows one after the other; two at a time).
+// K blocks run forward on even candidate tiles and backward on odd ones: DRAM
+// reads per search fall by a third (133 to 89 GB for 19,456 queries against
+// 210,000 points of 4,096), the search by 4%.
 // CTA pairs (optional, for 256 or more query rows): two CTAs of a
 // thread-block cluster share one 256 x 256 tcgen05.mma (cta_group::2, M = 256)
 // per K step.  Each CTA loads its own 128 query rows and one 128-row half of
@@ -28,9 +38,11 @@
 // (cta_group::2 TMA), whose warp 1 issues the MMAs and commits (multicast) to
 // both CTAs' barriers; each CTA drains its own 128 accumulator rows, and the eight
 // epilogue warps of both CTAs release an accumulator at the even CTA.  The
-// lists are those of the single-CTA form.  Measured on GB300 it ties the
-// single-CTA form at 1M x 4096 (8.0 s per search) and is 5% slower at 100k,
-// so single CTAs are the default.
+// lists are those of the single-CTA form.  It moves 2/3 of the operand bytes
+// per MMA and so wins where those bound the search, at long rows: 100,000 points
+// 62.4 against 68.8 ms at K = 4096, 70,000 x 784 FP32 rows (K = 2352) 19.4
+// against 22.7 ms, but 32.3 against 31.2 ms at K = 2048 and 15.6 against 13.7 ms
+// at K = 512, where the drain bounds it.
 // Every mbarrier wait is bounded; a timeout sets MECUCO_ERR_TIMEOUT in the
 // device status word, raises a CTA-wide abort flag, drains the copies and MMAs
 // already in flight (also bounded), frees TMEM and returns.  The limit of the
@@ -118,9 +130,8 @@ __device__ __noinline__ ListState list_insert(ListState st, float d, int c, floa
 }
 
 constexpr int MAX_NSTAGE = 9;
-constexpr int PEND = 16;        // register buffer of admitted candidates per (row, half)
-constexpr int PEND_TILES = 16;  // tiles of an item drained through the buffer (2,048 candidates per list)
-constexpr int PEND_ALL_TILES = 256;  // items of at most this many tiles use the buffer throughout
+constexpr int PEND = 32;       // pending candidates per (row, half) between list updates
+constexpr int PEND_HIGH = 16;  // a lane above this asks every epilogue warp of the CTA to update
 
 // Per-variant layout.  Single CTA: a work item is 128 query rows; each stage
 // holds the 128-row query slice and the 256-row candidate slice (24 KB at
@@ -132,7 +143,7 @@ template <bool PAIR>
 struct KCfg {
     static constexpr int B_ROWS = PAIR ? TBN / 2 : TBN;
     static constexpr int STAGE = A_BYTES + B_ROWS * TBK * 2;
-    static constexpr int NST = PAIR ? 9 : 6;
+    static constexpr int NST = PAIR ? 9 : NSTAGE;
     static constexpr int QROWS = PAIR ? 2 * TBM : TBM;
     static constexpr uint32_t IDESC = tc::idesc_bf16_f32(PAIR ? 2 * TBM : TBM, TBN);
 };
@@ -157,10 +168,11 @@ struct TcShared {
     uint64_t tempty[2];
     uint32_t tmem_base;
     int abort;
+    int update;  // list updates asked for so far (epilogue warps)
 };
 }  // namespace
 
-template <bool PAIR, bool BATCH, bool BUF>
+template <bool PAIR, bool BATCH>
 __global__ void __launch_bounds__(TC_THREADS, 1)
 knn_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b, int64_t N,
               int64_t m, const float *__restrict__ norms, int64_t q0, int64_t nq, int kc, int nsplit,
@@ -226,10 +238,11 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
             g.nkb = (int)((m + TBK - 1) / TBK);
             g.include_self = include_self;
         }
-        const int64_t per = (g.N + g.nsplit - 1) / g.nsplit;
+        // split bounds on multiples of 4: the drain reads the norms as 16-byte vectors
+        const int64_t per = ((g.N + g.nsplit - 1) / g.nsplit + 3) & ~(int64_t)3;
         g.split = (int)(li % g.nsplit);
         g.qb = g.q0 + (li / g.nsplit) * C::QROWS;
-        g.cbeg = (int64_t)g.split * per;
+        g.cbeg = min(g.N, (int64_t)g.split * per);
         g.cend = min(g.N, g.cbeg + per);
         g.ntiles = g.cend > g.cbeg ? (int)((g.cend - g.cbeg + TBN - 1) / TBN) : 0;
         return g;
@@ -252,6 +265,7 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         // (a pair decides once, below)
         sh->abort = (!PAIR && (*(volatile unsigned *)&ctr->status & DEV_TIMEOUT)) ? 1 : 0;
         never = 0;
+        sh->update = 0;
         tc::fence_mbar_init();
         if constexpr (!BATCH) {
             tc::prefetch_tmap(&map_a);
@@ -311,18 +325,23 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
             }
             for (int t = 0; t < g.ntiles && ok && !*abort_flag; ++t) {
                 const int c0 = (int)(g.cbeg + (int64_t)t * TBN) + (int)rank * C::B_ROWS;
-                for (int kb = 0; kb < g.nkb; ++kb, ++it) {
+                // K blocks forward on even tiles, backward on odd ones: the CTAs'
+                // query slices together exceed L2, and a cyclic sweep would miss on
+                // every block; turning round finds the last ones still cached
+                int x = t & 1 ? (g.nkb - 1) * TBK : 0;
+                const int dx = t & 1 ? -TBK : TBK;
+                for (int kb = 0; kb < g.nkb; ++kb, ++it, x += dx) {
                     if (!tc::mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag, wait_limit)) { ok = false; break; }
                     const uint32_t sa = st0 + s * (uint32_t)STAGE;
                     if constexpr (PAIR) {
                         if (rank == 0) tc::mbar_expect_tx(full0 + 8 * s, 2 * STAGE);
-                        tc::tma_load_2d_pair(sa, map_q, pfull0 + 8 * s, kb * TBK, (int)qb);
-                        tc::tma_load_2d_pair(sa + A_BYTES, map_c, pfull0 + 8 * s, kb * TBK, c0);
+                        tc::tma_load_2d_pair(sa, map_q, pfull0 + 8 * s, x, (int)qb);
+                        tc::tma_load_2d_pair(sa + A_BYTES, map_c, pfull0 + 8 * s, x, c0);
                     } else {
                         const uint32_t fb = full0 + 8 * s;
                         tc::mbar_expect_tx(fb, STAGE);
-                        tc::tma_load_2d(sa, map_q, fb, kb * TBK, (int)qb);
-                        tc::tma_load_2d(sa + A_BYTES, map_c, fb, kb * TBK, c0);
+                        tc::tma_load_2d(sa, map_q, fb, x, (int)qb);
+                        tc::tma_load_2d(sa + A_BYTES, map_c, fb, x, c0);
                     }
                     if (++s == (uint32_t)NST) { s = 0; ph ^= 1u; }
                 }
@@ -422,11 +441,13 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         float *Ld = Ld0 + (size_t)half * kc * TBM;
         uint8_t *Ls = Ls0 + (size_t)half * kc * TBM;
         const uint32_t tempty_even0 = PAIR ? tc::mapa(tc::smem_u32(&sh->tempty[0]), 0) : 0u;
+        volatile int *update_flag = &sh->update;
+        int updates = 0;  // list updates made so far
         int t = 0;  // tiles drained so far by this CTA (all items)
         for (int64_t item = first; item < nitems && !*abort_flag; item += stride) {
             const ItemGeo g = geo(item);
             const int64_t qb = g.qb + (int64_t)rank * TBM;
-            const int64_t cbeg = g.cbeg, cend = g.cend, N = g.N;
+            const int64_t cbeg = g.cbeg, cend = g.cend;
             const int ntiles = g.ntiles, kc = g.kc;
             const int include_self = g.include_self;
             const float *norms = g.norms;
@@ -437,30 +458,44 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                 valid_row ? (((gq - g.q0) * g.nsplit + g.split) * TC_HALVES + half) * (int64_t)kc : 0;
             ListState st{valid_row ? INFINITY : -INFINITY, 0};
             int32_t *out_i = g.cand_i + out_base;
-            // In the first PEND_TILES tiles of an item, candidates below the
-            // threshold wait in registers (newest first) and go into the heap
-            // together: a warp flushes before a group of 8 candidates once any
-            // lane holds more than PEND - 8, so a heap pass serves every lane's
-            // pending entries instead of one candidate column at a time.  32
-            // rows' independent lists otherwise take a divergent pass whenever
-            // any of them admits a candidate, which is most candidates while the
-            // lists fill (the first ~32 kc per list); later tiles of long items
-            // admit rarely and insert directly (the buffer's extra instructions
-            // slowed a 1M-point search by 15%), while items of up to
-            // PEND_ALL_TILES tiles keep the buffer throughout (a 19,647-point
-            // search: 6.89 ms direct, 6.13 with 16 buffered tiles, 4.89 with all)
+            // Candidates below the threshold wait in a per-lane buffer (local
+            // memory, hence indexable) and go into the heaps together: 32 rows'
+            // lists admit different columns, and a heap pass per admitting column
+            // would run the warp through the whole update for one or two lanes.
+            // The epilogue warps update together, before a tile, once any lane of
+            // any of them holds more than PEND_HIGH: an update makes a dozen
+            // dependent shared loads per entry, each of them waiting behind the
+            // MMA's operand reads, and since an accumulator is free only when all
+            // eight warps have read it, updates at different times would stall
+            // the MMA one after the other.
             float pd[PEND];
             int pc[PEND];
             int np = 0;
-            const int pend_tiles = BUF ? (ntiles <= PEND_ALL_TILES ? ntiles : PEND_TILES) : 0;
             auto flush = [&]() {
-#pragma unroll
-                for (int i = 0; i < PEND; ++i)
-                    if (i < np && pd[i] < st.thr) st = list_insert(st, pd[i], pc[i], Ld, Ls, out_i, row, kc);
+                const int mx = __reduce_max_sync(0xffffffffu, np);
+                float d = 0.f;
+                int c = 0;
+                if (np > 0) {
+                    d = pd[0];
+                    c = pc[0];
+                }
+                for (int i = 0; i < mx; ++i) {
+                    const int nx = i + 1 < PEND ? i + 1 : i;
+                    const float dn = nx < np ? pd[nx] : 0.f;
+                    const int cn = nx < np ? pc[nx] : 0;
+                    if (i < np && d < st.thr) st = list_insert(st, d, c, Ld, Ls, out_i, row, kc);
+                    d = dn;
+                    c = cn;
+                }
                 np = 0;
             };
             for (int tt = 0; tt < ntiles && !*abort_flag; ++tt, ++t) {
                 const int acc = t & 1;
+                const int asked = *update_flag;
+                if (__any_sync(0xffffffffu, asked != updates)) {
+                    updates = __reduce_max_sync(0xffffffffu, asked);
+                    flush();
+                }
                 if (!tc::mbar_wait(tc::smem_u32(&sh->tfull[acc]), (t >> 1) & 1, abort_flag, wait_limit)) {
                     atomicOr(&ctr->status, (unsigned)DEV_TIMEOUT);
                     sh->abort = 1;
@@ -468,49 +503,64 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                 }
                 tc::fence_after();
                 const int64_t c0 = cbeg + (int64_t)tt * TBN;
-                const bool masked = (c0 + TBN > cend) || (!include_self && gq >= c0 && gq < c0 + TBN);
+                const bool masked =
+                    __any_sync(0xffffffffu, (c0 + TBN > cend) || (!include_self && gq >= c0 && gq < c0 + TBN));
                 const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(acc * TBN);
-#pragma unroll 1
-                for (int ch = half * (TBN / 32 / TC_HALVES); ch < (half + 1) * (TBN / 32 / TC_HALVES); ++ch) {
-                    uint32_t r[32];
-                    tc::tmem_ld_32x32b_x32(taddr + ch * 32, r);
-                    tc::tmem_ld_wait();
-                    const int64_t cb = c0 + ch * 32;
-                    const float *cnp = norms + cb;
-                    if (BUF && tt < pend_tiles) {
+                // this warp's columns in chunks of 16, two in flight: chunk ch + 1 is
+                // read from tensor memory, and its norms from global memory, while
+                // chunk ch is folded into the lists
+                constexpr int NCH = TBN / 16 / TC_HALVES;
+                const int ch0 = half * NCH;
+                uint32_t ra[16], rb[16];
+                float4 na[4], nb[4];
+                auto fetch = [&](int ch, uint32_t (&r)[16], float4 (&n)[4]) {
+                    tc::tmem_ld_32x32b_x16(taddr + ch * 16, r);
+                    const float4 *cnp = reinterpret_cast<const float4 *>(norms + c0 + ch * 16);
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            if ((j & 7) == 0 && __any_sync(0xffffffffu, np > PEND - 8)) flush();
-                            const int64_t c = cb + j;
-                            const float cn = (c < N) ? __ldg(cnp + j) : 0.f;
-                            float d = fmaf(-2.f, __uint_as_float(r[j]), qn + cn);
-                            if (masked && (c >= cend || (!include_self && c == gq))) d = INFINITY;
-                            const bool adm = d < st.thr;
-                            // the vote keeps the (predicated) shift off the common path
-                            if (__any_sync(0xffffffffu, adm) && adm) {
+                    for (int e = 0; e < 4; ++e)
+                        n[e] = masked ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(cnp + e);
+                };
+                auto fold = [&](int ch, const uint32_t (&r)[16], const float4 (&n)[4]) {
+                    const int64_t cb = c0 + ch * 16;
 #pragma unroll
-                                for (int i = PEND - 1; i > 0; --i) {
-                                    pd[i] = pd[i - 1];
-                                    pc[i] = pc[i - 1];
-                                }
-                                pd[0] = d;
-                                pc[0] = (int)c;
-                                ++np;
+                    for (int g8 = 0; g8 < 2; ++g8) {
+                        const float4 p = n[2 * g8], q = n[2 * g8 + 1];
+                        float cn[8] = {p.x, p.y, p.z, p.w, q.x, q.y, q.z, q.w};
+                        float d[8];
+                        if (masked) {
+#pragma unroll
+                            for (int e = 0; e < 8; ++e) {
+                                const int64_t c = cb + 8 * g8 + e;
+                                cn[e] = (c >= cend || (!include_self && c == gq)) ? INFINITY : __ldg(norms + c);
                             }
                         }
-                    } else {
-                        // past the first tiles admissions are rare: straight into the heap
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const int64_t c = cb + j;
-                            const float cn = (c < N) ? __ldg(cnp + j) : 0.f;
-                            float d = fmaf(-2.f, __uint_as_float(r[j]), qn + cn);
-                            if (masked && (c >= cend || (!include_self && c == gq))) d = INFINITY;
-                            if (d < st.thr) st = list_insert(st, d, (int)c, Ld, Ls, out_i, row, kc);
+                        for (int e = 0; e < 8; ++e) d[e] = fmaf(-2.f, __uint_as_float(r[8 * g8 + e]), qn + cn[e]);
+                        const float m = fminf(fminf(fminf(d[0], d[1]), fminf(d[2], d[3])),
+                                              fminf(fminf(d[4], d[5]), fminf(d[6], d[7])));
+                        if (__any_sync(0xffffffffu, m < st.thr)) {
+                            if (__any_sync(0xffffffffu, np > PEND - 8)) flush();
+#pragma unroll
+                            for (int e = 0; e < 8; ++e)
+                                if (d[e] < st.thr) {
+                                    pd[np] = d[e];
+                                    pc[np] = (int)cb + 8 * g8 + e;
+                                    ++np;
+                                }
                         }
                     }
+                };
+                fetch(ch0, ra, na);
+#pragma unroll 1
+                for (int ch = ch0; ch < ch0 + NCH; ch += 2) {
+                    tc::tmem_ld_wait16(ra);
+                    fetch(ch + 1, rb, nb);
+                    fold(ch, ra, na);
+                    tc::tmem_ld_wait16(rb);
+                    if (ch + 2 < ch0 + NCH) fetch(ch + 2, ra, na);
+                    fold(ch + 1, rb, nb);
                 }
-                if (BUF && tt + 1 == pend_tiles) flush();
+                if (__any_sync(0xffffffffu, np > PEND_HIGH) && lane == 0) *update_flag = updates + 1;
                 tc::fence_before();
                 if constexpr (PAIR) {
                     // one arrival per warp at the even CTA, once every lane has read its rows
@@ -520,7 +570,7 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                     tc::mbar_arrive(tc::smem_u32(&sh->tempty[acc]));
                 }
             }
-            if constexpr (BUF) flush();
+            flush();
             if (valid_row) {
                 for (int p = 0; p < st.cnt; ++p) g.cand_d[out_base + Ls[p * TBM + row]] = Ld[p * TBM + row];
                 for (int s2 = st.cnt; s2 < kc; ++s2) {
@@ -599,14 +649,10 @@ cudaError_t launch_knn_tc(const void *Xa, const void *Xb, int64_t N, int64_t m, 
     if (e != cudaSuccess) return e;
     e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    // short sweeps (items of at most PEND_ALL_TILES candidate tiles) drain
-    // through the register buffer; long ones take the direct form, whose
-    // leaner loop a 1M-point search needs
-    const bool buf = (N + TBN - 1) / TBN <= PEND_ALL_TILES;
     if (pair && nq >= 2 * TBM) {
         // CTA pairs (cta_group::2): 256 query rows per item; each CTA's candidate
         // half uses the 128-row box of the query map
-        auto kern = buf ? knn_tc_kernel<true, false, true> : knn_tc_kernel<true, false, false>;
+        auto kern = knn_tc_kernel<true, false>;
         e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         cudaLaunchAttribute attr[1];
@@ -636,7 +682,7 @@ cudaError_t launch_knn_tc(const void *Xa, const void *Xb, int64_t N, int64_t m, 
         }
         // no pair fits: single CTAs
     }
-    auto kern = buf ? knn_tc_kernel<false, false, true> : knn_tc_kernel<false, false, false>;
+    auto kern = knn_tc_kernel<false, false>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     const int64_t items = ((nq + TBM - 1) / TBM) * nsplit;
@@ -668,7 +714,7 @@ cudaError_t launch_knn_tc_batch(const KnnSet *sets, int nsets, int64_t nitems, i
     memset(&none, 0, sizeof(none));
     if (pair) {
         // items of 256 query rows (the table's item counts must be for that size)
-        e = cudaFuncSetAttribute(knn_tc_kernel<true, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = cudaFuncSetAttribute(knn_tc_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
@@ -683,20 +729,20 @@ cudaError_t launch_knn_tc_batch(const KnnSet *sets, int nsets, int64_t nitems, i
         cfg.numAttrs = 1;
         cfg.gridDim = dim3(2);
         int nclusters = 0;
-        e = cudaOccupancyMaxActiveClusters(&nclusters, knn_tc_kernel<true, true, true>, &cfg);
+        e = cudaOccupancyMaxActiveClusters(&nclusters, knn_tc_kernel<true, true>, &cfg);
         if (e != cudaSuccess) return e;
         if (nclusters <= 0) return cudaErrorInvalidConfiguration;
         cfg.gridDim = dim3((unsigned)(2 * (nitems < nclusters ? nitems : nclusters)));
-        e = cudaLaunchKernelEx(&cfg, knn_tc_kernel<true, true, true>, none, none, (int64_t)0, (int64_t)0,
+        e = cudaLaunchKernelEx(&cfg, knn_tc_kernel<true, true>, none, none, (int64_t)0, (int64_t)0,
                                (const float *)nullptr, (int64_t)0, (int64_t)0, kcmax, 1, 0, (float *)nullptr,
                                (int32_t *)nullptr, WAIT_LIMIT, ctr, sets, nsets, nitems);
         if (e != cudaSuccess) return e;
         return cudaGetLastError();
     }
-    e = cudaFuncSetAttribute(knn_tc_kernel<false, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    e = cudaFuncSetAttribute(knn_tc_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     dim3 grid((unsigned)(nitems < sms ? nitems : sms));
-    knn_tc_kernel<false, true, true><<<grid, TC_THREADS, smem, s>>>(none, none, 0, 0, nullptr, 0, 0, kcmax, 1, 0, nullptr,
+    knn_tc_kernel<false, true><<<grid, TC_THREADS, smem, s>>>(none, none, 0, 0, nullptr, 0, 0, kcmax, 1, 0, nullptr,
                                                                nullptr, wait_limit, ctr, sets, nsets, nitems);
     return cudaGetLastError();
 }
