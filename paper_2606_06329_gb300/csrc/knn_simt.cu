@@ -305,23 +305,166 @@ cudaError_t launch_knn_simt(const void *X, mecuco_dtype dt, int64_t N, int64_t m
 }
 
 // ---------------------------------------------------------------------------
-// Exact re-rank + certification.  One warp per query row.  Each candidate's
-// squared distance sum_a (x_a - y_a)^2 is accumulated as a float-float pair
-// (TwoSum of the difference, FMA TwoProd of the square), so it carries ~2^-44
-// relative error: ranks agree with an FP64 brute force except at ties closer
-// than that.  Certification: every row left out of the candidate set has
-// d~ >= thr (the smallest admission threshold of the full splits), so its true
-// distance is >= thr - e_hi, e_hi bounding the overestimate d~ - d; the row is
-// certified when thr - e_hi exceeds the exact k-th distance.  The search's
+// Exact re-rank + certification.  One warp per query row.  An exact distance is
+// sum_a (x_a - y_a)^2 as a float-float pair: the difference by TwoSum, its
+// square added to a two-term sum by FMAs, so it carries ~2^-42 relative error:
+// ranks agree with an FP64 brute force except at ties closer than that.
+// Certification: a point left out - rejected by a list, or a candidate that is
+// not evaluated here - has d~ >= some threshold thr, so its true distance is >=
+// thr - e_hi, e_hi bounding the overestimate d~ - d; it cannot enter the top k
+// when thr - e_hi exceeds the exact k-th distance theta.  The search's
 // accumulation error has no documented worst-case bound on the tensor-core
 // path and is dominated by a per-row bias (the FP32 accumulator's rounding of
 // partial sums of similar size), so e_hi is estimated a posteriori from the
-// row's own candidates: the largest observed d~ - d plus 3x the observed spread
-// of d~ - d, plus 2^-21 (|x|^2 + max |y|^2) (a few units in the last place of
-// the norms).  Rows failing the test are re-solved exactly by the full scan.
+// row's own evaluated candidates: the largest observed d~ - d plus 3x the
+// observed spread of d~ - d, plus 2^-21 (|x|^2 + max |y|^2) (a few units in the
+// last place of the norms); FP32 rows searched in BF16 add the rounding's
+// a-priori bound.
+// The lists hold two to three times as many candidates as neighbours asked for,
+// so a row first evaluates the k + RR_EXTRA smallest by d~ (a threshold found by
+// bisection), and then only those with d~ <= theta + e_hi, usually none.  Rows
+// whose lists' own threshold (the smallest maximum of the full lists) does not
+// pass the test are re-solved exactly by the full scan.
+// Measured per 100k queries against the form that evaluated and ranked every
+// candidate: 512 columns BF16, k = 32, 128 candidates 6.4 to 2.5 ms; per 70k of
+// 784 FP32 columns, k = 50 6.7 to 3.6 ms; 2,000 x 32 with 1,024 candidates a row
+// 2.98 to 0.04 ms.  Bound by the FP32 pipe (12 operations a term, in packed
+// pairs, 22 before) up to about 1,000 columns, then by the candidate rows' DRAM
+// reads.
 // ---------------------------------------------------------------------------
 constexpr int RR_WARPS = 4;
 constexpr int RR_MAXL = 1024;
+constexpr int RR_EXTRA = 16;
+constexpr int RR_CAP = 128;  // evaluated candidates kept at a time (>= 64 + RR_EXTRA + slack, a multiple of 32)
+
+namespace {
+typedef unsigned long long f2;
+__device__ __forceinline__ f2 pack2(float lo, float hi) {
+    f2 v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ float2 unpack2(f2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f2 add2(f2 a, f2 b) {
+    f2 d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+// 16 bytes of a row as packed FP32 pairs
+template <typename T>
+__device__ __forceinline__ void widen(uint4 v, f2 (&o)[8 / sizeof(T)]);
+template <>
+__device__ __forceinline__ void widen<float>(uint4 v, f2 (&o)[2]) {
+    o[0] = pack2(__uint_as_float(v.x), __uint_as_float(v.y));
+    o[1] = pack2(__uint_as_float(v.z), __uint_as_float(v.w));
+}
+template <>
+__device__ __forceinline__ void widen<__nv_bfloat16>(uint4 v, f2 (&o)[4]) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        o[e] = pack2(__uint_as_float(w[e] << 16), __uint_as_float(w[e] & 0xffff0000u));
+}
+// (hi, lo) += (x - y)^2 for two terms at once.  hi carries an offset 2^b above
+// the sum, so that it stays in one binade: h = fma(d, d, hi) loses d^2 - (h - hi)
+// exactly (h - hi is exact), which the next FMA rounds once.
+struct PairAcc {
+    f2 hi, lo;
+};
+__device__ __forceinline__ void acc_sqdiff2(PairAcc &a, f2 x, f2 y, f2 minus, f2 two) {
+    const f2 d = fma2(y, minus, x);            // x - y, rounded
+    const f2 bb = fma2(x, minus, d);           // its rounding error, by TwoSum
+    const f2 t = fma2(fma2(bb, minus, d), minus, x);
+    const f2 dl = fma2(add2(y, bb), minus, t);
+    const f2 h = fma2(d, d, a.hi);
+    const f2 er = fma2(d, d, fma2(h, minus, a.hi));
+    a.hi = h;
+    a.lo = fma2(dl, fma2(d, two, dl), add2(a.lo, er));
+}
+// order-preserving image of a float
+__device__ __forceinline__ unsigned order_key(float v) {
+    const unsigned b = __float_as_uint(v);
+    return b & 0x80000000u ? ~b : b | 0x80000000u;
+}
+}  // namespace
+
+// Exact distances of the candidates j[u] (u < 4; -1: none) from row q, one per
+// group of G lanes and u, returned in every lane of the group.  base[u]: the
+// offset, a power of two above the distance (checked: a sum that reaches it is
+// done again without).
+template <typename T>
+__device__ __forceinline__ void exact_dist4(const T *__restrict__ X, int64_t m, int64_t ld, const T *__restrict__ xq,
+                                            int64_t q, const int (&j)[4], const float (&base)[4], int G, bool vec,
+                                            ff (&out)[4]) {
+    constexpr int VEC = 16 / (int)sizeof(T), NP = VEC / 2;
+    const int lane = threadIdx.x & 31, gl = lane & (G - 1);
+    const f2 minus = pack2(-1.f, -1.f), two = pack2(2.f, 2.f);
+    const T *xr[4];
+    PairAcc acc[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        xr[u] = X + (int64_t)(j[u] >= 0 ? j[u] : q) * ld;  // an empty slot reads the query row, discarded
+        acc[u].hi = pack2(base[u], base[u]);
+        acc[u].lo = pack2(0.f, 0.f);
+    }
+    int64_t a0 = 0;
+    if (vec) {
+        const int64_t mv = m / VEC * VEC;  // vector part of the row; the tail is scalar
+        for (int64_t a = (int64_t)gl * VEC; a < mv; a += G * VEC) {
+            uint4 yv[4];
+            const uint4 qv = __ldg(reinterpret_cast<const uint4 *>(xq + a));
+#pragma unroll
+            for (int u = 0; u < 4; ++u) yv[u] = __ldg(reinterpret_cast<const uint4 *>(xr[u] + a));
+            f2 xe[NP];
+            widen<T>(qv, xe);
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                f2 ye[NP];
+                widen<T>(yv[u], ye);
+#pragma unroll
+                for (int e = 0; e < NP; ++e) acc_sqdiff2(acc[u], xe[e], ye[e], minus, two);
+            }
+        }
+        a0 = mv;
+    }
+    for (int64_t a = a0 + gl; a < m; a += G) {
+        const float x = load_elem(xq + a);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) acc_sqdiff2(acc[u], pack2(x, 0.f), pack2(load_elem(xr[u] + a), 0.f), minus, two);
+    }
+    bool over = false;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const float2 h = unpack2(acc[u].hi), l = unpack2(acc[u].lo);
+        over = over || !(h.x < 2.f * base[u]) || !(h.y < 2.f * base[u]);
+        // two sums of a lane, then the group's: renormalised float-float additions
+        ff s, e;
+        two_sum(h.x - base[u], l.x, s.hi, s.lo);
+        two_sum(h.y - base[u], l.y, e.hi, e.lo);
+        out[u] = ff_add(s, e);
+    }
+    if (__any_sync(0xffffffffu, over)) {
+        // a sum outgrew its offset (the search's distance was far too small):
+        // without one, renormalising every term
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            out[u] = ff{0.f, 0.f};
+            for (int64_t a = gl; a < m; a += G) ff_acc_sqdiff(out[u], load_elem(xq + a), load_elem(xr[u] + a));
+        }
+    }
+    for (int o = G >> 1; o > 0; o >>= 1)
+#pragma unroll
+        for (int u = 0; u < 4; ++u) out[u] = ff_add(out[u], ff_shfl_xor(out[u], o));
+}
 
 template <typename T, bool BATCH>
 __global__ void __launch_bounds__(RR_WARPS * 32)
@@ -332,6 +475,7 @@ knn_rerank_kernel(const T *__restrict__ X_, int64_t N_, int64_t m_, int64_t ld_,
                   int32_t *__restrict__ flags_, DevCounters *ctr, const KnnSet *__restrict__ sets, int nsets,
                   int lmax, const float *__restrict__ resid_, const float *__restrict__ maxima_, int quant_) {
     extern __shared__ float rsm[];
+    constexpr unsigned FULL = 0xffffffffu;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     int64_t qi = (int64_t)blockIdx.x * RR_WARPS + w;  // the launch's row (the batch's row when batched)
     if (qi >= nq) return;
@@ -367,140 +511,207 @@ knn_rerank_kernel(const T *__restrict__ X_, int64_t N_, int64_t m_, int64_t ld_,
         quant = d.quant;
     }
     const int L = kc * nsplit;
-    const int LS = BATCH ? lmax : L;  // per-warp shared-memory stride
-    float *hi = rsm + (size_t)w * LS * 3;
-    float *lo = hi + L;
-    int *ci = reinterpret_cast<int *>(lo + L);
+    const int LS = BATCH ? lmax : L;  // per-warp shared-memory size in candidates
+    // the row's candidates: d~ as ordered keys and indices; the evaluated ones
+    unsigned *key = reinterpret_cast<unsigned *>(rsm + (size_t)w * (2 * LS + 4 * RR_CAP));
+    int *ci = reinterpret_cast<int *>(key + LS);
+    float *eh = reinterpret_cast<float *>(ci + LS), *el = eh + RR_CAP;
+    int *ei = reinterpret_cast<int *>(el + RR_CAP), *ec = ei + RR_CAP;
     const int64_t q = q0 + qi;
     const float *cd = cand_d + qi * (int64_t)L;
     const int32_t *cidx = cand_i + qi * (int64_t)L;
     const T *xq = X + q * ld;
+    const float nq_ = norms[q];
 
-    float err_max = -INFINITY, err_min = INFINITY, nmax = 0.f;
-    bool bad = false;
     // a complete search leaves -1 or a row of X in every slot; anything else
     // (slots a search that timed out never wrote) is skipped, never read
-    auto cand = [&](int c) {
-        int j = cidx[c];
-        if (j >= N) { bad = true; j = -1; }
-        return j;
-    };
-    auto record = [&](int c, int j, ff acc) {
-        if (j >= 0) {
-            const float e = cd[c] - acc.hi;  // overestimate of the search's distance
-            err_max = fmaxf(err_max, e);
-            err_min = fminf(err_min, e);
-            nmax = fmaxf(nmax, norms[j]);
-        } else {
-            acc.hi = INFINITY;
-        }
-        if (lane == 0) { hi[c] = acc.hi; lo[c] = acc.lo; ci[c] = j; }
-    };
-    // Rows as 16-byte vectors when every row starts 16-byte aligned: four
-    // candidates at a time, each lane summing its share of the four rows with
-    // independent compensated accumulators, so that 4 x (m / 32 / VEC) loads
-    // are in flight per lane instead of one 2- or 4-byte load per step.  The
-    // terms are the same; only the summation order differs from the scalar form.
-    constexpr int VEC = 16 / (int)sizeof(T);
-    const bool vec = (ld % VEC == 0) && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
-    int c = 0;
-    if (vec) {
-        const int64_t mv = m / VEC * VEC;  // vector part of the row; the tail is scalar
-        for (; c + 4 <= L; c += 4) {
-            int j[4];
-            const T *xr[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                j[u] = cand(c + u);
-                xr[u] = X + (int64_t)(j[u] >= 0 ? j[u] : q) * ld;  // an empty slot reads the query row, discarded
-            }
-            ff acc[4] = {{0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}, {0.f, 0.f}};
-            for (int64_t a = (int64_t)lane * VEC; a < mv; a += 32 * VEC) {
-                const uint4 qv = __ldg(reinterpret_cast<const uint4 *>(xq + a));
-                uint4 yv[4];
-#pragma unroll
-                for (int u = 0; u < 4; ++u) yv[u] = __ldg(reinterpret_cast<const uint4 *>(xr[u] + a));
-                const T *qe = reinterpret_cast<const T *>(&qv);
-#pragma unroll
-                for (int u = 0; u < 4; ++u) {
-                    const T *ye = reinterpret_cast<const T *>(&yv[u]);
-#pragma unroll
-                    for (int e = 0; e < VEC; ++e) ff_acc_sqdiff(acc[u], to_f32(qe[e]), to_f32(ye[e]));
-                }
-            }
-            for (int64_t a = mv + lane; a < m; a += 32)
-#pragma unroll
-                for (int u = 0; u < 4; ++u) ff_acc_sqdiff(acc[u], load_elem(xq + a), load_elem(xr[u] + a));
-#pragma unroll
-            for (int u = 0; u < 4; ++u) record(c + u, j[u], ff_warp_sum(acc[u]));
-        }
-    }
-    for (; c < L; ++c) {
-        const int j = cand(c);
-        ff acc{0.f, 0.f};
-        if (j >= 0) {
-            const T *xj = X + (int64_t)j * ld;
-            for (int64_t a = lane; a < m; a += 32) ff_acc_sqdiff(acc, load_elem(xq + a), load_elem(xj + a));
-            acc = ff_warp_sum(acc);
-        }
-        record(c, j, acc);
-    }
-    __syncwarp();
-    // thresholds: a split whose list is full admitted only d~ < its max
+    bool bad = false;
+    unsigned kmin = 0xffffffffu, kmax = 0u;
+    int live = 0;
     float thr = INFINITY;
     for (int sp = 0; sp < nsplit; ++sp) {
+        // a list that is full admitted only d~ < its maximum
         float mx = -INFINITY;
         bool full = true;
-        for (int c = lane; c < kc; c += 32) {
-            float v = cd[sp * kc + c];
-            full = full && (ci[sp * kc + c] >= 0);
-            mx = fmaxf(mx, v);
+        for (int c = sp * kc + lane; c < (sp + 1) * kc; c += 32) {
+            int j = cidx[c];
+            if (j >= N) { bad = true; j = -1; }
+            const float d = cd[c];
+            const unsigned kk = order_key(d);
+            key[c] = kk;
+            ci[c] = j;
+            mx = fmaxf(mx, d);
+            full = full && j >= 0;
+            if (j >= 0) {
+                ++live;
+                kmin = min(kmin, kk);
+                kmax = max(kmax, kk);
+            }
         }
         mx = warp_max(mx);
-        full = __all_sync(0xffffffffu, full);
-        if (full) thr = fminf(thr, mx);
+        if (__all_sync(FULL, full)) thr = fminf(thr, mx);
     }
-    // rank each candidate by (hi, lo, index); write the k best in order
-    float theta = 0.f;
-    for (int c = lane; c < L; c += 32) {
-        int j = ci[c];
-        if (j < 0) continue;
-        ff me{hi[c], lo[c]};
-        int rank = 0;
-        for (int o = 0; o < L; ++o) {
-            if (ci[o] < 0) continue;
-            if (ff_less(ff{hi[o], lo[o]}, ci[o], me, j)) ++rank;
-        }
-        if (rank < k) {
-            idx_out[qi * k + rank] = j;
-            if (dist_out) dist_out[qi * k + rank] = me.hi + me.lo;
-        }
-        if (rank == k - 1) theta = me.hi;
+    live = __reduce_add_sync(FULL, live);
+    kmin = __reduce_min_sync(FULL, kmin);
+    kmax = __reduce_max_sync(FULL, kmax);
+    __syncwarp();
+
+    constexpr int VEC = 16 / (int)sizeof(T);
+    const bool vec = (ld % VEC == 0) && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+    // lanes per candidate: a power of two that a narrow row still fills
+    int G = 32;
+    while (G > 4 && (vec ? (G / 2) * VEC : G / 2) >= m) G >>= 1;
+    const int per = 32 / G, gid = lane / G;
+
+    // the a-priori part of e_hi (FP32 rows searched in BF16): a bound on |x.y -
+    // (the search's product)| for any candidate y, with the dataset's largest |y|
+    // and rounding terms.
+    //   single (x = h + d):      |h||d_y| + |d||h_y| + |d||d_y|
+    //   split (x = h + l + r):   |l||l_y| + |h + l||r_y| + |r||h_y + l_y| + |r||r_y|
+    // The tensor core's FP32 accumulation stays with the estimate.
+    float e_apriori = -INFINITY;
+    if (quant != KNN_QUANT_NONE) {
+        const float t1 = resid[2 * q], t2 = resid[2 * q + 1], xn = sqrtf(nq_);
+        const float ym = sqrtf(maxima[0]), m1 = maxima[1], m2 = maxima[2];
+        const float b = quant == KNN_QUANT_SINGLE ? (xn + t1) * m1 + t1 * (ym + m1) + t1 * m1
+                                                  : t1 * m1 + (xn + t2) * m2 + t2 * (ym + m2) + t2 * m2;
+        e_apriori = 2.f * b * (1.f + 9.765625e-04f) + ldexpf(nq_ + maxima[0], -21);
     }
-    theta = warp_max(theta);
+
+    float err_max = -INFINITY, err_min = INFINITY, nmax = 0.f;
+    int n = 0;                 // evaluated candidates held (eh, el, ei)
+    unsigned done = 0u;        // candidates with key < done have been evaluated (every key is > 0)
+    unsigned want_key = 0u;    // and those below this one are to be (exclusive)
+    int want = min(live, k + RR_EXTRA);
+    float theta = INFINITY, e_hi = INFINITY;
+    auto count_below = [&](unsigned t) {  // live candidates with done <= key < t
+        int c = 0;
+        for (int i = lane; i < L; i += 32) c += ci[i] >= 0 && key[i] >= done && key[i] < t;
+        return (int)__reduce_add_sync(FULL, c);
+    };
+    // smallest t (to a few candidates) with count_below(t) >= w, at most room
+    auto key_for = [&](unsigned lo, unsigned hi, int w, int room) {
+        // invariant: count_below(lo) < w <= count_below(hi)
+        while (hi - lo > 1u) {
+            const unsigned mid = lo + (hi - lo) / 2u;
+            const int c = count_below(mid);
+            if (c >= w) {
+                hi = mid;
+                if (c <= w + 4 && c <= room) break;
+            } else {
+                lo = mid;
+            }
+        }
+        return hi;
+    };
+    for (;;) {
+        // ---- the next candidates: [done, want_key), as many as there is room for
+        if (n == 0) {
+            if (want <= 0) break;
+            want_key = key_for(kmin, kmax + 1u, want, RR_CAP);
+        }
+        const int room = RR_CAP - n;
+        const int cnt = count_below(want_key);
+        if (cnt > room) want_key = key_for(max(done, kmin), want_key, max(1, room - 4), room);
+        // (equal keys beyond the room cannot be told apart: give up, full scan)
+        int nb = 0;
+        for (int i0 = 0; i0 < L; i0 += 32) {
+            const int i = i0 + lane;
+            const bool take = i < L && ci[i] >= 0 && key[i] >= done && key[i] < want_key;
+            const unsigned mk = __ballot_sync(FULL, take);
+            const int pos = n + nb + __popc(mk & ((1u << lane) - 1u));
+            if (take && pos < RR_CAP) ec[pos] = i;
+            nb += __popc(mk);
+        }
+        const bool overflow = n + nb > RR_CAP;
+        if (overflow) nb = RR_CAP - n;
+        __syncwarp();
+        // ---- their exact distances
+        for (int c0 = n; c0 < n + nb; c0 += 4 * per) {
+            int cc[4], j[4];
+            float base[4], dt[4];
+            ff d[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                cc[u] = c0 + u * per + gid;
+                const int i = cc[u] < n + nb ? ec[cc[u]] : -1;
+                j[u] = i >= 0 ? ci[i] : -1;
+                dt[u] = i >= 0 ? cd[i] : 0.f;
+                // 2^b above twice the search's distance
+                base[u] = __uint_as_float(min((__float_as_uint(fabsf(dt[u])) & 0x7f800000u) + (2u << 23), 0x7e800000u));
+            }
+            exact_dist4<T>(X, m, ld, xq, q, j, base, G, vec, d);
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (j[u] >= 0) {
+                    const float e = dt[u] - d[u].hi;  // overestimate of the search's distance
+                    err_max = fmaxf(err_max, e);
+                    err_min = fminf(err_min, e);
+                    nmax = fmaxf(nmax, norms[j[u]]);
+                    if ((lane & (G - 1)) == 0) {
+                        eh[cc[u]] = d[u].hi;
+                        el[cc[u]] = d[u].lo;
+                        ei[cc[u]] = j[u];
+                    }
+                }
+        }
+        n += nb;
+        done = want_key;
+        __syncwarp();
+        err_max = warp_max(err_max);
+        err_min = -warp_max(-err_min);
+        nmax = warp_max(nmax);
+        e_hi = fmaxf(fmaxf(err_max, 0.f) + 3.f * (err_max - err_min) + ldexpf(nq_ + nmax, -21), e_apriori);
+        // ---- the k best of the evaluated ones, in order, to the front
+        float vh[RR_CAP / 32], vl[RR_CAP / 32];
+        int vi[RR_CAP / 32], vr[RR_CAP / 32];
+#pragma unroll
+        for (int t = 0; t < RR_CAP / 32; ++t) {
+            const int c = t * 32 + lane;
+            vr[t] = RR_CAP;
+            if (c < n) {
+                vh[t] = eh[c];
+                vl[t] = el[c];
+                vi[t] = ei[c];
+                int rank = 0;
+                for (int o = 0; o < n; ++o) rank += ff_less(ff{eh[o], el[o]}, ei[o], ff{vh[t], vl[t]}, vi[t]);
+                vr[t] = rank;
+            }
+        }
+        __syncwarp();
+#pragma unroll
+        for (int t = 0; t < RR_CAP / 32; ++t)
+            if (vr[t] < k) {
+                eh[vr[t]] = vh[t];
+                el[vr[t]] = vl[t];
+                ei[vr[t]] = vi[t];
+            }
+        __syncwarp();
+        n = min(n, k);
+        theta = n == k ? eh[k - 1] : INFINITY;
+        if (overflow) {
+            thr = -INFINITY;
+            break;
+        }
+        // ---- candidates left that could still enter: d~ <= theta + e_hi
+        const float lim = theta + e_hi;
+        want_key = lim < INFINITY ? min(order_key(lim) + 1u, kmax + 1u) : kmax + 1u;
+        if (want_key <= done || count_below(want_key) == 0) break;
+    }
+    for (int c = lane; c < n; c += 32) {
+        idx_out[qi * k + c] = ei[c];
+        if (dist_out) dist_out[qi * k + c] = eh[c] + el[c];
+    }
     if (lane == 0 && bad) atomicOr(&ctr->status, (unsigned)DEV_INVALID);
     if (lane == 0) {
-        const float spread = err_max - err_min;
-        float e_hi = fmaxf(err_max, 0.f) + 3.f * spread + ldexpf(norms[q] + nmax, -21);
-        if (quant != KNN_QUANT_NONE) {
-            // BF16 operands from FP32 rows: an a-priori bound (not estimated from
-            // the candidates) on |x.y - (the search's product)| for any
-            // candidate y, with the dataset's largest |y| and rounding terms.
-            //   single (x = h + d):      |h||d_y| + |d||h_y| + |d||d_y|
-            //   split (x = h + l + r):   |l||l_y| + |h + l||r_y| + |r||h_y + l_y| + |r||r_y|
-            // The tensor core's FP32 accumulation stays with the estimate.
-            const float t1 = resid[2 * q], t2 = resid[2 * q + 1], xq = sqrtf(norms[q]);
-            const float ym = sqrtf(maxima[0]), m1 = maxima[1], m2 = maxima[2];
-            const float b = quant == KNN_QUANT_SINGLE ? (xq + t1) * m1 + t1 * (ym + m1) + t1 * m1
-                                                      : t1 * m1 + (xq + t2) * m2 + t2 * (ym + m2) + t2 * m2;
-            const float eq = 2.f * b * (1.f + 9.765625e-04f) + ldexpf(norms[q] + maxima[0], -21);
-            e_hi = fmaxf(e_hi, eq);
-        }
-        int ok = (thr == INFINITY) || (thr - e_hi > theta);
+        // theta as before when fewer than k candidates exist: certified by thr = +inf
+        const int ok = (thr == INFINITY) || (n == k && thr - e_hi > theta);
         flags[qi] = ok ? 0 : 1;
         if (!ok) atomicAdd(&ctr->knn_uncertified, 1ull);
     }
 }
+
+size_t knn_rerank_smem(int L) { return (size_t)RR_WARPS * (2 * L + 4 * RR_CAP) * sizeof(float); }
 
 cudaError_t launch_knn_rerank(const void *X, mecuco_dtype dt, int64_t N, int64_t m, int64_t ld,
                               const float *norms, int64_t q0, int64_t nq, int kc, int nsplit, int k,
@@ -511,7 +722,7 @@ cudaError_t launch_knn_rerank(const void *X, mecuco_dtype dt, int64_t N, int64_t
     if (nq <= 0) return cudaSuccess;
     int L = kc * nsplit;
     if (L > RR_MAXL) return cudaErrorInvalidValue;
-    size_t smem = (size_t)RR_WARPS * L * 3 * sizeof(float);
+    size_t smem = knn_rerank_smem(L);
     dim3 grid((unsigned)((nq + RR_WARPS - 1) / RR_WARPS)), block(RR_WARPS * 32);
     cudaError_t e;
     if (dt == MECUCO_BF16) {
@@ -637,7 +848,7 @@ cudaError_t launch_knn_rerank_batch(const KnnSet *sets, int nsets, int64_t nrows
                                     DevCounters *ctr, cudaStream_t s) {
     if (nrows <= 0) return cudaSuccess;
     if (lmax > RR_MAXL) return cudaErrorInvalidValue;
-    size_t smem = (size_t)RR_WARPS * lmax * 3 * sizeof(float);
+    size_t smem = knn_rerank_smem(lmax);
     dim3 grid((unsigned)((nrows + RR_WARPS - 1) / RR_WARPS)), block(RR_WARPS * 32);
     cudaError_t e;
     if (dt == MECUCO_BF16) {
