@@ -280,9 +280,9 @@ KnnPlan plan_knn(mecuco_t h, const void *X, mecuco_dtype dt, int64_t N, int64_t 
     p.ldb = direct ? ld : (p.mk + 7) / 8 * 8;
     p.pair = p.tc && (h->knn_pair > 0 || (h->knn_pair < 0 && p.mk >= KNN_PAIR_MIN_K));
     p.qchunk = h->knn_qchunk > 0 ? h->knn_qchunk : (int64_t)1 << 18;
-    // query rows that one wave of the persistent search covers (tensor-core form)
+    // query rows that one wave of the search covers (one block, or pair, per SM)
     const int64_t wave = p.pair ? (int64_t)(h->num_sms / 2) * 256 : (int64_t)h->num_sms * 128;
-    if (p.tc && h->knn_qchunk <= 0 && p.qchunk > wave) p.qchunk = p.qchunk / wave * wave;
+    if (h->knn_qchunk <= 0 && p.qchunk > wave) p.qchunk = p.qchunk / wave * wave;
     if (p.qchunk > nrows) p.qchunk = nrows;
     // tensor-core search: each split leaves knn_tc_halves() lists per row, each of
     // capacity >= k (<= 64)
@@ -290,12 +290,11 @@ KnnPlan plan_knn(mecuco_t h, const void *X, mecuco_dtype dt, int64_t N, int64_t 
     p.kcl = p.tc ? std::min(p.kc, 64) : p.kc;
     p.cap = 1024 / (p.halves * p.kcl);
     auto fits = [&](int sp) { return sp <= p.cap && (sp == 1 || (N + sp - 1) / sp >= p.kc); };
-    if (h->knn_splits > 0 || !p.tc || h->knn_qchunk > 0) {
-        // keep every SM busy (tensor-core kernel: 1 CTA/SM; CUDA-core kernel: 2):
-        // split the candidate range when there are few query blocks (the re-rank
-        // then sees kc * nsplit candidates per row)
+    if (h->knn_splits > 0 || h->knn_qchunk > 0) {
+        // keep every SM busy: split the candidate range when there are few query
+        // blocks (the re-rank then sees kc * nsplit candidates per row)
         const int64_t qblocks = (p.qchunk + 127) / 128;
-        const int64_t want = (p.tc ? 1LL : 2LL) * h->num_sms;
+        const int64_t want = h->num_sms;
         int sp = 1;
         if (qblocks < want) sp = (int)std::min<int64_t>((want + qblocks - 1) / qblocks, 1024 / p.kc);
         sp = std::min(sp, p.cap);
@@ -304,22 +303,23 @@ KnnPlan plan_knn(mecuco_t h, const void *X, mecuco_dtype dt, int64_t N, int64_t 
         for (int64_t a = 0; a < nrows; a += p.qchunk) p.pieces.push_back({std::min(p.qchunk, nrows - a), sp});
         return p;
     }
-    // Tensor-core search: launches of whole waves with one list set per row, and
-    // the rows of the last, partial wave in a launch of their own whose candidate
-    // range is split so that its items fill the SMs again (62,500 rows against 1M
-    // points: 3.25 instead of 4 waves).  A split shortens the search but gives
-    // every row another set of lists to re-rank; the model weighs the two, in ns:
-    // a wave is max(4000, 7.5 K) per 256-row candidate tile (the drain, or the
-    // operands' way from L2), a row's set of lists 3 in the re-rank (reading and
-    // selecting; it evaluates k + 16 candidates however many there are).
-    const double tile = std::max(4000.0, 7.5 * (double)p.mk);
-    const double waves1 = (double)((N + 255) / 256) * tile, rr = 3.0;
+    // Launches of whole waves with one list set per row, and the rows of the
+    // last, partial wave in a launch of their own whose candidate range is split
+    // so that its items fill the SMs again (62,500 rows against 1M points: 3.25
+    // instead of 4 waves).  A split shortens the search but gives every row
+    // another set of lists to re-rank; the model weighs the two, in ns.  A wave
+    // costs, per candidate tile, max(4000, 7.5 K) on the tensor cores (256 rows;
+    // the drain, or the operands' way from L2) and 2500 + 75 m on the CUDA cores
+    // (128 rows); a row's set of lists 3 per 128 entries in the re-rank (reading
+    // and selecting: it evaluates k + 16 candidates however many there are).
+    const double tile = p.tc ? std::max(4000.0, 7.5 * (double)p.mk) : 2500.0 + 75.0 * (double)m;
+    const int64_t tile_rows = p.tc ? 256 : 128, item_rows = p.tc ? knn_tc_item_rows(p.pair) : 128;
+    const double waves1 = (double)((N + tile_rows - 1) / tile_rows) * tile, rr = 3.0 * p.halves * p.kcl / 128;
     for (int64_t left = nrows; left > 0;) {
         const int64_t take = left >= wave ? std::min(p.qchunk, left / wave * wave) : left;
         int best = 1;
         if (take < wave) {
-            const int64_t items = (take + knn_tc_item_rows(p.pair) - 1) / knn_tc_item_rows(p.pair);
-            const int64_t slots = wave / knn_tc_item_rows(p.pair);
+            const int64_t items = (take + item_rows - 1) / item_rows, slots = wave / item_rows;
             double cost = waves1 + rr * (double)take;
             for (int sp = 2; fits(sp); ++sp) {
                 const double c = (double)((items * sp + slots - 1) / slots) / sp * waves1 + rr * (double)take * sp;

@@ -23,8 +23,9 @@
 //               buffer and enter the heaps in common updates of all eight warps.
 // The drain (measured on GB300, 100,000 x 512 BF16, k = 32): 53 ms per search
 // when every admitting column ran the warp through a heap update, 26 ms with
-// buffered updates of each warp at its own time, 14.6 ms with common updates
-// (9.2 ms when nothing is admitted).  Listing the pending candidates by
+// buffered updates of each warp at its own time, 14.6 ms with common updates,
+// 13.4 ms with four children per heap node instead of two (9.2 ms when nothing is
+// admitted), 12.1 ms with the tail wave split.  Listing the pending candidates by
 // warp-wide bitonic merges into sorted lists instead of per-lane heaps took
 // 34 ms (a warp's 32 rows one after the other; two at a time).
 // K blocks run forward on even candidate tiles and backward on odd ones: DRAM
@@ -83,22 +84,24 @@ struct ListState {
     int cnt;    // entries in use
 };
 
-// Rare path of the drain: the row's list is a binary max-heap of kc distances
-// in shared memory (position p at Ld[p * TBM + row]); Ls[p * TBM + row] is the
-// slot of the global index array out[] that holds the entry's candidate, so
-// entries move inside the heap without touching global memory.  Filling appends
-// and sifts up; once full, a candidate below the root replaces it and sifts
-// down (O(log kc) instead of a scan for the new maximum).
+// The row's list is a max-heap of kc distances in shared memory (position p at
+// Ld[p * TBM + row], children 4 p + 1 .. 4 p + 4: a level's four loads are
+// independent, so a replacement in a full heap of 64 takes three dependent steps);
+// Ls[p * TBM + row] is the slot of the global index array out[] that holds the
+// entry's candidate, so entries move inside the heap without touching global
+// memory.  Filling appends and sifts up; once full, a candidate below the root
+// replaces it and sifts down.
 __device__ __noinline__ ListState list_insert(ListState st, float d, int c, float *Ld, uint8_t *Ls, int32_t *out,
                                               int row, int kc) {
     if (st.cnt < kc) {
         int pos = st.cnt;
         while (pos > 0) {
-            const int par = (pos - 1) >> 1;
+            const int par = (pos - 1) >> 2;
             const float pd = Ld[par * TBM + row];
+            const uint8_t ps = Ls[par * TBM + row];
             if (pd >= d) break;
             Ld[pos * TBM + row] = pd;
-            Ls[pos * TBM + row] = Ls[par * TBM + row];
+            Ls[pos * TBM + row] = ps;
             pos = par;
         }
         Ld[pos * TBM + row] = d;
@@ -112,20 +115,24 @@ __device__ __noinline__ ListState list_insert(ListState st, float d, int c, floa
     out[slot] = c;
     int pos = 0;
     for (;;) {
-        const int l = 2 * pos + 1;
+        const int l = 4 * pos + 1;
         if (l >= kc) break;
-        const float dl = Ld[l * TBM + row];
-        const float dr = l + 1 < kc ? Ld[(l + 1) * TBM + row] : -INFINITY;
-        const int ch = dr > dl ? l + 1 : l;
-        const float dc = dr > dl ? dr : dl;
+        float v[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) v[e] = l + e < kc ? Ld[(l + e) * TBM + row] : -INFINITY;
+        const float m01 = fmaxf(v[0], v[1]), m23 = fmaxf(v[2], v[3]);
+        const int b01 = v[1] > v[0] ? 1 : 0, b23 = v[3] > v[2] ? 3 : 2;
+        const float dc = fmaxf(m01, m23);
+        const int ch = l + (m23 > m01 ? b23 : b01);
         if (dc <= d) break;
         Ld[pos * TBM + row] = dc;
         Ls[pos * TBM + row] = Ls[ch * TBM + row];
+        if (pos == 0) st.thr = dc;
         pos = ch;
     }
     Ld[pos * TBM + row] = d;
     Ls[pos * TBM + row] = slot;
-    st.thr = Ld[row];
+    if (pos == 0) st.thr = d;
     return st;
 }
 
