@@ -1292,7 +1292,8 @@ mecuco_status mecuco_curvature_backward(mecuco_t h, const void *X, mecuco_dtype 
     if ((st = begin_call(h, s)) != MECUCO_OK) return st;
     if ((st = ensure_items(h, k)) != MECUCO_OK) return st;
     // per point: forward buffers (incl. U0) + dG, dR, dQ + C and dM (k^3 each)
-    const int64_t per_point = m3_pair_floats(k) + 7LL * k * k + 4LL * k + 2LL * k * k * k;
+    const int64_t k8 = (k + 7) / 8 * 8;  // C's rows
+    const int64_t per_point = m3_pair_floats(k) + 7LL * k * k + 4LL * k + (int64_t)k * k * (k + k8);
     int64_t chunk = h->chunk_points > 0 ? h->chunk_points
                                          : std::max<int64_t>(256, std::min<int64_t>(65536, ((int64_t)2 << 30) /
                                                                                              (per_point * 4)));
@@ -1303,7 +1304,7 @@ mecuco_status mecuco_curvature_backward(mecuco_t h, const void *X, mecuco_dtype 
     t.take<float>((size_t)chunk * k * k);
     t.take<float>((size_t)chunk * k);
     t.take<float>((size_t)chunk * k * k);
-    t.take<float>((size_t)chunk * k * k * k);
+    t.take<float>((size_t)chunk * k * k * k8);
     t.take<float>((size_t)chunk * k * k * k);
     if ((st = ensure(h->ws, h->ws_bytes, t.off, h->ws_cap)) != MECUCO_OK) return st;
     Carver c(h->ws);
@@ -1312,7 +1313,7 @@ mecuco_status mecuco_curvature_backward(mecuco_t h, const void *X, mecuco_dtype 
     float *dG = c.take<float>((size_t)chunk * k * k);
     float *dR = c.take<float>((size_t)chunk * k);
     float *dQ = c.take<float>((size_t)chunk * k * k);
-    float *Cb = c.take<float>((size_t)chunk * k * k * k);
+    float *Cb = c.take<float>((size_t)chunk * k * k * k8);
     float *dM = c.take<float>((size_t)chunk * k * k * k);
     CK(cudaMemsetAsync(dX_out, 0, sizeof(float) * (size_t)N * m, s));
     const bool need_q = var == MECUCO_FAST_HAAR;

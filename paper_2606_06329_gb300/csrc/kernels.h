@@ -329,8 +329,8 @@ cudaError_t launch_tangent_basis(const void *X, mecuco_dtype dt, int64_t N, int6
 // d(sum_i gk_i K_i)/dX for the points of one chunk (idx offset to the chunk),
 // accumulated into dX (row stride ldd) with atomics.  Inputs are sigma/U (the
 // eigenpairs of the rotated Gram) and M/R/Q of the rotated patch Z = U0^T X_c
-// (rot = U0 per point, np x k x k); dG, dR, dQ (np x k x k, k, k x k), C and
-// dMbuf (np x k^3 each) are scratch.
+// (rot = U0 per point, np x k x k); dG, dR, dQ (np x k x k, k, k x k), C
+// (np x k x k rows of k rounded up to 8) and dMbuf (np x k^3) are scratch.
 cudaError_t launch_adjoint(const void *X, mecuco_dtype dt, int64_t N, int64_t m, int64_t ld, const int32_t *idx,
                            int k, int64_t np, int variant, float rank_eps, const float *rot, const float *sigma,
                            const float *U, const float *M, const float *R, const float *Q, const float *gk, float *dG,
