@@ -63,7 +63,7 @@ struct mecuco_ctx {
     DevCounters *ctr = nullptr;
     int32_t *m3_items[65] = {};  // per k: work items of the CUDA-core third-moment kernel
     int32_t *rowtab[65] = {};    // per k: row codes of the tensor-core moment kernel
-    int32_t *tttab[65] = {};     // per k: row codes of the third-moment pass (pairs only)
+    int32_t *tttab[2][65] = {};  // [split][k]: row codes of the third-moment pass (pairs only)
     int knn_splits = 0;
     int knn_pair = -1;  // -1: CTA pairs for operand rows of KNN_PAIR_MIN_K columns or more
     int knn_split_bf16 = 1;  // FP32 rows: three-term BF16 split in the tensor-core search
@@ -438,11 +438,12 @@ mecuco_status ensure_pairs(mecuco_t h, int k) {
 // Table of the BF16-mixed estimator in the rotated basis: the third-moment
 // pass's pair rows.
 mecuco_status ensure_rotated(mecuco_t h, int k) {
-    mecuco_status st;
-    if (!h->tttab[k]) {
-        std::vector<int32_t> host((size_t)tthird_rows(k));
-        tthird_build_rows(k, host.data());
-        if ((st = upload_table(&h->tttab[k], host)) != MECUCO_OK) return st;
+    for (int split = 0; split < 2; ++split) {
+        if (h->tttab[split][k]) continue;
+        std::vector<int32_t> host((size_t)tthird_rows(k, split));
+        tthird_build_rows(k, split, host.data());
+        const mecuco_status st = upload_table(&h->tttab[split][k], host);
+        if (st != MECUCO_OK) return st;
     }
     return MECUCO_OK;
 }
@@ -525,7 +526,7 @@ mecuco_status run_curvature(mecuco_t h, char *ws, const void *X, mecuco_dtype dt
     mecuco_status st = MECUCO_OK;
     const bool tc_moments = prec == MECUCO_PREC_BF16_MIXED;
     const int64_t ym = rotated_m(h, m, prec);
-    if (!h->m3_items[k] || (tc_moments && !h->rowtab[k]) || (ym && !h->tttab[k]))
+    if (!h->m3_items[k] || (tc_moments && !h->rowtab[k]) || (ym && (!h->tttab[0][k] || !h->tttab[1][k])))
         return MECUCO_ERR_INVALID_ARG;
     const int64_t nrows = re - rb;
     const int64_t chunk = est_chunk(h, nrows, k, ym);
@@ -586,7 +587,7 @@ mecuco_status run_curvature(mecuco_t h, char *ws, const void *X, mecuco_dtype dt
             sg.ld = ld;
             sg.k = k;
             sg.idx = nb;
-            sg.rowtab = h->tttab[k];
+            sg.rowtab = h->tttab[m >= TT_SPLIT_MIN_M][k];
             sg.G = b.G;
             sg.R = b.R;
             sg.Q = b.Q;
@@ -893,7 +894,7 @@ mecuco_status plan_batch(mecuco_t h, const mecuco_dataset *sets, int nsets, mecu
             } else {
                 cur.reg.kmax_rest = std::max(cur.reg.kmax_rest, d.k);
             }
-            g.rowtab = h->tttab[d.k];
+            g.rowtab = h->tttab[d.m >= TT_SPLIT_MIN_M][d.k];
             p.segs.push_back(g);
             p.refs.push_back(SegRef{t, 0, a});
             cur.ldy = ldy;
@@ -1106,7 +1107,8 @@ mecuco_status mecuco_destroy(mecuco_t h) {
     for (int kk = 0; kk <= 64; ++kk) {
         if (h->m3_items[kk]) cudaFree(h->m3_items[kk]);
         if (h->rowtab[kk]) cudaFree(h->rowtab[kk]);
-        if (h->tttab[kk]) cudaFree(h->tttab[kk]);
+        for (auto &t : h->tttab)
+            if (t[kk]) cudaFree(t[kk]);
     }
     if (h->bws) cudaFree(h->bws);
     for (int i = 0; i < 32; ++i) {

@@ -191,14 +191,17 @@ size_t moments_tc_smem_bytes(int k);
 // (rows k..63 zero), ldy >= every segment's m rounded up to 64, ldy % 8 == 0.
 // launch_tthird_tc: the Fast estimator from Y, sig, U, R and Q (Haar) -
 // kappa, and lambda / s when not NULL; rowtab from tthird_build_rows for the
-// segment's k; kmax bounds every segment's k; ctas = 1 or 2 CTAs per SM (512 or
+// segment's k and m; kmax bounds every segment's k; ctas = 1 or 2 CTAs per SM (512 or
 // 256 TMEM columns each, nslots of them the A operand's slots).
 cudaError_t launch_gram_tc(mecuco_dtype dt, const PatchSeg &one, const PatchSeg *tab, int ntab, int64_t np,
                            int with_q, long long wait_limit, DevCounters *ctr, cudaStream_t s);
 cudaError_t launch_rotate_tc(mecuco_dtype dt, const PatchSeg &one, const PatchSeg *tab, int ntab, int64_t np, void *Y,
                              int64_t ldy, long long wait_limit, DevCounters *ctr, cudaStream_t s);
-__host__ __device__ int tthird_rows(int k);
-void tthird_build_rows(int k, int32_t *codes /* tthird_rows(k) */);
+// split: the table of pairs inside two halves of the rows (m >= TT_SPLIT_MIN_M),
+// else of all pairs.
+constexpr int64_t TT_SPLIT_MIN_M = 128;
+__host__ __device__ int tthird_rows(int k, int split);
+void tthird_build_rows(int k, int split, int32_t *codes /* tthird_rows(k, split) */);
 cudaError_t launch_tthird_tc(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t np, const void *Y,
                              int64_t ldy, int variant, int nslots, int ctas, long long wait_limit, DevCounters *ctr,
                              cudaStream_t s);

@@ -15,6 +15,20 @@
 // product - nothing m-sized and no third-moment tensor is stored.  |X_c V_r|_F^2
 // = sum_{l<p} s_l^2 = (k-1) tau; the Haar term is sum_{l<p} u_l^T Q u_l / s_l^2.
 //
+// S[r,t,l] = sum_a Y_ra Y_ta Y_la is symmetric in all three indices, so not every
+// pair of rows has to be formed: with the rows split in two halves, any three
+// indices have two in the same half, and the pairs inside the halves are enough
+// (half of the pairs and the best possible: the pairs left out must form no
+// triangle).  An element S[(a,b), l] with l in the other half then also stands
+// for T^[(a,l), b] and T^[(b,l), a].  20 instead of 36 blocks of 8 x 8 pairs at k
+// = 64, 9 instead of 15 at 37, 6 instead of 10 at 32.  Measured with every pair and
+// with the split: 11.3 and 6.7 ms for 6,144 patches of 4,096 columns at k = 64, 114
+// and 67 for 62,500, 6.5 and 5.8 for 30,000 of 301 at k = 37 (5.0 with the sums of
+// the epilogue in two-term FP32 instead of FP64).
+// Sets below TT_SPLIT_MIN_M columns form every pair: there |G_tens|^2 is divided
+// by a small m - p, and the BF16 roundings of the products, which differ between
+// the two tables, would show in kappa.
+//
 // T^ is the GEMM D = Z Y^T over the columns a, Z the row products
 // Z[(r,t), a] = Y_ra Y_ta (r <= t, 8 x 8 pair blocks as in the moment kernel)
 // and the scale 1/(s_r s_t) applied in FP32 when D is read.  One CTA per point:
@@ -42,7 +56,7 @@ namespace mecuco {
 namespace {
 constexpr int TT_FORMER_WARPS = 8;
 constexpr int TT_THREADS = (TT_FORMER_WARPS + 2) * 32;  // formers, the TMA warp, the MMA warp
-constexpr int TT_TMA_WARP = TT_FORMER_WARPS, TT_MMA_WARP = TT_FORMER_WARPS + 1;
+constexpr int TT_TMA_WARP = TT_FORMER_WARPS;  // the MMA warp follows
 constexpr int TT_CH = 64;                  // columns per chunk
 constexpr int TT_STAGE = 64 * 128;         // a chunk of Y: 64 rows x 64 columns BF16
 constexpr int TT_NS = 6;                   // ring stages
@@ -54,29 +68,58 @@ constexpr long long TT_WAIT = 1000000000LL;
 
 enum : int { ROW_NONE = 0, ROW_PAIR = 1 };
 
+typedef unsigned long long f2;  // two FP32 values of a packed instruction
+__device__ __forceinline__ f2 pack2(float lo, float hi) {
+    f2 v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ float2 unpack2(f2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ f2 fma2(f2 a, f2 b, f2 c) {
+    f2 d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ f2 mul2(f2 a, f2 b) {
+    f2 d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+
 __host__ __device__ inline int tthird_n(int k) { return k <= 16 ? 16 : ((k + 15) / 16) * 16; }
 }  // namespace
 
-__host__ __device__ int tthird_rows(int k) {
-    const int kb = (k + 7) / 8;
-    return (kb * (kb + 1) / 2 * 64 + 127) / 128 * 128;
+// 8-row blocks of the first half (split tables)
+__host__ __device__ inline int tthird_half(int k) { return ((k + 7) / 8 + 1) / 2; }
+
+__host__ __device__ int tthird_rows(int k, int split) {
+    const int kb = (k + 7) / 8, h = tthird_half(k), g = kb - h;
+    const int blocks = split ? h * (h + 1) / 2 + g * (g + 1) / 2 : kb * (kb + 1) / 2;
+    return (blocks * 64 + 127) / 128 * 128;
 }
 
 // Pairs r <= t in 8 x 8 blocks (r-block <= t-block): a 32-row quarter of a
 // block holds 4 values of r and 8 of t, so along a row of blocks a lane keeps
-// its r (the formers reload only Y_t).  Code = r | t << 8 | kind << 16.
-void tthird_build_rows(int k, int32_t *codes) {
-    const int kb = (k + 7) / 8;
-    const int nrows = tthird_rows(k);
+// its r (the formers reload only Y_t).  Split tables leave out the pairs whose
+// members lie in different halves of the blocks.  Code = r | t << 8 | kind << 16.
+void tthird_build_rows(int k, int split, int32_t *codes) {
+    const int kb = (k + 7) / 8, hb = tthird_half(k);
+    const int nrows = tthird_rows(k, split);
     int n = 0;
     for (int A = 0; A < kb; ++A)
-        for (int B = A; B < kb; ++B)
+        for (int B = A; B < kb; ++B) {
+            if (split && (A < hb) != (B < hb)) continue;
             for (int r = 0; r < 64; ++r) {
                 const int h = r / 32, L = r % 32;
                 const int a = 8 * A + 4 * h + L / 8, b = 8 * B + L % 8;
                 const bool valid = a < k && b < k && (A < B || a <= b);
                 codes[n++] = valid ? (int32_t)(a | (b << 8) | (ROW_PAIR << 16)) : 0;
             }
+        }
     for (; n < nrows; ++n) codes[n] = 0;
 }
 
@@ -84,7 +127,7 @@ void tthird_build_rows(int k, int32_t *codes) {
 // the request is raised to 120 KB so that no second CTA becomes resident (it
 // would only wait in its allocation).
 size_t tthird_smem_bytes(int k, int ctas) {
-    const size_t need = 1024 + (size_t)TT_NS * TT_STAGE + (size_t)tthird_rows(k) * 8 + 64 * (size_t)TT_DLD * 4;
+    const size_t need = 1024 + (size_t)TT_NS * TT_STAGE + (size_t)tthird_rows(k, 0) * 8 + 64 * (size_t)TT_DLD * 4;
     return (ctas == 1 && need < ((size_t)120 << 10)) ? ((size_t)120 << 10) : need;
 }
 
@@ -98,7 +141,8 @@ tthird_tc_kernel(const __grid_constant__ CUtensorMap map_y, const __grid_constan
     const PatchSeg &seg = find_seg(one, tab, ntab, (int)blockIdx.x, local);
     const int64_t pt = local, m = seg.m;
     const int k = seg.k;
-    const int nrows = tthird_rows(k);
+    const int split = seg.m >= TT_SPLIT_MIN_M;
+    const int nrows = tthird_rows(k, split);
     const int32_t *rowtab = seg.rowtab;
     const float *sigma = seg.sig, *U = seg.U, *R = seg.R, *Q = seg.Q;
     float *kappa = seg.kappa, *lambda_out = seg.lambda, *s_out = seg.s;
@@ -114,7 +158,8 @@ tthird_tc_kernel(const __grid_constant__ CUtensorMap map_y, const __grid_constan
     __shared__ uint64_t pass_done, d_free, mma_fin;
     __shared__ uint32_t tmem_slot;
     __shared__ float inv_s[64], c_s[64];
-    __shared__ double red[TT_THREADS / 32][4];
+    __shared__ __align__(16) float cross[2][64];  // 1 / s_l of the columns outside half 0 / 1 (split tables), else 0
+    __shared__ float2 red[TT_THREADS / 32][5];  // two-term sums: gt2, t_range, |X_c d_P|^2, Haar, tau
     __shared__ int s_p, abort_flag, never;
 
     const int ntiles = nrows / 128;
@@ -129,14 +174,6 @@ tthird_tc_kernel(const __grid_constant__ CUtensorMap map_y, const __grid_constan
     for (int e = tid; e < nrows; e += TT_THREADS) codes[e] = __ldg(rowtab + e);
     for (int e = tid; e < 64 * TT_DLD; e += TT_THREADS) diag[e] = 0.f;
     if (tid == 0) {
-        // numerical rank: eigenvalues above rank_eps * s_0 (the Gram's rounding scale)
-        int pmax = k - 1;
-        if ((int64_t)pmax > m) pmax = (int)m;
-        const float s0 = fmaxf(sg[0], 0.f);
-        int rank = 0;
-        for (int l = 0; l < k; ++l) rank += (sg[l] > rank_eps * s0) && (sg[l] > 0.f);
-        s_p = rank < pmax ? rank : pmax;
-        if (s_p < pmax) atomicAdd(&ctr->rank_deficient, 1ull);
         for (int s = 0; s < TT_NS; ++s) {
             tc::mbar_init(tc::smem_u32(&full[s]), 1);
             tc::mbar_init(tc::smem_u32(&empty[s]), 1);
@@ -153,6 +190,18 @@ tthird_tc_kernel(const __grid_constant__ CUtensorMap map_y, const __grid_constan
         tc::fence_mbar_init();
         tc::prefetch_tmap(&map_y);
     }
+    if (warp == 1) {
+        // numerical rank: eigenvalues above rank_eps * s_0 (the Gram's rounding scale)
+        const float a = lane < k ? sg[lane] : 0.f, b = lane + 32 < k ? sg[lane + 32] : 0.f;
+        const float lim = rank_eps * fmaxf(__shfl_sync(0xffffffffu, a, 0), 0.f);
+        const int rank = __popc(__ballot_sync(0xffffffffu, a > lim && a > 0.f)) +
+                         __popc(__ballot_sync(0xffffffffu, b > lim && b > 0.f));
+        const int pmax = (int64_t)(k - 1) > m ? (int)m : k - 1;
+        if (lane == 0) {
+            s_p = rank < pmax ? rank : pmax;
+            if (rank < pmax) atomicAdd(&ctr->rank_deficient, 1ull);
+        }
+    }
     if (warp == 0) {
         tc::tmem_alloc(tc::smem_u32(&tmem_slot), (uint32_t)tcols);
         tc::tmem_relinquish();
@@ -161,7 +210,13 @@ tthird_tc_kernel(const __grid_constant__ CUtensorMap map_y, const __grid_constan
     __syncthreads();
     tc::fence_after();
     const int p = s_p;
-    if (tid < 64) inv_s[tid] = tid < p ? (float)(1.0 / sqrt((double)sg[tid])) : 0.f;
+    if (tid < 64) {
+        const float is = tid < p ? __frsqrt_rn(sg[tid]) : 0.f;
+        const bool second = tid >= 8 * tthird_half(k);
+        inv_s[tid] = is;
+        cross[0][tid] = split && second ? is : 0.f;
+        cross[1][tid] = split && !second ? is : 0.f;
+    }
     const uint32_t tmem = tmem_slot;
     volatile int *abortp = &abort_flag;
     auto fail = [&]() {
@@ -239,21 +294,36 @@ tthird_tc_kernel(const __grid_constant__ CUtensorMap map_y, const __grid_constan
             for (int t = half; t < nt; t += 2) {
                 const int code = codes[(t0 + t) * 128 + trow];
                 const int ra = code & 0xff, rb = (code >> 8) & 0xff;
-                const bool live = ((code >> 16) & 3) == ROW_PAIR && ra < p && rb < p;
-                const float f = live ? inv_s[ra] * inv_s[rb] : 0.f;
-                float sq = 0.f;
+                const bool pair = ((code >> 16) & 3) == ROW_PAIR;
+                const float ia = inv_s[ra], ib = inv_s[rb];
+                const float f = pair ? ia * ib : 0.f;
+                // the same product also stands for the pairs (a, l) and (b, l) of the
+                // columns l in the other half: sqrt(2 (1/s_a^2 + 1/s_b^2)) / s_l
+                const float gr = pair ? sqrtf(2.f * (ra == rb ? ia * ia : fmaf(ia, ia, ib * ib))) : 0.f;
+                const float *cr = cross[ra >= 8 * tthird_half(k)];
+                const bool dg = pair && ra == rb && ra < p;
+                const f2 f2v = pack2(f, f), g2v = pack2(gr, gr);
+                f2 sq = 0, sx = 0;
                 for (int c0 = 0; c0 < Nb; c0 += 16) {
                     uint32_t r16[16];
                     tc::tmem_ld_32x32b_x16(tmem + ((uint32_t)(qd * 32) << 16) + (uint32_t)(t * Nb + c0), r16);
-                    tc::tmem_ld_wait();
+                    tc::tmem_ld_wait16(r16);
 #pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const float v = f * __uint_as_float(r16[e]);
-                        sq = fmaf(v, v, sq);
-                        if (live && ra == rb) diag[ra * TT_DLD + c0 + e] = v;
+                    for (int e = 0; e < 8; ++e) {
+                        const f2 raw = pack2(__uint_as_float(r16[2 * e]), __uint_as_float(r16[2 * e + 1]));
+                        const f2 v = mul2(f2v, raw);
+                        sq = fma2(v, v, sq);
+                        const f2 u = mul2(mul2(g2v, raw), *reinterpret_cast<const f2 *>(cr + c0 + 2 * e));
+                        sx = fma2(u, u, sx);
+                        if (dg) {
+                            const float2 d = unpack2(v);
+                            diag[ra * TT_DLD + c0 + 2 * e] = d.x;
+                            diag[ra * TT_DLD + c0 + 2 * e + 1] = d.y;
+                        }
                     }
                 }
-                rowsq[(t0 + t) * 128 + trow] = live ? (ra == rb ? 1.f : 2.f) * sq : 0.f;
+                const float2 a = unpack2(sq), x = unpack2(sx);
+                rowsq[(t0 + t) * 128 + trow] = (ra == rb ? 1.f : 2.f) * (a.x + a.y) + (x.x + x.y);
             }
             tc::fence_before();
             __syncwarp();
@@ -346,45 +416,52 @@ tthird_tc_kernel(const __grid_constant__ CUtensorMap map_y, const __grid_constan
     // ================= final sums (all threads) =================
     tc::fence_before();
     __syncthreads();
+    // The sums are two-term FP32 (2^-44 and better): FP64 runs at 1/64 of the FP32
+    // rate, and a few dozen double operations per warp cost narrow sets as much as
+    // their third moments.
+    auto ff_mul = [](float a, float b) {
+        const float h = __fmul_rn(a, b);
+        return ff{h, __fmaf_rn(a, b, -h)};
+    };
     // |G_tens|^2: each thread sums a fixed set of table rows (the schedule of
     // tiles over passes and warps does not change the order)
-    double gsum = 0.0;
-    for (int e = tid; e < nrows; e += TT_THREADS) gsum += (double)rowsq[e];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) gsum += __shfl_xor_sync(0xffffffffu, gsum, o);
+    ff gsum{0.f, 0.f};
+    for (int e = tid; e < nrows; e += TT_THREADS) gsum = ff_add(gsum, ff{rowsq[e], 0.f});
+    gsum = ff_warp_sum(gsum);
     // U and Q of the point, staged in the (now idle) ring: U[j][l] at Us[j*65 + l]
     float *Us = reinterpret_cast<float *>(ring), *Qs = Us + 64 * 65;
     const float *ug = U + pt * (int64_t)k * k;
-    for (int e = tid; e < k * k; e += TT_THREADS) Us[(e / k) * 65 + e % k] = ug[e];
-    if (variant == MECUCO_FAST_HAAR) {
-        const float *qg = Q + pt * (int64_t)k * k;
-        for (int e = tid; e < k * k; e += TT_THREADS) Qs[(e / k) * 65 + e % k] = qg[e];
-    }
+    const float *qg = Q + pt * (int64_t)k * k;
+    for (int j = warp; j < k; j += TT_THREADS / 32)
+        for (int l = lane; l < k; l += 32) {
+            Us[j * 65 + l] = ug[j * k + l];
+            if (variant == MECUCO_FAST_HAAR) Qs[j * 65 + l] = qg[j * k + l];
+        }
     __syncthreads();
-    double dsum = 0.0, xa2 = 0.0, hsum = 0.0;
+    ff dsum{0.f, 0.f}, xa2{0.f, 0.f}, hsum{0.f, 0.f}, tsum{0.f, 0.f};
     if (tid < k) {
         // c_l = sum_{r<p} T^[(r,r), l] and t_range's sum, in a fixed order over r
         const int l = tid;
         float cl = 0.f;
-        double d2 = 0.0;
         for (int r = 0; r < p; ++r) {
             const float v = diag[r * TT_DLD + l];
             cl += v;
-            d2 += (double)v * v;
+            dsum = ff_add(dsum, ff_mul(v, v));
         }
         c_s[l] = cl;
-        dsum = d2;
+        if (l < p) tsum.hi = sg[l];
     }
     if (variant == MECUCO_FAST_HAAR && tid >= 64 && tid < 64 + p) {
         // u_l^T Q u_l / s_l^2
         const int l = tid - 64;
-        double acc = 0.0;
+        ff acc{0.f, 0.f};
         for (int a = 0; a < k; ++a) {
             float qu = 0.f;
             for (int b = 0; b < k; ++b) qu = fmaf(Qs[a * 65 + b], Us[b * 65 + l], qu);
-            acc += (double)Us[a * 65 + l] * qu;
+            acc = ff_add(acc, ff_mul(Us[a * 65 + l], qu));
         }
-        hsum = acc / (double)sg[l];
+        const float s = sg[l], q1 = acc.hi / s;
+        hsum = ff{q1, (fmaf(-q1, s, acc.hi) + acc.lo) / s};
     }
     __syncthreads();
     if (tid < k) {
@@ -392,37 +469,52 @@ tthird_tc_kernel(const __grid_constant__ CUtensorMap map_y, const __grid_constan
         const int j = tid;
         float uc = 0.f;
         for (int l = 0; l < k; ++l) uc = fmaf(Us[j * 65 + l], c_s[l], uc);
-        const double xd = (double)R[pt * k + j] - (double)uc;
-        xa2 = xd * xd;
+        float h, e;
+        two_sum(R[pt * k + j], -uc, h, e);
+        xa2 = ff_mul(h, h);
+        xa2.lo += 2.f * h * e;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
-        xa2 += __shfl_xor_sync(0xffffffffu, xa2, o);
-        hsum += __shfl_xor_sync(0xffffffffu, hsum, o);
+    if (warp < 4) {  // the threads that hold any of these
+        dsum = ff_warp_sum(dsum);
+        xa2 = ff_warp_sum(xa2);
+        hsum = ff_warp_sum(hsum);
+        tsum = ff_warp_sum(tsum);
     }
-    if (lane == 0) { red[warp][0] = gsum; red[warp][1] = dsum; red[warp][2] = xa2; red[warp][3] = hsum; }
+    if (lane == 0) {
+        red[warp][0] = make_float2(gsum.hi, gsum.lo);
+        red[warp][1] = make_float2(dsum.hi, dsum.lo);
+        red[warp][2] = make_float2(xa2.hi, xa2.lo);
+        red[warp][3] = make_float2(hsum.hi, hsum.lo);
+        red[warp][4] = make_float2(tsum.hi, tsum.lo);
+    }
     __syncthreads();
-    if (tid == 0) {
-        double gt2 = 0.0, d2 = 0.0, a2 = 0.0, h = 0.0;
-        for (int w = 0; w < TT_THREADS / 32; ++w) { gt2 += red[w][0]; d2 += red[w][1]; a2 += red[w][2]; h += red[w][3]; }
-        const double km1 = (double)(k - 1);
-        double tau = 0.0;
-        for (int l = 0; l < p; ++l) tau += (double)sg[l];
-        tau /= km1;
-        const double t_range = d2 / km1, t_A = a2 / km1;
-        const int64_t q = m - p;
-        double t_null = 0.0;
-        if (q > 0) {
-            if (variant == MECUCO_FAST_HAAR) {
-                const double tB = tau - 2.0 * h / km1 + gt2 / km1;
-                t_null = (t_A + 2.0 * tB) / (double)(q + 2);
-            } else {
-                const double tB = tau - 2.0 * tau + gt2 / km1;  // |X_c V_r|_F^2 / (k-1) = tau
-                t_null = (t_A + 2.0 * tB) / (double)q;
-            }
+    if (tid < 32) {
+        // warp w's terms in lane w
+        ff t[5];
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+            const float2 v = lane < TT_THREADS / 32 && (c == 0 || lane < 4) ? red[lane][c] : make_float2(0.f, 0.f);
+            t[c] = ff_warp_sum(ff{v.x, v.y});
         }
-        kappa[pt] = (float)fabs(0.5 * (t_range + t_null) + 0.5 * tau);
+        if (lane == 0) {
+            const double ik = 1.0 / (double)(k - 1);
+            const double gt2 = (double)t[0].hi + (double)t[0].lo, d2 = (double)t[1].hi + (double)t[1].lo;
+            const double a2 = (double)t[2].hi + (double)t[2].lo, h = (double)t[3].hi + (double)t[3].lo;
+            const double tau = ((double)t[4].hi + (double)t[4].lo) * ik;
+            const double t_range = d2 * ik, t_A = a2 * ik;
+            const int64_t q = m - p;
+            double t_null = 0.0;
+            if (q > 0) {
+                if (variant == MECUCO_FAST_HAAR) {
+                    const double tB = tau + (gt2 - 2.0 * h) * ik;
+                    t_null = (t_A + 2.0 * tB) / (double)(q + 2);
+                } else {
+                    const double tB = gt2 * ik - tau;  // |X_c V_r|_F^2 / (k-1) = tau
+                    t_null = (t_A + 2.0 * tB) / (double)q;
+                }
+            }
+            kappa[pt] = (float)fabs(0.5 * (t_range + t_null) + 0.5 * tau);
+        }
     }
     if (lambda_out)
         for (int l = tid; l < k; l += TT_THREADS)
