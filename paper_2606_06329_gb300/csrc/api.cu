@@ -465,12 +465,12 @@ struct EstBufs {
     float *rQ, *rB, *rsig, *rV;  // randomised SVD: range basis, projected Gram and its eigenpairs
 };
 // ym > 0: the rotated-basis estimator (BF16-mixed form) with Y for ambient
-// dimension ym in place of the third moments M.
-void est_scratch(Carver &c, int64_t chunk, int k, EstBufs *b, int rsvd_cols = 0, int64_t ym = 0) {
+// dimension ym; with_m: the third moments M are stored (randomised SVD, gradient).
+void est_scratch(Carver &c, int64_t chunk, int k, EstBufs *b, int rsvd_cols, int64_t ym, bool with_m) {
     b->G = c.take<float>((size_t)chunk * k * k);
     b->R = c.take<float>((size_t)chunk * k);
     b->Q = c.take<float>((size_t)chunk * k * k);
-    b->M = ym ? nullptr : c.take<float>((size_t)chunk * m3_pair_floats(k));
+    b->M = with_m ? c.take<float>((size_t)chunk * m3_pair_floats(k)) : nullptr;
     b->Y = ym ? c.take<uint16_t>((size_t)chunk * 64 * rot_ld(ym)) : nullptr;
     b->sig = c.take<float>((size_t)chunk * k);
     b->U = c.take<float>((size_t)chunk * k * k);
@@ -486,7 +486,8 @@ void est_scratch(Carver &c, int64_t chunk, int k, EstBufs *b, int rsvd_cols = 0,
 // batched call) - larger chunks leave smaller partial last waves: at k = 64,
 // 14k-point chunks took the per-chunk kernels 2.6% less time than 3.6k ones.
 int64_t est_chunk(mecuco_t h, int64_t nrows, int k, int64_t ym = 0) {
-    const int64_t per_point = (ym ? 32 * rot_ld(ym) : m3_pair_floats(k)) + 4LL * k * k + 3LL * k;
+    const int64_t per_point =
+        (ym ? 32 * rot_ld(ym) : h->rsvd.cols ? m3_pair_floats(k) : 0) + 4LL * k * k + 3LL * k;
     int64_t chunk = h->chunk_points;
     if (chunk <= 0) {
         const size_t budget = ((size_t)8 << 30) / (size_t)std::max(1, h->chunk_share);
@@ -512,7 +513,7 @@ size_t curvature_bytes(mecuco_t h, const void *X, mecuco_dtype dt, int64_t N, in
     size_t need = idx_given ? 0 : knn_bytes(h, X, dt, N, m, ld, nrows, k, prec, idx_bytes);
     Carver c(nullptr, idx_bytes);
     EstBufs b;
-    est_scratch(c, chunk, k, &b, h->rsvd.cols, ym);
+    est_scratch(c, chunk, k, &b, h->rsvd.cols, ym, h->rsvd.cols > 0);
     return std::max(need, c.off);
 }
 
@@ -540,7 +541,7 @@ mecuco_status run_curvature(mecuco_t h, char *ws, const void *X, mecuco_dtype dt
     }
     Carver c(ws, idx_bytes);
     EstBufs b;
-    est_scratch(c, chunk, k, &b, h->rsvd.cols, ym);
+    est_scratch(c, chunk, k, &b, h->rsvd.cols, ym, h->rsvd.cols > 0);
     const int fp64 = h->jacobi_fp64 >= 0 ? h->jacobi_fp64 : (prec == MECUCO_PREC_BF16_MIXED ? 1 : 0);
     const float *Qarg = var == MECUCO_FAST_HAAR ? b.Q : nullptr;
     for (int64_t p0 = 0; p0 < nrows; p0 += chunk) {
@@ -619,16 +620,15 @@ mecuco_status run_curvature(mecuco_t h, char *ws, const void *X, mecuco_dtype dt
             LAUNCH(h, MECUCO_STAGE_GRAM, s,
                    launch_patch_gram(X, dt, N, m, ld, nb, k, 0, np, b.U0, b.G, b.R, var == MECUCO_FAST_HAAR ? b.Q : nullptr,
                                      h->ctr, s));
-            LAUNCH(h, MECUCO_STAGE_MOMENTS, s,
-                   launch_patch_m3(X, dt, N, m, ld, nb, k, 0, np, b.U0, b.M, h->m3_items[k], h->ctr, s));
             LAUNCH(h, MECUCO_STAGE_JACOBI, s,
                    launch_jacobi(b.G, k, np, fp64, h->jacobi_max_sweeps, b.sig, b.U, h->ctr, s,
                                  kJacobiPreTight, h->jacobi_warp));
             if (fp64 == 1 || fp64 == 3) ++h->launches;
             LAUNCH(h, MECUCO_STAGE_ESTIMATOR, s,
-                   launch_estimator(b.sig, b.U, b.M, b.R, Qarg, k, m, np, (int)var, rank_eps_rotated(k, m),
-                                    kappa_out + p0, lambda_out ? lambda_out + p0 * k : nullptr,
-                                    s_out ? s_out + p0 * k : nullptr, h->ctr, s));
+                   launch_patch_kappa(X, dt, N, m, ld, nb, k, np, b.U0, b.sig, b.U, b.R, Qarg, (int)var,
+                                      rank_eps_rotated(k, m), h->m3_items[k], kappa_out + p0,
+                                      lambda_out ? lambda_out + p0 * k : nullptr, s_out ? s_out + p0 * k : nullptr,
+                                      h->ctr, s));
             if (U_out) LAUNCH(h, MECUCO_STAGE_JACOBI, s,
                               launch_compose_rotation(b.U0, b.U, k, np, U_out + p0 * (int64_t)k * k, s));
         }
@@ -851,7 +851,7 @@ mecuco_status plan_batch(mecuco_t h, const mecuco_dataset *sets, int nsets, mecu
         if (cur.np == 0) return;
         Carver e(base, after_idx);
         EstBufs b;
-        est_scratch(e, cur.np, cur.kmax, &b, 0, cur.ldy);
+        est_scratch(e, cur.np, cur.kmax, &b, 0, cur.ldy, false);
         est_end = std::max(est_end, e.off);
         cur.Y = b.Y;
         for (int i = cur.seg0; i < cur.seg0 + cur.nseg; ++i) {
@@ -1302,7 +1302,7 @@ mecuco_status mecuco_curvature_backward(mecuco_t h, const void *X, mecuco_dtype 
     chunk = std::min(chunk, N);
     Carver t(nullptr);
     EstBufs b;
-    est_scratch(t, chunk, k, &b);
+    est_scratch(t, chunk, k, &b, 0, 0, true);
     t.take<float>((size_t)chunk * k * k);
     t.take<float>((size_t)chunk * k);
     t.take<float>((size_t)chunk * k * k);
@@ -1310,7 +1310,7 @@ mecuco_status mecuco_curvature_backward(mecuco_t h, const void *X, mecuco_dtype 
     t.take<float>((size_t)chunk * k * k * k);
     if ((st = ensure(h->ws, h->ws_bytes, t.off, h->ws_cap)) != MECUCO_OK) return st;
     Carver c(h->ws);
-    est_scratch(c, chunk, k, &b);
+    est_scratch(c, chunk, k, &b, 0, 0, true);
     float *U0 = b.U0;
     float *dG = c.take<float>((size_t)chunk * k * k);
     float *dR = c.take<float>((size_t)chunk * k);

@@ -160,6 +160,15 @@ cudaError_t launch_patch_m3(const void *X, mecuco_dtype dt, int64_t N, int64_t m
                             const int32_t *idx, int k, int64_t p0, int64_t np, const float *rot,
                             float *M, const int32_t *items, DevCounters *ctr, cudaStream_t s);
 
+// Step 4 from the third moments of Y = V^T Z, Z = rot^T X_c, with sigma/V the
+// eigenpairs of the Gram of Z, R and Q (Haar) those of Z: kappa (np) and, when not
+// NULL, lambda_out (np x k) and s_out (np x k).  M is not formed.
+cudaError_t launch_patch_kappa(const void *X, mecuco_dtype dt, int64_t N, int64_t m, int64_t ld,
+                               const int32_t *idx, int k, int64_t np, const float *rot, const float *sigma,
+                               const float *V, const float *R, const float *Q, int variant, float rank_eps,
+                               const int32_t *items, float *kappa, float *lambda_out, float *s_out,
+                               DevCounters *ctr, cudaStream_t s);
+
 __host__ __device__ inline int pair_index(int a, int b, int k) { return a * k - (a * (a - 1)) / 2 + (b - a); }
 inline int64_t m3_pair_floats(int k) { return (int64_t)k * (k + 1) / 2 * k; }
 #ifdef __CUDACC__

@@ -48,6 +48,7 @@
 #include <algorithm>
 
 #include "common.cuh"
+#include "fast_terms.cuh"
 #include "kernels.h"
 #include "tc_ptx.cuh"
 
@@ -159,7 +160,7 @@ tthird_tc_kernel(const __grid_constant__ CUtensorMap map_y, const __grid_constan
     __shared__ uint32_t tmem_slot;
     __shared__ float inv_s[64], c_s[64];
     __shared__ __align__(16) float cross[2][64];  // 1 / s_l of the columns outside half 0 / 1 (split tables), else 0
-    __shared__ float2 red[TT_THREADS / 32][5];  // two-term sums: gt2, t_range, |X_c d_P|^2, Haar, tau
+    __shared__ float2 red[TT_THREADS / 32][5];
     __shared__ int s_p, abort_flag, never;
 
     const int ntiles = nrows / 128;
@@ -191,16 +192,8 @@ tthird_tc_kernel(const __grid_constant__ CUtensorMap map_y, const __grid_constan
         tc::prefetch_tmap(&map_y);
     }
     if (warp == 1) {
-        // numerical rank: eigenvalues above rank_eps * s_0 (the Gram's rounding scale)
-        const float a = lane < k ? sg[lane] : 0.f, b = lane + 32 < k ? sg[lane + 32] : 0.f;
-        const float lim = rank_eps * fmaxf(__shfl_sync(0xffffffffu, a, 0), 0.f);
-        const int rank = __popc(__ballot_sync(0xffffffffu, a > lim && a > 0.f)) +
-                         __popc(__ballot_sync(0xffffffffu, b > lim && b > 0.f));
-        const int pmax = (int64_t)(k - 1) > m ? (int)m : k - 1;
-        if (lane == 0) {
-            s_p = rank < pmax ? rank : pmax;
-            if (rank < pmax) atomicAdd(&ctr->rank_deficient, 1ull);
-        }
+        const int rank = fast_rank(sg, k, m, rank_eps, ctr);
+        if (lane == 0) s_p = rank;
     }
     if (warp == 0) {
         tc::tmem_alloc(tc::smem_u32(&tmem_slot), (uint32_t)tcols);
@@ -416,18 +409,10 @@ tthird_tc_kernel(const __grid_constant__ CUtensorMap map_y, const __grid_constan
     // ================= final sums (all threads) =================
     tc::fence_before();
     __syncthreads();
-    // The sums are two-term FP32 (2^-44 and better): FP64 runs at 1/64 of the FP32
-    // rate, and a few dozen double operations per warp cost narrow sets as much as
-    // their third moments.
-    auto ff_mul = [](float a, float b) {
-        const float h = __fmul_rn(a, b);
-        return ff{h, __fmaf_rn(a, b, -h)};
-    };
     // |G_tens|^2: each thread sums a fixed set of table rows (the schedule of
     // tiles over passes and warps does not change the order)
     ff gsum{0.f, 0.f};
-    for (int e = tid; e < nrows; e += TT_THREADS) gsum = ff_add(gsum, ff{rowsq[e], 0.f});
-    gsum = ff_warp_sum(gsum);
+    for (int e = tid; e < nrows; e += TT_THREADS) gsum = sum_add(gsum, ff{rowsq[e], 0.f});
     // U and Q of the point, staged in the (now idle) ring: U[j][l] at Us[j*65 + l]
     float *Us = reinterpret_cast<float *>(ring), *Qs = Us + 64 * 65;
     const float *ug = U + pt * (int64_t)k * k;
@@ -438,84 +423,7 @@ tthird_tc_kernel(const __grid_constant__ CUtensorMap map_y, const __grid_constan
             if (variant == MECUCO_FAST_HAAR) Qs[j * 65 + l] = qg[j * k + l];
         }
     __syncthreads();
-    ff dsum{0.f, 0.f}, xa2{0.f, 0.f}, hsum{0.f, 0.f}, tsum{0.f, 0.f};
-    if (tid < k) {
-        // c_l = sum_{r<p} T^[(r,r), l] and t_range's sum, in a fixed order over r
-        const int l = tid;
-        float cl = 0.f;
-        for (int r = 0; r < p; ++r) {
-            const float v = diag[r * TT_DLD + l];
-            cl += v;
-            dsum = ff_add(dsum, ff_mul(v, v));
-        }
-        c_s[l] = cl;
-        if (l < p) tsum.hi = sg[l];
-    }
-    if (variant == MECUCO_FAST_HAAR && tid >= 64 && tid < 64 + p) {
-        // u_l^T Q u_l / s_l^2
-        const int l = tid - 64;
-        ff acc{0.f, 0.f};
-        for (int a = 0; a < k; ++a) {
-            float qu = 0.f;
-            for (int b = 0; b < k; ++b) qu = fmaf(Qs[a * 65 + b], Us[b * 65 + l], qu);
-            acc = ff_add(acc, ff_mul(Us[a * 65 + l], qu));
-        }
-        const float s = sg[l], q1 = acc.hi / s;
-        hsum = ff{q1, (fmaf(-q1, s, acc.hi) + acc.lo) / s};
-    }
-    __syncthreads();
-    if (tid < k) {
-        // X_c d_P = R - U c
-        const int j = tid;
-        float uc = 0.f;
-        for (int l = 0; l < k; ++l) uc = fmaf(Us[j * 65 + l], c_s[l], uc);
-        float h, e;
-        two_sum(R[pt * k + j], -uc, h, e);
-        xa2 = ff_mul(h, h);
-        xa2.lo += 2.f * h * e;
-    }
-    if (warp < 4) {  // the threads that hold any of these
-        dsum = ff_warp_sum(dsum);
-        xa2 = ff_warp_sum(xa2);
-        hsum = ff_warp_sum(hsum);
-        tsum = ff_warp_sum(tsum);
-    }
-    if (lane == 0) {
-        red[warp][0] = make_float2(gsum.hi, gsum.lo);
-        red[warp][1] = make_float2(dsum.hi, dsum.lo);
-        red[warp][2] = make_float2(xa2.hi, xa2.lo);
-        red[warp][3] = make_float2(hsum.hi, hsum.lo);
-        red[warp][4] = make_float2(tsum.hi, tsum.lo);
-    }
-    __syncthreads();
-    if (tid < 32) {
-        // warp w's terms in lane w
-        ff t[5];
-#pragma unroll
-        for (int c = 0; c < 5; ++c) {
-            const float2 v = lane < TT_THREADS / 32 && (c == 0 || lane < 4) ? red[lane][c] : make_float2(0.f, 0.f);
-            t[c] = ff_warp_sum(ff{v.x, v.y});
-        }
-        if (lane == 0) {
-            const double ik = 1.0 / (double)(k - 1);
-            const double gt2 = (double)t[0].hi + (double)t[0].lo, d2 = (double)t[1].hi + (double)t[1].lo;
-            const double a2 = (double)t[2].hi + (double)t[2].lo, h = (double)t[3].hi + (double)t[3].lo;
-            const double tau = ((double)t[4].hi + (double)t[4].lo) * ik;
-            const double t_range = d2 * ik, t_A = a2 * ik;
-            const int64_t q = m - p;
-            double t_null = 0.0;
-            if (q > 0) {
-                if (variant == MECUCO_FAST_HAAR) {
-                    const double tB = tau + (gt2 - 2.0 * h) * ik;
-                    t_null = (t_A + 2.0 * tB) / (double)(q + 2);
-                } else {
-                    const double tB = gt2 * ik - tau;  // |X_c V_r|_F^2 / (k-1) = tau
-                    t_null = (t_A + 2.0 * tB) / (double)q;
-                }
-            }
-            kappa[pt] = (float)fabs(0.5 * (t_range + t_null) + 0.5 * tau);
-        }
-    }
+    fast_kappa<TT_THREADS>(k, p, m, variant, gsum, sg, R + pt * k, diag, TT_DLD, Us, 65, Qs, 65, c_s, red, kappa + pt);
     if (lambda_out)
         for (int l = tid; l < k; l += TT_THREADS)
             lambda_out[pt * k + l] = (l < p) ? fmaxf(sg[l], 0.f) / (float)(k - 1) : 0.f;
