@@ -64,6 +64,33 @@ __host__ __device__ inline size_t bw_smem_bytes(int k) {
     return (size_t)5 * ((k + 3) / 4 * 4) * bw_ld(k) * sizeof(float);
 }
 
+// Asynchronous copies into shared memory; a thread waits for its own groups.
+template <int B>
+__device__ __forceinline__ void cp_async(float *dst, const float *src) {
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    if (B == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+// k rows of k floats, row r from src(r), to dst (row stride ld): 16-byte copies
+// where the rows are aligned to them.  All NT threads; no commit.
+template <int NT, typename F>
+__device__ __forceinline__ void copy_rows_async(float *dst, int ld, int k, F src) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if ((k & 3) == 0) {
+        const int q4 = k >> 2, rpw = 32 / q4, rr = lane / q4, c = 4 * (lane - rr * q4);
+        if (rr < rpw)
+            for (int r = warp * rpw + rr; r < k; r += NT / 32 * rpw) cp_async<16>(dst + r * ld + c, src(r) + c);
+    } else {
+        for (int r = warp; r < k; r += NT / 32)
+            for (int c = lane; c < k; c += 32) cp_async<4>(dst + r * ld + c, src(r) + c);
+    }
+}
+
 // v[i][c] = sum_{x < n} A[x][i0 + i] B[x][c0 + c], x ascending (rows of A and B
 // stand for the product's contracted index).
 __device__ __forceinline__ void tile_mul(const float *A, const float *B, int ld, int n, int i0, int c0,
@@ -107,8 +134,10 @@ __device__ __forceinline__ void tile_store_t(float *D, int ld, int i0, int c0, c
 // sign at the end.  Per j five k x k x k products (M_j W, W^T B, B dS, W dS,
 // (W dS) W^T) from 16-byte shared loads and packed FMAs, every sum in ascending
 // order of its index.  Bound by the FP32 lanes and the shared reads that feed
-// them.  Both adjoint kernels of 8,000 points at 256 columns, k = 32: 42.2 ms with
-// two passes over j and scalar products, 11.8 as they are.
+// them; M_{j+1} is copied into shared memory behind the products of j.  Both
+// adjoint kernels of 8,000 points at 256 columns, k = 32: 42.2 ms with two passes
+// over j and scalar products, 11.8 with one pass on packed FMAs, 6.2 with the
+// copies of M, dM and C (below) under way while the rows before are worked on.
 template <int NT, int MINB>
 __global__ void __launch_bounds__(NT, MINB)
 adjoint_kspace_kernel(const float *__restrict__ sigma, const float *__restrict__ U, const float *__restrict__ M,
@@ -119,9 +148,9 @@ adjoint_kspace_kernel(const float *__restrict__ sigma, const float *__restrict__
     const int k4 = (k + 3) / 4 * 4, ld = bw_ld(k), nt = k4 / 4;
     float *W = bsm;              // W[r][l]
     float *Wt = W + k4 * ld;     // W[l][r]
-    float *Ms = Wt + k4 * ld;    // M_j, then (W dS_j)^T
+    float *Ms = Wt + k4 * ld;    // M_j
     float *Bs = Ms + k4 * ld;    // M_j W, then dS_j
-    float *Bt = Bs + k4 * ld;    // (M_j W)^T
+    float *Bt = Bs + k4 * ld;    // (M_j W)^T, then (W dS_j)^T
     __shared__ float Adiag[64], xd[64], sg[64];
     __shared__ double red[NT / 32][2];
     __shared__ float s_scal[8];
@@ -167,13 +196,15 @@ adjoint_kspace_kernel(const float *__restrict__ sigma, const float *__restrict__
     const float dg2 = s_scal[0], ga = s_scal[1], gc = s_scal[2];
     float dW[4][4] = {};
     double acc_range = 0.0, acc_gt2 = 0.0, acc_A = 0.0;
+    auto load_m = [&](int j) {
+        copy_rows_async<NT>(Ms, ld, k, [&](int r) {
+            return D + (int64_t)pair_index(j < r ? j : r, j < r ? r : j, k) * k;
+        });
+        cp_async_commit();
+    };
+    load_m(0);
     for (int j = 0; j < k; ++j) {
-        __syncthreads();
-        for (int r = warp; r < k; r += NT / 32) {
-            const int a = j < r ? j : r, b = j < r ? r : j;
-            const float *src = D + (int64_t)pair_index(a, b, k) * k;
-            for (int t = lane; t < k; t += 32) Ms[r * ld + t] = src[t];
-        }
+        cp_async_wait<0>();
         __syncthreads();
         float v[4][4];
         // B = M_j W (M_j symmetric)
@@ -183,6 +214,7 @@ adjoint_kspace_kernel(const float *__restrict__ sigma, const float *__restrict__
             tile_store_t(Bt, ld, i0, c0, v);
         }
         __syncthreads();
+        if (j + 1 < k) load_m(j + 1);  // M_j has been read
         // S = W^T B
         if (mine) {
             tile_mul(W, Bs, ld, k, i0, c0, v);
@@ -221,19 +253,20 @@ adjoint_kspace_kernel(const float *__restrict__ sigma, const float *__restrict__
         }
         __syncthreads();
         if (mine) {
-            // dW += 2 B dS_j; (W dS_j)^T over M_j
+            // dW += 2 B dS_j; (W dS_j)^T over B^T
             tile_mul(Bt, Bs, ld, p, i0, c0, v);
 #pragma unroll
             for (int i = 0; i < 4; ++i)
 #pragma unroll
                 for (int c = 0; c < 4; ++c) dW[i][c] = fmaf(2.f, v[i][c], dW[i][c]);
             tile_mul(Wt, Bs, ld, p, i0, c0, v);
-            tile_store_t(Ms, ld, i0, c0, v);
         }
+        __syncthreads();
+        if (mine) tile_store_t(Bt, ld, i0, c0, v);
         __syncthreads();
         // dM_j = (W dS_j) W^T
         if (mine) {
-            tile_mul(Ms, Wt, ld, p, i0, c0, v);
+            tile_mul(Bt, Wt, ld, p, i0, c0, v);
             float *dMj = dMbuf + (pt * (int64_t)k + j) * k * k;
 #pragma unroll
             for (int i = 0; i < 4; ++i)
@@ -385,20 +418,28 @@ adjoint_kspace_kernel(const float *__restrict__ sigma, const float *__restrict__
     for (int r = warp; r < k; r += NT / 32)
         for (int t = lane; t < k; t += 32)
             dG[pt * (int64_t)k * k + r * k + t] = sgn * (0.5f * (Bt[r * ld + t] + Bt[t * ld + r]));
-    // ---- C_i[r][t] = dM[i,r,t] + dM[r,i,t] + dM[t,i,r]: rows dM[r, i, .] staged in
-    // Ms, so that every global access is along a row
+    // ---- C_i[r][t] = dM[i,r,t] + dM[r,i,t] + dM[t,i,r]: the rows dM[r, i, .] and
+    // dM[i, r, .] staged in shared memory, those of i + 1 on the way while C_i is
+    // written, so that every global access is along a row
     const float *dMp = dMbuf + pt * (int64_t)k * k * k;
     const int k8 = (k + 7) / 8 * 8;  // C's rows, zero past k
     float *Cp = Cout + pt * (int64_t)k * k * k8;
+    float *across[2] = {W, Ms}, *along[2] = {Wt, Bs};
+    auto load_c = [&](int i) {
+        copy_rows_async<NT>(i & 1 ? across[1] : across[0], ld, k, [&](int r) { return dMp + (r * k + i) * k; });
+        copy_rows_async<NT>(i & 1 ? along[1] : along[0], ld, k, [&](int r) { return dMp + (i * k + r) * k; });
+        cp_async_commit();
+    };
+    load_c(0);  // W, Ms, Wt and Bs were last read before the barrier above; dM_j was written before many
     for (int i = 0; i < k; ++i) {
+        cp_async_wait<0>();
         __syncthreads();
-        for (int r = warp; r < k; r += NT / 32)
-            for (int t = lane; t < k; t += 32) Ms[r * ld + t] = dMp[(r * k + i) * k + t];
-        __syncthreads();
+        if (i + 1 < k) load_c(i + 1);  // its buffers were read in the step before
+        const float *ac = i & 1 ? across[1] : across[0], *al = i & 1 ? along[1] : along[0];
         for (int r = warp; r < k; r += NT / 32)
             for (int t = lane; t < k8; t += 32)
                 Cp[(i * k + r) * k8 + t] =
-                    t < k ? sgn * (dMp[(i * k + r) * k + t] + Ms[r * ld + t] + Ms[t * ld + r]) : 0.f;
+                    t < k ? sgn * (al[r * ld + t] + ac[r * ld + t] + ac[t * ld + r]) : 0.f;
     }
 }
 
@@ -407,15 +448,49 @@ adjoint_kspace_kernel(const float *__restrict__ sigma, const float *__restrict__
 // (four per lane of every warp).  Warp w forms rows i = w, w + 8, ... of dZ:
 // 2 dG z + dR and the quadratic form z^T C_i z, whose matrix is symmetric, by 8 x
 // 8 blocks on and above the diagonal (the ones above count twice) - 8 rows of C_i
-// z for 4 columns in registers, packed along the rows, C_i's entries read as
-// warp-uniform 16-byte loads.  Then dX_c = U0 dZ, the centring adjoint subtracts
+// z for 4 columns in registers, packed along the rows.  The warp copies the next
+// AP_ROWS rows of such a block column into its own pair of buffers while it works
+// on the present ones, whose entries it reads as uniform 16-byte loads.  Then dX_c = U0 dZ, the centring adjoint subtracts
 // the column mean, and the result is atomically added to dX rows idx[pt, :].
 // Bound by the FP32 lanes (the quadratic forms: k^3 multiply-adds a column); the
 // figures stand at adjoint_kspace_kernel.
 constexpr int AP_CH = 128;
-__host__ __device__ inline size_t adjoint_patch_smem() {
-    return sizeof(float) * (size_t)(2 * 64 * AP_CH + 64 * 65 + 2 * AP_CH);
+constexpr int AP_ROWS = 32;  // rows of C_i per buffer
+__host__ __device__ inline size_t adjoint_patch_smem(int k) {
+    const size_t k8 = (k + 7) / 8 * 8;
+    return sizeof(float) * (2 * k8 * AP_CH + 8 * 2 * AP_ROWS * 8 + 2 * AP_CH + 64 * 65);
 }
+
+// A run of rows [s0, s1) of the block column r0 of C_i: the rows right of the
+// diagonal block (i.e. below it, C_i being symmetric) in runs of AP_ROWS, then the
+// diagonal block's own, then the next block column, then the warp's next i.
+struct AdjRun {
+    int i, r0, s0, s1;
+    bool diag;
+    __device__ void start(int k) {
+        s0 = r0 + 8;
+        diag = s0 >= k;
+        if (diag) s0 = r0;
+        s1 = diag ? k : min(s0 + AP_ROWS, k);
+    }
+    __device__ void next(int k) {
+        if (!diag && s1 < k) {
+            s0 = s1;
+            s1 = min(s0 + AP_ROWS, k);
+        } else if (!diag) {
+            diag = true;
+            s0 = r0;
+            s1 = r0 + 8;
+        } else {
+            r0 += 8;
+            if (r0 >= k) {
+                r0 = 0;
+                i += 8;
+            }
+            start(k);
+        }
+    }
+};
 
 // sum over rows l < k of Us(l) * Z[l][4 lane ..], as two packed pairs
 template <typename F>
@@ -439,14 +514,15 @@ adjoint_patch_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld, 
                      const float *__restrict__ dR,
                      const float *__restrict__ dQ, const float *__restrict__ C, float *__restrict__ dX, int64_t ldd) {
     extern __shared__ __align__(16) float psm[];
-    float *Xs = psm;                  // [64][AP_CH] X_c, then dZ
-    float *Zs = Xs + 64 * AP_CH;      // [64][AP_CH] Z (rows k .. zero), then dX_c
-    float(*Us)[65] = reinterpret_cast<float(*)[65]>(Zs + 64 * AP_CH);
-    float *wa = reinterpret_cast<float *>(Us) + 64 * 65, *xq = wa + AP_CH;  // Haar: |z|^2, z^T dQ z per column
+    const int kk = k * k, k8 = (k + 7) / 8 * 8;
+    float *Xs = psm;                  // [k8][AP_CH] X_c, then dZ
+    float *Zs = Xs + k8 * AP_CH;      // [k8][AP_CH] Z (rows k .. zero), then dX_c
+    float *Cs = Zs + k8 * AP_CH;      // per warp: two buffers of AP_ROWS x 8 of C_i
+    float *wa = Cs + 8 * 2 * AP_ROWS * 8, *xq = wa + AP_CH;  // Haar: |z|^2, z^T dQ z per column
+    float(*Us)[65] = reinterpret_cast<float(*)[65]>(xq + AP_CH);
     __shared__ int rows[64];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t pt = blockIdx.x;
-    const int kk = k * k, k8 = (k + 7) / 8 * 8;
     const bool haar = variant == MECUCO_FAST_HAAR;
     if (tid < k) {
         int r = idx[pt * k + tid];
@@ -495,6 +571,19 @@ adjoint_patch_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld, 
             }
             __syncthreads();
         }
+        float *Cw = Cs + warp * 2 * AP_ROWS * 8;
+        int buf = 0;
+        AdjRun nx{warp, 0, 0, 0, false};
+        nx.start(k);
+        auto load_run = [&](const AdjRun &run, float *dst) {
+            if (run.i < k && run.s0 + lane < run.s1) {
+                const float *src = Cp + ((int64_t)run.i * k + run.s0 + lane) * k8 + run.r0;
+                cp_async<16>(dst + lane * 8, src);
+                cp_async<16>(dst + lane * 8 + 4, src + 4);
+            }
+            cp_async_commit();
+        };
+        load_run(nx, Cw);
         for (int i = warp; i < k; i += 8) {
             const float4 g = row_mix(Zs, k, lane, [&](int r) { return __ldg(Gp + i * k + r); });
             float y[4] = {2.f * g.x, 2.f * g.y, 2.f * g.z, 2.f * g.w};
@@ -507,34 +596,42 @@ adjoint_patch_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld, 
                 for (int c = 0; c < 4; ++c)
                     y[c] += 2.f * wa[4 * lane + c] * qe[c] + 2.f * ze[c] * xq[4 * lane + c];
             }
-            const float *Ci = Cp + (int64_t)i * k * k8;
             f2 cq[4] = {};
             for (int r0 = 0; r0 < k; r0 += 8) {
                 f2 t[4][4] = {};  // [row pair][column]
-                auto step = [&](int s) {
-                    const float4 z = *reinterpret_cast<const float4 *>(Zs + s * AP_CH + 4 * lane);
-                    f2 cp[4];
-                    const ulonglong2 c0 = __ldg(reinterpret_cast<const ulonglong2 *>(Ci + s * k8 + r0));
-                    const ulonglong2 c1 = __ldg(reinterpret_cast<const ulonglong2 *>(Ci + s * k8 + r0) + 1);
-                    cp[0] = c0.x, cp[1] = c0.y, cp[2] = c1.x, cp[3] = c1.y;
-                    const float zc[4] = {z.x, z.y, z.z, z.w};
+                bool diag;
+                do {
+                    const AdjRun run = nx;  // of this i and r0
+                    nx.next(k);
+                    load_run(nx, Cw + (buf ^ 1) * AP_ROWS * 8);
+                    cp_async_wait<1>();  // the present run has landed
+                    __syncwarp();
+                    const float *cb = Cw + buf * AP_ROWS * 8, *zs = Zs + run.s0 * AP_CH + 4 * lane;
+                    diag = run.diag;
+                    if (diag) {  // what came before counts twice
+                        const f2 two = pack2(2.f, 2.f);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const f2 z2 = pack2(zc[c], zc[c]);
+                        for (int e = 0; e < 4; ++e)
 #pragma unroll
-                        for (int e = 0; e < 4; ++e) t[e][c] = fma2(cp[e], z2, t[e][c]);
+                            for (int c = 0; c < 4; ++c) t[e][c] = fma2(t[e][c], two, 0ull);
                     }
-                };
-                // blocks right of the diagonal one count twice
 #pragma unroll 4
-                for (int s = r0 + 8; s < k; ++s) step(s);
-                const f2 two = pack2(2.f, 2.f);
+                    for (int s = 0; s < run.s1 - run.s0; ++s) {
+                        const float4 z = *reinterpret_cast<const float4 *>(zs + s * AP_CH);
+                        const ulonglong2 c0 = *reinterpret_cast<const ulonglong2 *>(cb + s * 8);
+                        const ulonglong2 c1 = *reinterpret_cast<const ulonglong2 *>(cb + s * 8 + 4);
+                        const f2 cp[4] = {c0.x, c0.y, c1.x, c1.y};
+                        const float zc[4] = {z.x, z.y, z.z, z.w};
 #pragma unroll
-                for (int e = 0; e < 4; ++e)
+                        for (int c = 0; c < 4; ++c) {
+                            const f2 z2 = pack2(zc[c], zc[c]);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) t[e][c] = fma2(t[e][c], two, 0ull);
-                const int s1 = min(k, r0 + 8);
-                for (int s = r0; s < s1; ++s) step(s);
+                            for (int e = 0; e < 4; ++e) t[e][c] = fma2(cp[e], z2, t[e][c]);
+                        }
+                    }
+                    __syncwarp();  // the buffer has been read
+                    buf ^= 1;
+                } while (!diag);
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     const float4 za = *reinterpret_cast<const float4 *>(Zs + (r0 + 2 * e) * AP_CH + 4 * lane);
@@ -592,7 +689,7 @@ cudaError_t launch_adjoint(const void *X, mecuco_dtype dt, int64_t N, int64_t m,
                     : k <= 44 ? kspace(adjoint_kspace_kernel<128, 4>, 128)
                               : kspace(adjoint_kspace_kernel<256, 2>, 256);
     if (e != cudaSuccess) return e;
-    const size_t psmem = adjoint_patch_smem();
+    const size_t psmem = adjoint_patch_smem(k);
     if (dt == MECUCO_BF16) {
         e = cudaFuncSetAttribute(adjoint_patch_kernel<__nv_bfloat16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)psmem);
