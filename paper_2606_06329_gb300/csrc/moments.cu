@@ -20,7 +20,7 @@
 // adjoint uses this.
 //
 // A chunk is MCH columns: gathered row by row (a warp per row, a lane per
-// column), centred (a lane per column, the rows shared between the warps: in
+// column, the next chunk's values on their way in registers), centred (a lane per column, the rows shared between the warps: in
 // two-term FP32 for the rotated form, whose small directions would show the
 // rounding of the means), then rotated, or copied, into column-major order, which
 // is what 16-byte operand loads want.  Every sum of a result runs in ascending
@@ -63,15 +63,31 @@ __device__ __forceinline__ int checked_row(int r, int64_t N, DevCounters *ctr) {
 constexpr int MCH = 32;  // columns per chunk
 constexpr int XLD = 34;  // row stride of a row-major chunk (even: 8-byte loads)
 
-template <typename T, int NT>
-__device__ __forceinline__ void load_chunk(float *Xr, const T *__restrict__ X, int64_t ld, const int *rows, int k,
-                                           int64_t a0, int64_t m) {
-    const int lane = threadIdx.x & 31;
-    const bool in = a0 + lane < m;
-#pragma unroll 8
-    for (int r = threadIdx.x >> 5; r < k; r += NT / 32)
-        Xr[r * XLD + lane] = in ? load_elem(X + (int64_t)rows[r] * ld + a0 + lane) : 0.f;
-}
+// Rows warp, warp + NT / 32, ... (NR at most) of a chunk in registers: loaded while
+// the chunk before is worked on, then stored.
+template <int NT, int NR>
+struct ChunkRows {
+    float v[NR];
+    template <typename T>
+    __device__ __forceinline__ void load(const T *__restrict__ X, int64_t ld, const int *rows, int k, int64_t a0,
+                                         int64_t m) {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+        const bool in = a0 + lane < m;
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            const int r = warp + i * (NT / 32);
+            v[i] = in && r < k ? load_elem(X + (int64_t)rows[r] * ld + a0 + lane) : 0.f;
+        }
+    }
+    __device__ __forceinline__ void store(float *Xr, int k) const {
+        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            const int r = warp + i * (NT / 32);
+            if (r < k) Xr[r * XLD + lane] = v[i];
+        }
+    }
+};
 
 // x - mean, rounded once (two-term sums); part: NT floats x 2.  Ends before a barrier.
 template <int NT>
@@ -165,15 +181,19 @@ __device__ __forceinline__ void transpose_chunk(const float *Xr, float *Z, int k
 // CTAs leave room for many points on an SM, which hides the barriers between the
 // steps of a chunk.  Measured (the plain and the rotated Gram of 20,000 points, 256
 // columns, k = 32): 4.7 ms with FP64 centring by 64 threads, scalar operand loads
-// and 64 of 256 threads at work, 1.7 as it is.
+// and 64 of 256 threads at work, 1.7 without the next chunk under way, 1.5 with it
+// (1.6 without the bound on the registers).
 // ---------------------------------------------------------------------------
 __host__ __device__ inline size_t gram_smem_floats(int k, bool rot, int nt) {
     const int kp = (k + 3) / 4 * 4, ldz = kp + 4;
     return (size_t)(rot ? k * ldz : 0) + MCH * ldz + kp * XLD + 2 * nt;
 }
 
+// largest k of a CTA of NT threads over its warps
+constexpr int GRAM_NR(int nt) { return nt == 64 ? 20 : nt == 128 ? 15 : 13; }
+
 template <typename T, int NT, bool ROT, bool WQ>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(NT, NT == 64 ? 10 : NT == 128 ? 5 : 4)
 patch_gram_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld, const int32_t *__restrict__ idx,
                   int k, int64_t p0, const float *__restrict__ rot, float *__restrict__ G, float *__restrict__ R,
                   float *__restrict__ Q, DevCounters *ctr) {
@@ -195,8 +215,11 @@ patch_gram_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld, con
     f2 g[4][2] = {}, qq[4][2] = {};
     float rsum = 0.f;
     __syncthreads();
+    ChunkRows<NT, GRAM_NR(NT)> next;
+    next.load(X, ld, rows, k, 0, m);
     for (int64_t a0 = 0; a0 < m; a0 += MCH) {
-        load_chunk<T, NT>(Xr, X, ld, rows, k, a0, m);
+        next.store(Xr, k);
+        if (a0 + MCH < m) next.load(X, ld, rows, k, a0 + MCH, m);
         __syncthreads();
         if (ROT) centre_two_term<NT>(Xr, k, part);
         else centre_plain<NT>(Xr, k, part);
@@ -327,7 +350,8 @@ cudaError_t launch_patch_gram(const void *X, mecuco_dtype dt, int64_t N, int64_t
 // Bound by the FP32 lanes: 64 multiply-adds a column and item in 32 packed
 // instructions, and the steps between the barriers of a chunk.
 // Measured (20,000 points, 256 columns, k = 32): 8.1 ms for M and 6.3 for the pass
-// over it, 4.4 for KAPPA; the gradient's M (8,000 points) 3.3 -> 1.7 ms.
+// over it, 4.4 for KAPPA, 4.2 with the next chunk under way; the gradient's M (8,000
+// points) 3.3 -> 1.6 ms.
 // ---------------------------------------------------------------------------
 int m3_items(int k) {
     int nb = (k + 7) / 8, n = 0;
@@ -359,6 +383,9 @@ __host__ __device__ inline size_t third_smem_floats(int k, bool kappa, int nt) {
     return (size_t)(kappa ? 3 : 1) * kp * ldz + MCH * ldz + (kappa ? 2 : 1) * kp * XLD + 2 * nt;
 }
 }  // namespace
+
+// largest k of a CTA of NT threads over its warps
+constexpr int THIRD_NR(int nt) { return nt == 96 ? 8 : nt == 160 ? 7 : 5; }
 
 template <typename T, int NT, int MINB, bool KAPPA>
 __global__ void __launch_bounds__(NT, MINB)
@@ -406,8 +433,11 @@ patch_m3_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld, const
         for (int r = 0; r < 8; ++r)
 #pragma unroll
             for (int t = 0; t < 4; ++t) acc[r][t] = 0ull;
+        ChunkRows<NT, THIRD_NR(NT)> next;
+        next.load(X, ld, rows, k, 0, m);
         for (int64_t a0 = 0; a0 < m; a0 += MCH) {
-            load_chunk<T, NT>(Xr, X, ld, rows, k, a0, m);
+            next.store(Xr, k);
+            if (a0 + MCH < m) next.load(X, ld, rows, k, a0 + MCH, m);
             __syncthreads();
             if (rot) centre_two_term<NT>(Xr, k, part);
             else centre_plain<NT>(Xr, k, part);
