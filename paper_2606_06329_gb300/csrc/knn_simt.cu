@@ -3,6 +3,8 @@
 // certification test, and the exact full-scan fallback.
 #include <math.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "kernels.h"
 
@@ -177,24 +179,27 @@ __device__ __forceinline__ f2 add2(f2 a, f2 b) {
 
 // ---------------------------------------------------------------------------
 // Candidate search, plain FP32.  A block of 256 threads owns 128 query rows and
-// sweeps its split of the candidate rows in tiles of 128; thread (tx, ty) of a
-// 16 x 16 grid accumulates rows 8 ty .. + 7 against columns 4 tx .. + 3 and
-// 64 + 4 tx .. + 3 as packed FP32 pairs (two columns per FMA; the query operand
-// is stored twice in a row, so that a 16-byte load brings it as pairs), over
-// K slices of 16 that are double-buffered through registers.
+// sweeps its split of the candidate rows in tiles of 256; thread (tx, ty) of a
+// 16 x 16 grid accumulates rows 8 ty .. + 7 against columns 64 g + 4 tx .. + 3
+// (g < 4) as packed FP32 pairs (two columns per FMA), over K slices of 16 that are
+// double-buffered through registers.  A 16-byte shared load takes the banks four
+// cycles whatever its lanes share, so the tile is as large as the registers
+// allow: 6 loads feed 64 packed FMAs, 192 of 256 cycles.
 // Selection: every row keeps its kc smallest d~ = |x|^2 + |y|^2 - 2 x.y as a
 // max-heap in shared memory.  A thread reserves room for its admitted entries
 // (below the heap's root) in the row's pending buffer with one shared atomic per
 // row, and 128 threads, one per row, fold the buffers into the heaps together
 // once any holds more than SP_HIGH; a tile that does not fit (the first ones,
-// which admit everything) is taken in four parts of 32 columns.
-// Measured per search: 50,000 x 256, k = 32 81 -> 33 ms (38 TFLOP/s; FP32-issue
-// bound with one block per SM); 20,000 x 24, k = 32 10.8 -> 1.7 ms (selection
+// which admit everything) is taken in eight parts of 32 columns.
+// Measured per search: 50,000 x 256, k = 32 81 -> 27 ms (47 TFLOP/s; FP32-issue
+// bound with one block per SM; 33 with 128-wide tiles and the query slice stored
+// twice, 28.5 with it stored once); 20,000 x 24, k = 32 10.8 -> 1.7 ms (selection
 // bound).  Before, 8 scalar loads per operand and K step and one thread per row
 // walking all 128 distances of a tile.
 // ---------------------------------------------------------------------------
-constexpr int SBM = 128, SBN = 128, SBK = 16, STHREADS = 256;
-constexpr int SLDA = 2 * SBM + 4, SLDB = SBN + 4;  // row strides of the operand slices (floats)
+constexpr int SBM = 128, SBN = 256, SBK = 16, STHREADS = 256;
+constexpr int SLDA = SBM + 4, SLDB = SBN + 4;  // row strides of the operand slices (floats)
+constexpr int NG = SBN / 64, NC = 4 * NG;      // groups of 4 columns, and columns, of a thread
 constexpr int SPEND = 32;    // pending candidates per row
 constexpr int SP_HIGH = 16;  // above this, a row asks for an update
 
@@ -273,7 +278,7 @@ knn_simt_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld,
                 const float *__restrict__ norms, int64_t q0, int64_t nq, int kc, int nsplit,
                 int include_self, float *__restrict__ cand_d, int32_t *__restrict__ cand_i) {
     extern __shared__ __align__(16) float smem[];
-    float *As = smem;                          // [2][SBK][SLDA] query slice, every value twice
+    float *As = smem;                          // [2][SBK][SLDA] query slice
     float *Bs = As + 2 * SBK * SLDA;           // [2][SBK][SLDB]
     float *Pd = Bs + 2 * SBK * SLDB;           // [SPEND][SBM] pending distances
     int *Pc = reinterpret_cast<int *>(Pd + SPEND * SBM);
@@ -332,56 +337,61 @@ knn_simt_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld,
     };
     bool filling = true;  // some list of the block may still be short
     for (int64_t c0 = cbeg; c0 < cend; c0 += SBN) {
-        f2 acc[8][4];
+        f2 acc[8][NC / 2];
 #pragma unroll
         for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int j = 0; j < 4; ++j) acc[i][j] = 0ull;
-        const T *crow[2];
+            for (int j = 0; j < NC / 2; ++j) acc[i][j] = 0ull;
+        const T *crow[NG];
 #pragma unroll
-        for (int h = 0; h < 2; ++h) crow[h] = X + min(c0 + lr + 64 * h, N - 1) * ld;
-        float4 ra[2], rb[2];
+        for (int h = 0; h < NG; ++h) crow[h] = X + min(c0 + lr + 64 * h, N - 1) * ld;
+        float4 ra[2], rb[NG];
         auto fetch = [&](int sl) {
             const int64_t a = (int64_t)sl * SBK + 4 * lq;
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                ra[h] = load4(qrow[h], a, m, vec);
-                rb[h] = load4(crow[h], a, m, vec);
-            }
+            for (int h = 0; h < 2; ++h) ra[h] = load4(qrow[h], a, m, vec);
+#pragma unroll
+            for (int h = 0; h < NG; ++h) rb[h] = load4(crow[h], a, m, vec);
         };
         auto stage = [&](int buf) {
             float *A = As + buf * SBK * SLDA, *B = Bs + buf * SBK * SLDB;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const float av[4] = {ra[h].x, ra[h].y, ra[h].z, ra[h].w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) A[(4 * lq + e) * SLDA + lr + 64 * h] = av[e];
+            }
+#pragma unroll
+            for (int h = 0; h < NG; ++h) {
                 const float bv[4] = {rb[h].x, rb[h].y, rb[h].z, rb[h].w};
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    *reinterpret_cast<float2 *>(A + (4 * lq + e) * SLDA + 2 * (lr + 64 * h)) = make_float2(av[e], av[e]);
-                    B[(4 * lq + e) * SLDB + lr + 64 * h] = bv[e];
-                }
+                for (int e = 0; e < 4; ++e) B[(4 * lq + e) * SLDB + lr + 64 * h] = bv[e];
             }
         };
         fetch(0);
-        if (tid < SBN) cns[tid] = (c0 + tid < cend) ? norms[c0 + tid] : INFINITY;
+        cns[tid] = (c0 + tid < cend) ? norms[c0 + tid] : INFINITY;
         stage(0);
         __syncthreads();
         for (int sl = 0; sl < nslice; ++sl) {
             if (sl + 1 < nslice) fetch(sl + 1);
-            const float *A = As + (sl & 1) * SBK * SLDA + 16 * ty, *B = Bs + (sl & 1) * SBK * SLDB + 4 * tx;
+            const float *A = As + (sl & 1) * SBK * SLDA + 8 * ty, *B = Bs + (sl & 1) * SBK * SLDB + 4 * tx;
 #pragma unroll
             for (int kk = 0; kk < SBK; ++kk) {
-                ulonglong2 a2[4], b2[2];
+                const float4 a0 = *reinterpret_cast<const float4 *>(A + kk * SLDA);
+                const float4 a1 = *reinterpret_cast<const float4 *>(A + kk * SLDA + 4);
+                f2 b[NC / 2];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) a2[i] = *reinterpret_cast<const ulonglong2 *>(A + kk * SLDA + 4 * i);
-                b2[0] = *reinterpret_cast<const ulonglong2 *>(B + kk * SLDB);
-                b2[1] = *reinterpret_cast<const ulonglong2 *>(B + kk * SLDB + 64);
-                const f2 b[4] = {b2[0].x, b2[0].y, b2[1].x, b2[1].y};
+                for (int g = 0; g < NG; ++g) {
+                    const ulonglong2 b2 = *reinterpret_cast<const ulonglong2 *>(B + kk * SLDB + 64 * g);
+                    b[2 * g] = b2.x;
+                    b[2 * g + 1] = b2.y;
+                }
+                const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const f2 a = i & 1 ? a2[i / 2].y : a2[i / 2].x;
+                    const f2 a = pack2(av[i], av[i]);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) acc[i][j] = fma2(a, b[j], acc[i][j]);
+                    for (int j = 0; j < NC / 2; ++j) acc[i][j] = fma2(a, b[j], acc[i][j]);
                 }
             }
             if (sl + 1 < nslice) stage((sl + 1) & 1);
@@ -389,24 +399,25 @@ knn_simt_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld,
         }
         // distances in place: column 2j of a pair and 2j + 1
         const bool selfs = !include_self && c0 < qb + SBM && qb < c0 + SBN;
-        float cn[8];
+        // append this thread's entries of its columns [J0, J1); flags[0] if a row's
+        // buffer has no room for them
+        auto append = [&](auto J0, auto J1) {
+            constexpr int j0 = decltype(J0)::value, j1 = decltype(J1)::value;
+            float cn[j1 - j0];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) cn[j] = cns[(j >> 2) * 64 + 4 * tx + (j & 3)];
-        // append this thread's entries of columns [j0, j1) (of its 8); false if a
-        // row's buffer has no room for them
-        auto append = [&](int j0, int j1) {
+            for (int j = j0; j < j1; ++j) cn[j - j0] = cns[(j >> 2) * 64 + 4 * tx + (j & 3)];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
                 const int r = 8 * ty + i;
                 const float q = qns[r], t = thr[r];
-                float d[8];
+                float d[j1 - j0];
                 unsigned adm = 0;
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
+                for (int j = j0; j < j1; ++j) {
                     const float2 v = unpack2(acc[i][j >> 1]);
-                    d[j] = fmaf(-2.f, (j & 1) ? v.y : v.x, q + cn[j]);
+                    d[j - j0] = fmaf(-2.f, (j & 1) ? v.y : v.x, q + cn[j - j0]);
                     const int c = (j >> 2) * 64 + 4 * tx + (j & 3);
-                    const bool in = j >= j0 && j < j1 && d[j] < t && !(selfs && c0 + c == qb + r);
+                    const bool in = d[j - j0] < t && !(selfs && c0 + c == qb + r);
                     adm |= (in ? 1u : 0u) << j;
                 }
                 if (adm) {
@@ -417,9 +428,9 @@ knn_simt_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld,
                     } else {
                         if (pos + na > SP_HIGH) flags[1] = 1;
 #pragma unroll
-                        for (int j = 0; j < 8; ++j)
+                        for (int j = j0; j < j1; ++j)
                             if ((adm >> j) & 1u) {
-                                Pd[pos * SBM + r] = d[j];
+                                Pd[pos * SBM + r] = d[j - j0];
                                 Pc[pos * SBM + r] = (int)c0 + (j >> 2) * 64 + 4 * tx + (j & 3);
                                 ++pos;
                             }
@@ -429,7 +440,7 @@ knn_simt_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld,
         };
         bool parts = filling;
         if (!parts) {
-            append(0, 8);
+            append(std::integral_constant<int, 0>(), std::integral_constant<int, NC>());
             __syncthreads();
             parts = flags[0] != 0;
             if (parts) {
@@ -443,8 +454,16 @@ knn_simt_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld,
         if (parts) {
             update();
 #pragma unroll 1
-            for (int p = 0; p < 4; ++p) {
-                append(2 * p, 2 * p + 2);  // at most 32 entries a row
+            for (int p = 0; p < NC / 2; ++p) {  // two columns a thread: at most 32 entries a row
+                using std::integral_constant;
+                if (p == 0) append(integral_constant<int, 0>(), integral_constant<int, 2>());
+                else if (p == 1) append(integral_constant<int, 2>(), integral_constant<int, 4>());
+                else if (p == 2) append(integral_constant<int, 4>(), integral_constant<int, 6>());
+                else if (p == 3) append(integral_constant<int, 6>(), integral_constant<int, 8>());
+                else if (p == 4) append(integral_constant<int, 8>(), integral_constant<int, 10>());
+                else if (p == 5) append(integral_constant<int, 10>(), integral_constant<int, 12>());
+                else if (p == 6) append(integral_constant<int, 12>(), integral_constant<int, 14>());
+                else append(integral_constant<int, 14>(), integral_constant<int, 16>());
                 __syncthreads();
                 update();
             }
@@ -474,23 +493,16 @@ cudaError_t launch_knn_simt(const void *X, mecuco_dtype dt, int64_t N, int64_t m
                             const float *norms, int64_t q0, int64_t nq, int kc, int nsplit,
                             int include_self, float *cand_d, int32_t *cand_i, cudaStream_t s) {
     if (nq <= 0) return cudaSuccess;
-    size_t smem = simt_smem_bytes(kc);
-    dim3 grid((unsigned)((nq + SBM - 1) / SBM), (unsigned)nsplit), block(STHREADS);
-    cudaError_t e;
-    if (dt == MECUCO_BF16) {
-        e = cudaFuncSetAttribute(knn_simt_kernel<__nv_bfloat16>,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const dim3 grid((unsigned)((nq + SBM - 1) / SBM), (unsigned)nsplit);
+    const size_t smem = simt_smem_bytes(kc);
+    auto run = [&](auto kern, const auto *Xp) -> cudaError_t {
+        const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
-        knn_simt_kernel<<<grid, block, smem, s>>>((const __nv_bfloat16 *)X, N, m, ld, norms, q0, nq,
-                                                  kc, nsplit, include_self, cand_d, cand_i);
-    } else {
-        e = cudaFuncSetAttribute(knn_simt_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
-        if (e != cudaSuccess) return e;
-        knn_simt_kernel<<<grid, block, smem, s>>>((const float *)X, N, m, ld, norms, q0, nq, kc,
-                                                  nsplit, include_self, cand_d, cand_i);
-    }
-    return cudaGetLastError();
+        kern<<<grid, STHREADS, smem, s>>>(Xp, N, m, ld, norms, q0, nq, kc, nsplit, include_self, cand_d, cand_i);
+        return cudaGetLastError();
+    };
+    return dt == MECUCO_BF16 ? run(knn_simt_kernel<__nv_bfloat16>, (const __nv_bfloat16 *)X)
+                             : run(knn_simt_kernel<float>, (const float *)X);
 }
 
 // ---------------------------------------------------------------------------
