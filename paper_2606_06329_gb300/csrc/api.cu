@@ -1293,30 +1293,39 @@ mecuco_status mecuco_curvature_backward(mecuco_t h, const void *X, mecuco_dtype 
     cudaStream_t s = (cudaStream_t)stream;
     if ((st = begin_call(h, s)) != MECUCO_OK) return st;
     if ((st = ensure_items(h, k)) != MECUCO_OK) return st;
-    // per point: forward buffers (incl. U0) + dG, dR, dQ + C and dM (k^3 each)
-    const int64_t k8 = (k + 7) / 8 * 8;  // C's rows
+    // per point: forward buffers (incl. U0) + dG, dR, dQ + C (its rows rounded up to k8) and dM
+    const int64_t k8 = (k + 7) / 8 * 8;
     const int64_t per_point = m3_pair_floats(k) + 7LL * k * k + 4LL * k + (int64_t)k * k * (k + k8);
     int64_t chunk = h->chunk_points > 0 ? h->chunk_points
                                          : std::max<int64_t>(256, std::min<int64_t>(65536, ((int64_t)2 << 30) /
                                                                                              (per_point * 4)));
     chunk = std::min(chunk, N);
-    Carver t(nullptr);
     EstBufs b;
-    est_scratch(t, chunk, k, &b, 0, 0, true);
-    t.take<float>((size_t)chunk * k * k);
-    t.take<float>((size_t)chunk * k);
-    t.take<float>((size_t)chunk * k * k);
-    t.take<float>((size_t)chunk * k * k * k8);
-    t.take<float>((size_t)chunk * k * k * k);
-    if ((st = ensure(h->ws, h->ws_bytes, t.off, h->ws_cap)) != MECUCO_OK) return st;
+    float *dG, *dR, *dQ, *Cb, *dM;
+    auto carve = [&](Carver &c) {
+        est_scratch(c, chunk, k, &b, 0, 0, true);
+        dG = c.take<float>((size_t)chunk * k * k);
+        dR = c.take<float>((size_t)chunk * k);
+        dQ = c.take<float>((size_t)chunk * k * k);
+        Cb = c.take<float>((size_t)chunk * k * k * k8);
+        dM = c.take<float>((size_t)chunk * k * k * k);
+        return c.off;
+    };
+    auto bytes = [&] {
+        Carver c(nullptr);
+        return carve(c);
+    };
+    size_t need = bytes();
+    if (h->ws_cap && need > h->ws_cap && k8 != k && chunk > 1) {
+        // under a limit that holds the chunk but not the padding of C's rows: a
+        // chunk of as many bytes
+        chunk = std::max<int64_t>(1, chunk * (per_point - (int64_t)k * k * (k8 - k)) / per_point - 1);
+        need = bytes();
+    }
+    if ((st = ensure(h->ws, h->ws_bytes, need, h->ws_cap)) != MECUCO_OK) return st;
     Carver c(h->ws);
-    est_scratch(c, chunk, k, &b, 0, 0, true);
+    carve(c);
     float *U0 = b.U0;
-    float *dG = c.take<float>((size_t)chunk * k * k);
-    float *dR = c.take<float>((size_t)chunk * k);
-    float *dQ = c.take<float>((size_t)chunk * k * k);
-    float *Cb = c.take<float>((size_t)chunk * k * k * k8);
-    float *dM = c.take<float>((size_t)chunk * k * k * k);
     CK(cudaMemsetAsync(dX_out, 0, sizeof(float) * (size_t)N * m, s));
     const bool need_q = var == MECUCO_FAST_HAAR;
     const int rot_mode = h->jacobi_fp64 >= 0 ? h->jacobi_fp64 : 3;

@@ -1,5 +1,6 @@
 // estimator.cu - Step 4 (eqs. tnull, tA, tB, fast_curv; Alg. 1 Fast branch):
-// the Fast-mode curvature from the patch moments and the eigenpairs of G.
+// the Fast-mode curvature from the patch moments and Ritz pairs of G (the
+// randomised SVD; eigenpairs take the sums of fast_terms.cuh instead).
 //
 // With X_c = U_p S V_r^T (U_p the top-p eigenvectors of G = X_c X_c^T, S the
 // singular values) put W = U_p S^-1 (k x p), so V_r = X_c^T W.  Every term of
@@ -10,11 +11,9 @@
 //   X_c d_P = R - A 1_p                                   (d_P = 1 - V_r^{o2} 1)
 //   t_A     = |R - A 1_p|^2 / (k-1)
 //   G_tens[j] = W^T M_j W  (p x p),  |G_tens|_F^2 = sum_j |W^T M_j W|_F^2
-//   |X_c V_r|_F^2 = |G W|_F^2, which is sum_{l<p} s_l^2 = (k-1) tau when U_p
-//   holds eigenvectors of G, so the printed
-//   t_B = tau - 2 tau + |G_tens|^2/(k-1);  t_null = (t_A + 2 t_B)/(m - p).
-//   Given G (Ritz pairs of a randomised range finder, whose residuals G u_l -
-//   s_l^2 u_l are not 0) |G W|_F^2 is computed instead.
+//   |X_c V_r|_F^2 = |G W|_F^2, computed as such: the Ritz pairs' residuals
+//   G u_l - s_l^2 u_l are not 0, so it is not sum_{l<p} s_l^2 = (k-1) tau;
+//   t_B = tau - 2 |G W|_F^2/(k-1) + |G_tens|^2/(k-1);  t_null = (t_A + 2 t_B)/(m - p).
 //   Haar variant: sum_{j,a} X_c[j,a]^2 (1 - d_P[a]) = sum_l w_l^T Q w_l,
 //   t_B^H = tau - 2 (that)/(k-1) + |G_tens|^2/(k-1), t_null^H = (t_A + 2 t_B^H)/(m - p + 2)
 //   K = |(t_range + t_null)/2 + tau/2|.
@@ -165,16 +164,14 @@ estimator_kernel(const float *__restrict__ sigma, const float *__restrict__ U, c
             acc_h += (double)Ws[r][l] * t;
         }
     }
-    // |G W|_F^2 (only with G given)
+    // |G W|_F^2
     double acc_b2 = 0.0;
-    if (Gm) {
-        const float *gm = Gm + pt * (int64_t)k * k;
-        for (int e = tid; e < k * p; e += 256) {
-            const int r = e / p, l = e % p;
-            float t = 0.f;
-            for (int c = 0; c < k; ++c) t = fmaf(gm[r * k + c], Ws[c][l], t);
-            acc_b2 += (double)t * t;
-        }
+    const float *gm = Gm + pt * (int64_t)k * k;
+    for (int e = tid; e < k * p; e += 256) {
+        const int r = e / p, l = e % p;
+        float t = 0.f;
+        for (int c = 0; c < k; ++c) t = fmaf(gm[r * k + c], Ws[c][l], t);
+        acc_b2 += (double)t * t;
     }
     // block reduction of (acc_gt2, acc_h, acc_b2) and thread 0's (acc_range, acc_A)
     double v0 = acc_gt2, v1 = acc_h, v2 = acc_b2;
@@ -203,8 +200,7 @@ estimator_kernel(const float *__restrict__ sigma, const float *__restrict__ U, c
                 double tB = tau - 2.0 * h / km1 + gt2 / km1;
                 t_null = (t_A + 2.0 * tB) / (double)(q + 2);
             } else {
-                const double t_B2 = Gm ? b2 / km1 : tau;  // |X_c V_r|_F^2 / (k-1)
-                double tB = tau - 2.0 * t_B2 + gt2 / km1;
+                double tB = tau - 2.0 * (b2 / km1) + gt2 / km1;
                 t_null = (t_A + 2.0 * tB) / (double)q;
             }
         }

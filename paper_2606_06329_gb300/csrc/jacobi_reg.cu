@@ -1,6 +1,6 @@
 // jacobi_reg.cu - Step 3 (eq. svd_cov; Alg. 1 SVD_p): the eigenvectors of each
 // k x k patch Gram G = X_c X_c^T to the accuracy a refinement step needs
-// (jacobi_refine_ff_kernel follows), as a register-resident one-sided Jacobi.
+// (jacobi_refine_res_kernel follows), as a register-resident one-sided Jacobi.
 //
 // With a diagonally pivoted Cholesky factor G = L L^T, plane rotations of L's
 // columns until they are mutually orthogonal give L V = U diag(s) (Veselic &

@@ -274,16 +274,16 @@ inline JacobiReg jacobi_reg_all(int k, int64_t np) {  // every point of a single
 cudaError_t launch_jacobi_reg(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t nwarps,
                               int max_sweeps, float stop_cos, DevCounters *ctr, cudaStream_t s);
 
-// ---- Step 4: k-space estimator ----------------------------------------------
-// sigma/U from launch_jacobi, M pair-major from launch_patch_m3, R and Q from
-// launch_patch_gram (Q only for the Haar variant).  Writes kappa (np) and,
+// ---- Step 4: k-space estimator (randomised SVD) ------------------------------
+// For Ritz pairs (the randomised SVD): sigma/U from launch_rsvd_compose, M
+// pair-major from launch_patch_m3 or launch_moments_tc, R and Q from the Gram
+// pass (Q only for the Haar variant).  Writes kappa (np) and,
 // when not NULL, lambda_out (np x k) and the singular values s_out (np x k).
-// G (np x k x k, nullable): the patch Grams, given when U holds Ritz vectors
-// rather than eigenvectors of G (|X_c V_r|_F^2 is then computed as |G W|_F^2).
+// G (np x k x k): the patch Grams (|X_c V_r|_F^2 is computed as |G W|_F^2).
 cudaError_t launch_estimator(const float *sigma, const float *U, const float *M, const float *R,
                              const float *Q, int k, int64_t m, int64_t np, int variant, float rank_eps,
                              float *kappa, float *lambda_out, float *s_out, DevCounters *ctr,
-                             cudaStream_t s, const float *G = nullptr);
+                             cudaStream_t s, const float *G);
 
 // Numerical-rank thresholds (eigenvalues kept above eps * s_0):
 //  - a Gram accumulated in FP32 (or from BF16 products) carries rounding of
