@@ -308,33 +308,31 @@ def _stage_fracs(stages, steps, shapes, prec, rotations, peaks, elt=2):
     (CUDA events around every launch).  shapes: the (N, m, k) of every dataset
     of the step; the algorithmic work per stage is summed over them:
       knn_search  2 N^2 m FLOP (tensor, BF16; FP32 lanes in the plain form)
-      knn_rerank  N x 128 candidate rows x m x elt bytes read (2 lists of 64 per
-                  row from the tensor-core search), against HBM
+      knn_rerank  N x (k + 16) candidate rows x m x elt bytes read, against HBM
       gram        the gathered patches, N k m elements, against HBM
       rotate      the gathered patches plus the rotated patches written
                   (N x k rows x m BF16), against HBM
       moments     k(k+1)(k+2)/6 m multiply-adds per point (the distinct third
                   moments), x 2 FLOP (tensor, BF16)
-      jacobi      18 k FLOP per plane rotation (two-sided update of A and the
-                  eigenvector update; k weighted by the rotations a k x k patch
-                  takes, ~k^2: sum N k^3 / sum N k^2) + 8 k^3 per patch for the
-                  refinement's three products, against the FP32 lanes
-      estimator   k (2 k^2 p + k p (p + 1)) FLOP per point (B = M_j W and the
-                  upper triangle of W^T B), p = k - 1, against the FP32 lanes"""
+      jacobi      8 k FLOP per plane rotation (one-sided: the inner product of
+                  two columns and their rotation; k weighted by the rotations a
+                  k x k patch takes, ~k^2: sum N k^3 / sum N k^2) + 8 k^3 per
+                  patch for the refinement's products, against the FP32 lanes
+      estimator   plain form: the distinct third moments as above and the two
+                  rotations of the patch, 4 k^2 m FLOP, against the FP32 lanes"""
     bf = peaks.get("bf16_tflops_sustained", peaks.get("bf16_tflops"))
     hbm = peaks.get("hbm_gbs")
     tot = {key: 0.0 for key in ("knn_search", "knn_rerank", "gram", "rotate", "moments", "jacobi_ref", "estimator",
                                 "nk3", "nk2")}
     for N, m, k in shapes:
         N, m, k = float(N), float(m), float(k)
-        p = k - 1
         tot["knn_search"] += 2.0 * N * N * m
-        tot["knn_rerank"] += N * 128.0 * m * elt
+        tot["knn_rerank"] += N * (k + 16.0) * m * elt
         tot["gram"] += N * k * m * elt
         tot["rotate"] += N * k * m * elt + N * k * m * 2.0
         tot["moments"] += 2.0 * k * (k + 1) * (k + 2) / 6.0 * m * N
         tot["jacobi_ref"] += 8.0 * k ** 3 * N
-        tot["estimator"] += k * (2.0 * k * k * p + k * p * (p + 1)) * N
+        tot["estimator"] += (k * (k + 1) * (k + 2) / 3.0 + 4.0 * k * k) * m * N
         tot["nk3"] += N * k ** 3
         tot["nk2"] += N * k ** 2
     kw = tot["nk3"] / tot["nk2"]
@@ -344,7 +342,7 @@ def _stage_fracs(stages, steps, shapes, prec, rotations, peaks, elt=2):
         "gram": (tot["gram"], "hbm"),
         "rotate": (tot["rotate"], "hbm"),
         "moments": (tot["moments"], "tensor"),
-        "jacobi": (18.0 * kw * rotations + tot["jacobi_ref"], "alu"),
+        "jacobi": (8.0 * kw * rotations + tot["jacobi_ref"], "alu"),
         "estimator": (tot["estimator"], "alu"),
     }
     out = {}
@@ -462,8 +460,8 @@ def run_ours(args):
                     "share_of_step": knn_ms / elapsed_ms}
 
     jac = args.jacobi_fp64 if args.jacobi_fp64 is not None else (1 if prec == "bf16_mixed" else 0)
-    jac_desc = {0: "FP32 sweeps", 1: "FP32 sweeps (to 2^-14), then one Ogita-Aishima refinement step with "
-                                     "two-term-FP32 products (~2^-48)",
+    jac_desc = {0: "FP32 sweeps", 1: "one-sided FP32 sweeps on the Cholesky factor, then one Ogita-Aishima "
+                                     "refinement step through the residual (two-term-FP32 products)",
                 2: "every sweep in FP64"}[jac]
     line = {"metric": METRIC, "value": value, "unit": "points/s", "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
@@ -507,7 +505,7 @@ def run_ours(args):
         plain = {"idx": idx_p.cpu().numpy(), "kappa": kap_p.cpu().numpy()}
         line["plain_fp32"] = {"value": S / (pms * 1e-3), "unit": "points/s",
                               "sample": f"query rows [0,{S}) of the same workload against all {N} points, "
-                                        f"kNN + estimator in plain FP32 (FP32 search, FP64 centring, rotated "
+                                        f"kNN + estimator in plain FP32 (FP32 search, two-term centring, rotated "
                                         f"patch, FP32 Jacobi + two-term-FP32 refinement); {pms:.0f} ms",
                               "chosen_over_plain": value / world / (S / (pms * 1e-3)),
                               "knn_simt_roofline": {"bound": "alu", "achieved": p_ach, "peak": FP32_PEAK_TFLOPS,
@@ -589,7 +587,8 @@ STAGE_KERNELS = {
     "knn_search": "knn_tc_kernel (distance GEMM + fused candidate select)",
     "knn_rerank": "knn_rerank_kernel", "gram": "gram_tc_kernel", "rotate": "rotate_tc_kernel",
     "moments": "tthird_tc_kernel (third moments of the rotated patch + estimator)",
-    "jacobi": "jacobi_kernel + jacobi_refine_ff_kernel", "estimator": "estimator_kernel",
+    "jacobi": "jacobi_reg_kernel + jacobi_warp_kernel + jacobi_refine_res_kernel",
+    "estimator": "patch_m3_kernel (third moments + estimator)",
 }
 
 
