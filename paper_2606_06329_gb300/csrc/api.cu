@@ -308,13 +308,12 @@ KnnPlan plan_knn(mecuco_t h, const void *X, mecuco_dtype dt, int64_t N, int64_t 
     // so that its items fill the SMs again (62,500 rows against 1M points: 3.25
     // instead of 4 waves).  A split shortens the search but gives every row
     // another set of lists to re-rank; the model weighs the two, in ns.  A wave
-    // costs, per candidate tile, max(4000, 7.5 K) on the tensor cores (256 rows;
-    // the drain, or the operands' way from L2) and 2500 + 75 m on the CUDA cores
-    // (128 rows); a row's set of lists 3 per 128 entries in the re-rank (reading
+    // costs, per tile of 256 candidates, max(4000, 7.5 K) on the tensor cores (the
+    // drain, or the operands' way from L2) and 4500 + 122 m on the CUDA cores; a row's set of lists 3 per 128 entries in the re-rank (reading
     // and selecting: it evaluates k + 16 candidates however many there are).
-    const double tile = p.tc ? std::max(4000.0, 7.5 * (double)p.mk) : 2500.0 + 75.0 * (double)m;
-    const int64_t tile_rows = p.tc ? 256 : 128, item_rows = p.tc ? knn_tc_item_rows(p.pair) : 128;
-    const double waves1 = (double)((N + tile_rows - 1) / tile_rows) * tile, rr = 3.0 * p.halves * p.kcl / 128;
+    const double tile = p.tc ? std::max(4000.0, 7.5 * (double)p.mk) : 4500.0 + 122.0 * (double)m;
+    const int64_t item_rows = p.tc ? knn_tc_item_rows(p.pair) : 128;
+    const double waves1 = (double)((N + 255) / 256) * tile, rr = 3.0 * p.halves * p.kcl / 128;
     for (int64_t left = nrows; left > 0;) {
         const int64_t take = left >= wave ? std::min(p.qchunk, left / wave * wave) : left;
         int best = 1;
