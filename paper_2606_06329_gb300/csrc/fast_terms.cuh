@@ -45,58 +45,86 @@ __device__ __forceinline__ int fast_rank(const float *__restrict__ sg, int k, in
 // T^[(r,r), l] (r < p, l < k); Us, Qs: U and Q of the point in shared memory (Q for
 // the Haar variant only), R and the eigenvalues sg in global memory; c_s (64) and
 // red (a row per warp): scratch in shared memory.  Called by all THREADS threads (k <=
-// 64 <= THREADS, or k <= 32 and THREADS >= 64), Us, Qs and diag visible to all.
+// 64 <= THREADS), Us, Qs and diag visible to all.
 // The sums are two-term FP32 (2^-44 and better): FP64 runs at 1/64 of the FP32
-// rate, and a few dozen double operations per warp cost narrow sets as much as
-// their third moments.
+// rate.  A CTA has nothing else to do meanwhile, so what counts is the length of
+// the dependent chains: the sums of squares and the k quadratic forms of Q are
+// spread over all threads, eight lanes to a form, and the two reciprocals in FP64
+// are computed beside them (one thread per form: 44,000 of the 95,000 cycles that a
+// point of 301 columns took at k = 37, Haar; 30,000 points 5.0 -> 3.8 ms).
 template <int THREADS>
 __device__ __forceinline__ void fast_kappa(int k, int p, int64_t m, int variant, ff gsum,
                                            const float *__restrict__ sg, const float *__restrict__ R,
                                            const float *diag, int ldd, const float *Us, int ldu, const float *Qs,
                                            int ldq, float *c_s, float2 (*red)[5], float *__restrict__ kappa) {
-    constexpr int NW = THREADS / 32, HW = THREADS >= 128 ? 64 : 32, AW = NW < 4 ? NW : 4;
+    constexpr int NW = THREADS / 32;
+    __shared__ double recip[2];  // 1 / (k - 1); 1 / q, or 1 / (q + 2) for the Haar variant (0 for q = 0)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    gsum = sum_warp(gsum);
+    const int64_t q = m - p;
+    if (tid == THREADS - 1) {
+        recip[0] = 1.0 / (double)(k - 1);
+        recip[1] = q > 0 ? 1.0 / (double)(variant == MECUCO_FAST_HAAR ? q + 2 : q) : 0.0;
+    }
     ff dsum{0.f, 0.f}, xa2{0.f, 0.f}, hsum{0.f, 0.f}, tsum{0.f, 0.f};
     if (tid < k) {
-        // c_l = sum_{r<p} T^[(r,r), l] and t_range's sum, in a fixed order over r
+        // c_l = sum_{r<p} T^[(r,r), l], r ascending
         const int l = tid;
         float cl = 0.f;
-        for (int r = 0; r < p; ++r) {
-            const float v = diag[r * ldd + l];
-            cl += v;
-            dsum = sum_add(dsum, sum_mul(v, v));
-        }
+#pragma unroll 8
+        for (int r = 0; r < p; ++r) cl += diag[r * ldd + l];
         c_s[l] = cl;
         if (l < p) tsum.hi = sg[l];
     }
-    if (variant == MECUCO_FAST_HAAR && tid >= HW && tid < HW + p) {
-        // u_l^T Q u_l / s_l^2
-        const int l = tid - HW;
-        ff acc{0.f, 0.f};
-        for (int a = 0; a < k; ++a) {
-            float qu = 0.f;
-            for (int b = 0; b < k; ++b) qu = fmaf(Qs[a * ldq + b], Us[b * ldu + l], qu);
-            acc = sum_add(acc, sum_mul(Us[a * ldu + l], qu));
+    // t_range's sum: rows of T^[(r,r), .] by warp
+    for (int r = warp; r < p; r += NW)
+        for (int l = lane; l < k; l += 32) {
+            const float v = diag[r * ldd + l];
+            dsum = sum_add(dsum, sum_mul(v, v));
         }
-        const float s = sg[l], q1 = acc.hi / s;
-        hsum = ff{q1, finite_err(q1, (fmaf(-q1, s, acc.hi) + acc.lo) / s)};
+    if (variant == MECUCO_FAST_HAAR) {
+        // u_l^T Q u_l / s_l^2: eight lanes per l, lane g rows g, g + 8, ... of Q
+        const int g = lane & 7;
+        for (int l0 = 0; l0 < p; l0 += THREADS / 8) {
+            const int l = l0 + (tid >> 3), lc = l < p ? l : 0;
+            float qu[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) qu[i] = 0.f;
+            const int na = (k + 7) / 8;
+            for (int b = 0; b < k; ++b) {
+                const float u = Us[b * ldu + lc];
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (i < na) qu[i] = fmaf(Qs[min(g + 8 * i, k - 1) * ldq + b], u, qu[i]);
+            }
+            ff acc{0.f, 0.f};
+#pragma unroll
+            for (int i = 0; i < 8; ++i)
+                if (g + 8 * i < k) acc = sum_add(acc, sum_mul(Us[(g + 8 * i) * ldu + lc], qu[i]));
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) acc = sum_add(acc, ff_shfl_xor(acc, o));
+            if (g == 0 && l < p) {
+                const float s = sg[l], q1 = acc.hi / s;
+                hsum = sum_add(hsum, ff{q1, finite_err(q1, (fmaf(-q1, s, acc.hi) + acc.lo) / s)});
+            }
+        }
     }
     __syncthreads();
     if (tid < k) {
         // X_c d_P = R - U c
         const int j = tid;
         float uc = 0.f;
+#pragma unroll 8
         for (int l = 0; l < k; ++l) uc = fmaf(Us[j * ldu + l], c_s[l], uc);
         float h, e;
         two_sum(R[j], -uc, h, e);
         xa2 = sum_mul(h, h);
         xa2.lo = finite_err(xa2.hi, xa2.lo + 2.f * h * e);
     }
-    if (warp < AW) {  // the threads that hold any of these
-        dsum = sum_warp(dsum);
+    gsum = sum_warp(gsum);
+    dsum = sum_warp(dsum);
+    if (variant == MECUCO_FAST_HAAR) hsum = sum_warp(hsum);
+    if (warp < 2) {  // the threads that hold any of these
         xa2 = sum_warp(xa2);
-        hsum = sum_warp(hsum);
         tsum = sum_warp(tsum);
     }
     if (lane == 0) {
@@ -112,25 +140,20 @@ __device__ __forceinline__ void fast_kappa(int k, int p, int64_t m, int variant,
         ff t[5];
 #pragma unroll
         for (int c = 0; c < 5; ++c) {
-            const float2 v = lane < NW && (c == 0 || lane < AW) ? red[lane][c] : make_float2(0.f, 0.f);
+            const float2 v = lane < NW ? red[lane][c] : make_float2(0.f, 0.f);
             t[c] = sum_warp(ff{v.x, v.y});
         }
         if (lane == 0) {
-            const double ik = 1.0 / (double)(k - 1);
+            const double ik = recip[0];
             const double gt2 = (double)t[0].hi + (double)t[0].lo, d2 = (double)t[1].hi + (double)t[1].lo;
             const double a2 = (double)t[2].hi + (double)t[2].lo, h = (double)t[3].hi + (double)t[3].lo;
             const double tau = ((double)t[4].hi + (double)t[4].lo) * ik;
             const double t_range = d2 * ik, t_A = a2 * ik;
-            const int64_t q = m - p;
             double t_null = 0.0;
             if (q > 0) {
-                if (variant == MECUCO_FAST_HAAR) {
-                    const double tB = tau + (gt2 - 2.0 * h) * ik;
-                    t_null = (t_A + 2.0 * tB) / (double)(q + 2);
-                } else {
-                    const double tB = gt2 * ik - tau;  // |X_c V_r|_F^2 / (k-1) = tau
-                    t_null = (t_A + 2.0 * tB) / (double)q;
-                }
+                // |X_c V_r|_F^2 / (k-1) = tau in the literal form
+                const double tB = variant == MECUCO_FAST_HAAR ? tau + (gt2 - 2.0 * h) * ik : gt2 * ik - tau;
+                t_null = (t_A + 2.0 * tB) * recip[1];
             }
             *kappa = (float)fabs(0.5 * (t_range + t_null) + 0.5 * tau);
         }

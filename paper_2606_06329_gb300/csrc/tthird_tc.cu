@@ -24,7 +24,7 @@
 // = 64, 9 instead of 15 at 37, 6 instead of 10 at 32.  Measured with every pair and
 // with the split: 11.3 and 6.7 ms for 6,144 patches of 4,096 columns at k = 64, 114
 // and 67 for 62,500, 6.5 and 5.8 for 30,000 of 301 at k = 37 (5.0 with the sums of
-// the epilogue in two-term FP32 instead of FP64).
+// the epilogue in two-term FP32 instead of FP64, 3.8 with them spread over the CTA).
 // Sets below TT_SPLIT_MIN_M columns form every pair: there |G_tens|^2 is divided
 // by a small m - p, and the BF16 roundings of the products, which differ between
 // the two tables, would show in kappa.
