@@ -451,7 +451,12 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
         volatile int *update_flag = &sh->update;
         int updates = 0;  // list updates made so far
         int t = 0;  // tiles drained so far by this CTA (all items)
-        for (int64_t item = first; item < nitems && !*abort_flag; item += stride) {
+        // The loops below hold warp-wide votes, reductions and tensor-memory loads, so
+        // a warp leaves them as one: a lane's own reading of the abort flag, or its own
+        // wait running out, is voted on before any lane acts on it.
+        auto aborted = [&]() { return __any_sync(0xffffffffu, *abort_flag != 0) != 0; };
+        bool ok = true;
+        for (int64_t item = first; item < nitems && ok && !aborted(); item += stride) {
             const ItemGeo g = geo(item);
             const int64_t qb = g.qb + (int64_t)rank * TBM;
             const int64_t cbeg = g.cbeg, cend = g.cend;
@@ -496,16 +501,24 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                 }
                 np = 0;
             };
-            for (int tt = 0; tt < ntiles && !*abort_flag; ++tt, ++t) {
+            for (int tt = 0; tt < ntiles; ++tt, ++t) {
+                if (aborted()) {
+                    ok = false;
+                    break;
+                }
                 const int acc = t & 1;
                 const int asked = *update_flag;
                 if (__any_sync(0xffffffffu, asked != updates)) {
                     updates = __reduce_max_sync(0xffffffffu, asked);
                     flush();
                 }
-                if (!tc::mbar_wait(tc::smem_u32(&sh->tfull[acc]), (t >> 1) & 1, abort_flag, wait_limit)) {
-                    atomicOr(&ctr->status, (unsigned)DEV_TIMEOUT);
-                    sh->abort = 1;
+                ok = __all_sync(0xffffffffu, tc::mbar_wait(tc::smem_u32(&sh->tfull[acc]), (t >> 1) & 1, abort_flag,
+                                                           wait_limit));
+                if (!ok) {
+                    if (lane == 0) {
+                        atomicOr(&ctr->status, (unsigned)DEV_TIMEOUT);
+                        sh->abort = 1;
+                    }
                     break;
                 }
                 tc::fence_after();
@@ -577,7 +590,7 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
                     tc::mbar_arrive(tc::smem_u32(&sh->tempty[acc]));
                 }
             }
-            flush();
+            if (ok) flush();  // after a timeout the lists are invalid
             if (valid_row) {
                 for (int p = 0; p < st.cnt; ++p) g.cand_d[out_base + Ls[p * TBM + row]] = Ld[p * TBM + row];
                 for (int s2 = st.cnt; s2 < kc; ++s2) {
