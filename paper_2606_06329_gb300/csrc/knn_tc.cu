@@ -28,9 +28,15 @@
 // admitted), 12.1 ms with the tail wave split.  Listing the pending candidates by
 // warp-wide bitonic merges into sorted lists instead of per-lane heaps took
 // 34 ms (a warp's 32 rows one after the other; two at a time).
-// K blocks run forward on even candidate tiles and backward on odd ones: DRAM
-// reads per search fall by a third (133 to 89 GB for 19,456 queries against
-// 210,000 points of 4,096), the search by 4%.
+// K blocks run in ascending order on every candidate tile.  The tensor core's
+// accumulator truncates, so d~ is too large by an error that grows with the partial
+// sums; it is much the same for all near candidates of a row, and what is common to
+// them cancels in the re-rank's certificate, which estimates the error from the row's
+// own candidates.  Running the blocks backward on every second tile reads a third
+// less from DRAM (89 against 133 GB for 19,456 queries and 210,000 points of 4,096;
+// 4% of the search) but leaves two errors per row, by the parity of the candidate's
+// tile: on clusters off the origin (2,048 BF16 rows of 4,096 columns, noise 1 to 2% of
+// the centre) up to 2,048 of 2,048 rows came out certified and wrong.
 // CTA pairs (optional, for 256 or more query rows): two CTAs of a
 // thread-block cluster share one 256 x 256 tcgen05.mma (cta_group::2, M = 256)
 // per K step.  Each CTA loads its own 128 query rows and one 128-row half of
@@ -332,23 +338,21 @@ knn_tc_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__
             }
             for (int t = 0; t < g.ntiles && ok && !*abort_flag; ++t) {
                 const int c0 = (int)(g.cbeg + (int64_t)t * TBN) + (int)rank * C::B_ROWS;
-                // K blocks forward on even tiles, backward on odd ones: the CTAs'
-                // query slices together exceed L2, and a cyclic sweep would miss on
-                // every block; turning round finds the last ones still cached
-                int x = t & 1 ? (g.nkb - 1) * TBK : 0;
-                const int dx = t & 1 ? -TBK : TBK;
-                for (int kb = 0; kb < g.nkb; ++kb, ++it, x += dx) {
+                // K blocks in ascending order on every tile: the accumulator truncates,
+                // and only an error that is alike for all candidates of a row cancels in
+                // the certificate (see the file's head)
+                for (int kb = 0; kb < g.nkb; ++kb, ++it) {
                     if (!tc::mbar_wait(empty0 + 8 * s, ph ^ 1u, abort_flag, wait_limit)) { ok = false; break; }
                     const uint32_t sa = st0 + s * (uint32_t)STAGE;
                     if constexpr (PAIR) {
                         if (rank == 0) tc::mbar_expect_tx(full0 + 8 * s, 2 * STAGE);
-                        tc::tma_load_2d_pair(sa, map_q, pfull0 + 8 * s, x, (int)qb);
-                        tc::tma_load_2d_pair(sa + A_BYTES, map_c, pfull0 + 8 * s, x, c0);
+                        tc::tma_load_2d_pair(sa, map_q, pfull0 + 8 * s, kb * TBK, (int)qb);
+                        tc::tma_load_2d_pair(sa + A_BYTES, map_c, pfull0 + 8 * s, kb * TBK, c0);
                     } else {
                         const uint32_t fb = full0 + 8 * s;
                         tc::mbar_expect_tx(fb, STAGE);
-                        tc::tma_load_2d(sa, map_q, fb, x, (int)qb);
-                        tc::tma_load_2d(sa + A_BYTES, map_c, fb, x, c0);
+                        tc::tma_load_2d(sa, map_q, fb, kb * TBK, (int)qb);
+                        tc::tma_load_2d(sa + A_BYTES, map_c, fb, kb * TBK, c0);
                     }
                     if (++s == (uint32_t)NST) { s = 0; ph ^= 1u; }
                 }
