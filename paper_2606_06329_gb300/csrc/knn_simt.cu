@@ -759,52 +759,49 @@ knn_rerank_kernel(const T *__restrict__ X_, int64_t N_, int64_t m_, int64_t ld_,
     }
 
     float err_max = -INFINITY, err_min = INFINITY, nmax = 0.f;
-    int n = 0;                 // evaluated candidates held (eh, el, ei)
-    unsigned done = 0u;        // candidates with key < done have been evaluated (every key is > 0)
-    unsigned want_key = 0u;    // and those below this one are to be (exclusive)
-    int want = min(live, k + RR_EXTRA);
+    int n = 0;            // evaluated candidates held (eh, el, ei)
     float theta = INFINITY, e_hi = INFINITY;
-    auto count_below = [&](unsigned t) {  // live candidates with done <= key < t
+    const unsigned kend = min(kmax, 0xfffffffeu) + 1u;  // past every key
+    auto count_below = [&](unsigned t) {  // candidates not evaluated yet with key < t
         int c = 0;
-        for (int i = lane; i < L; i += 32) c += ci[i] >= 0 && key[i] >= done && key[i] < t;
+        for (int i = lane; i < L; i += 32) c += ci[i] >= 0 && key[i] < t;
         return (int)__reduce_add_sync(FULL, c);
     };
-    // smallest t (to a few candidates) with count_below(t) >= w, at most room
-    auto key_for = [&](unsigned lo, unsigned hi, int w, int room) {
-        // invariant: count_below(lo) < w <= count_below(hi)
-        while (hi - lo > 1u) {
-            const unsigned mid = lo + (hi - lo) / 2u;
+    // first the k + RR_EXTRA smallest: a key with that many candidates below it (to a
+    // few), by bisection; count_below(lo) < want <= count_below(hi)
+    unsigned want_key = kend;
+    if (const int want = min(live, k + RR_EXTRA); want > 0) {
+        unsigned lo = kmin;
+        while (want_key - lo > 1u) {
+            const unsigned mid = lo + (want_key - lo) / 2u;
             const int c = count_below(mid);
-            if (c >= w) {
-                hi = mid;
-                if (c <= w + 4 && c <= room) break;
+            if (c >= want) {
+                want_key = mid;
+                if (c <= want + 4) break;
             } else {
                 lo = mid;
             }
         }
-        return hi;
-    };
-    for (;;) {
-        // ---- the next candidates: [done, want_key), as many as there is room for
-        if (n == 0) {
-            if (want <= 0) break;
-            want_key = key_for(kmin, kmax + 1u, want, RR_CAP);
-        }
+    }
+    while (live > 0) {
+        // ---- the next candidates: those below want_key, as many as there is room for
+        // (the rest, equal keys for instance, in the passes that follow); an evaluated
+        // one leaves the list
         const int room = RR_CAP - n;
-        const int cnt = count_below(want_key);
-        if (cnt > room) want_key = key_for(max(done, kmin), want_key, max(1, room - 4), room);
-        // (equal keys beyond the room cannot be told apart: give up, full scan)
         int nb = 0;
-        for (int i0 = 0; i0 < L; i0 += 32) {
+        for (int i0 = 0; i0 < L && nb < room; i0 += 32) {
             const int i = i0 + lane;
-            const bool take = i < L && ci[i] >= 0 && key[i] >= done && key[i] < want_key;
+            const bool take = i < L && ci[i] >= 0 && key[i] < want_key;
             const unsigned mk = __ballot_sync(FULL, take);
-            const int pos = n + nb + __popc(mk & ((1u << lane) - 1u));
-            if (take && pos < RR_CAP) ec[pos] = i;
+            const int pos = nb + __popc(mk & ((1u << lane) - 1u));
+            if (take && pos < room) {
+                ec[n + pos] = i;
+                ei[n + pos] = ci[i];
+                ci[i] = -1;
+            }
             nb += __popc(mk);
         }
-        const bool overflow = n + nb > RR_CAP;
-        if (overflow) nb = RR_CAP - n;
+        nb = min(nb, room);
         __syncwarp();
         // ---- their exact distances
         for (int c0 = n; c0 < n + nb; c0 += 4 * per) {
@@ -814,9 +811,9 @@ knn_rerank_kernel(const T *__restrict__ X_, int64_t N_, int64_t m_, int64_t ld_,
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 cc[u] = c0 + u * per + gid;
-                const int i = cc[u] < n + nb ? ec[cc[u]] : -1;
-                j[u] = i >= 0 ? ci[i] : -1;
-                dt[u] = i >= 0 ? cd[i] : 0.f;
+                const bool in = cc[u] < n + nb;
+                j[u] = in ? ei[cc[u]] : -1;
+                dt[u] = in ? cd[ec[cc[u]]] : 0.f;
                 // 2^b above twice the search's distance
                 base[u] = __uint_as_float(min((__float_as_uint(fabsf(dt[u])) & 0x7f800000u) + (2u << 23), 0x7e800000u));
             }
@@ -831,12 +828,10 @@ knn_rerank_kernel(const T *__restrict__ X_, int64_t N_, int64_t m_, int64_t ld_,
                     if ((lane & (G - 1)) == 0) {
                         eh[cc[u]] = d[u].hi;
                         el[cc[u]] = d[u].lo;
-                        ei[cc[u]] = j[u];
                     }
                 }
         }
         n += nb;
-        done = want_key;
         __syncwarp();
         err_max = warp_max(err_max);
         err_min = -warp_max(-err_min);
@@ -869,14 +864,10 @@ knn_rerank_kernel(const T *__restrict__ X_, int64_t N_, int64_t m_, int64_t ld_,
         __syncwarp();
         n = min(n, k);
         theta = n == k ? eh[k - 1] : INFINITY;
-        if (overflow) {
-            thr = -INFINITY;
-            break;
-        }
         // ---- candidates left that could still enter: d~ <= theta + e_hi
         const float lim = theta + e_hi;
-        want_key = lim < INFINITY ? min(order_key(lim) + 1u, kmax + 1u) : kmax + 1u;
-        if (want_key <= done || count_below(want_key) == 0) break;
+        want_key = lim < INFINITY ? min(order_key(lim) + 1u, kend) : kend;
+        if (count_below(want_key) == 0) break;
     }
     for (int c = lane; c < n; c += 32) {
         idx_out[qi * k + c] = ei[c];
