@@ -514,16 +514,21 @@ cudaError_t launch_knn_simt(const void *X, mecuco_dtype dt, int64_t N, int64_t m
 // not evaluated here - has d~ >= some threshold thr, so its true distance is >=
 // thr - e_hi, e_hi bounding the overestimate d~ - d; it cannot enter the top k
 // when thr - e_hi exceeds the exact k-th distance theta.  The search's
-// accumulation error has no documented worst-case bound on the tensor-core
-// path and is dominated by a per-row bias (the FP32 accumulator's rounding of
-// partial sums of similar size), so e_hi is estimated a posteriori from the
-// row's own evaluated candidates: the largest observed d~ - d plus 3x the
-// observed spread of d~ - d, plus 2^-21 (|x|^2 + max |y|^2) (a few units in the
-// last place of the norms); FP32 rows searched in BF16 add the rounding's
-// a-priori bound.
+// accumulation error has no useful worst-case bound and is dominated by a part that
+// the near candidates of a row have in common (the FP32 accumulator's truncation of
+// partial sums of similar size, in one order of the columns), so e_hi is estimated a
+// posteriori from the row's own evaluated candidates: the largest observed d~ - d
+// plus 3x the observed spread of d~ - d, plus 2^-21 (|x|^2 + |y|^2) (a few units in
+// the last place of the norms, |y| the largest evaluated or that of a point at
+// theta); FP32 rows searched in BF16 add the rounding's a-priori bound.
 // The lists hold two to three times as many candidates as neighbours asked for,
 // so a row first evaluates the k + RR_EXTRA smallest by d~ (a threshold found by
-// bisection), and then only those with d~ <= theta + e_hi, usually none.  Rows
+// bisection) and RR_SAMPLE others, and then only those with d~ <= theta + e_hi,
+// usually none.  The others are taken at equal steps through the lists, whose order
+// does not follow d~, with the largest d~ among them: the smallest d~ are those that
+// the search underestimates most, and where they are copies of one point they show
+// the error of that point alone (of 2,400 FP32 rows of 4,096 columns with 23 copies in
+// each cluster, up to 16 came out certified and wrong without the sample).  Rows
 // whose lists' own threshold (the smallest maximum of the full lists) does not
 // pass the test are re-solved exactly by the full scan.
 // Measured per 100k queries against the form that evaluated and ranked every
@@ -536,7 +541,8 @@ cudaError_t launch_knn_simt(const void *X, mecuco_dtype dt, int64_t N, int64_t m
 constexpr int RR_WARPS = 4;
 constexpr int RR_MAXL = 1024;
 constexpr int RR_EXTRA = 16;
-constexpr int RR_CAP = 128;  // evaluated candidates kept at a time (>= 64 + RR_EXTRA + slack, a multiple of 32)
+constexpr int RR_SAMPLE = 16;
+constexpr int RR_CAP = 128;  // evaluated candidates kept at a time (>= 64 + RR_EXTRA + RR_SAMPLE + slack, a multiple of 32)
 
 namespace {
 // 16 bytes of a row as packed FP32 pairs
@@ -783,15 +789,25 @@ knn_rerank_kernel(const T *__restrict__ X_, int64_t N_, int64_t m_, int64_t ld_,
             }
         }
     }
+    // and, in the same pass, RR_SAMPLE candidates spread over the lists and the largest
+    // d~ of all: the sample that the error estimate needs besides the nearest
+    int every = (live + RR_SAMPLE - 1) / RR_SAMPLE;  // 0: no sample (the later passes)
     while (live > 0) {
         // ---- the next candidates: those below want_key, as many as there is room for
         // (the rest, equal keys for instance, in the passes that follow); an evaluated
         // one leaves the list
         const int room = RR_CAP - n;
-        int nb = 0;
+        int nb = 0, seen = 0;
         for (int i0 = 0; i0 < L && nb < room; i0 += 32) {
             const int i = i0 + lane;
-            const bool take = i < L && ci[i] >= 0 && key[i] < want_key;
+            const bool in = i < L && ci[i] >= 0;
+            bool take = in && key[i] < want_key;
+            if (every) {
+                const unsigned am = __ballot_sync(FULL, in);
+                const int ord = seen + __popc(am & ((1u << lane) - 1u));
+                take = take || (in && (ord % every == 0 || key[i] == kmax));
+                seen += __popc(am);
+            }
             const unsigned mk = __ballot_sync(FULL, take);
             const int pos = nb + __popc(mk & ((1u << lane) - 1u));
             if (take && pos < room) {
@@ -802,6 +818,7 @@ knn_rerank_kernel(const T *__restrict__ X_, int64_t N_, int64_t m_, int64_t ld_,
             nb += __popc(mk);
         }
         nb = min(nb, room);
+        every = 0;
         __syncwarp();
         // ---- their exact distances
         for (int c0 = n; c0 < n + nb; c0 += 4 * per) {
@@ -836,7 +853,6 @@ knn_rerank_kernel(const T *__restrict__ X_, int64_t N_, int64_t m_, int64_t ld_,
         err_max = warp_max(err_max);
         err_min = -warp_max(-err_min);
         nmax = warp_max(nmax);
-        e_hi = fmaxf(fmaxf(err_max, 0.f) + 3.f * (err_max - err_min) + ldexpf(nq_ + nmax, -21), e_apriori);
         // ---- the k best of the evaluated ones, in order, to the front
         float vh[RR_CAP / 32], vl[RR_CAP / 32];
         int vi[RR_CAP / 32], vr[RR_CAP / 32];
@@ -864,6 +880,10 @@ knn_rerank_kernel(const T *__restrict__ X_, int64_t N_, int64_t m_, int64_t ld_,
         __syncwarp();
         n = min(n, k);
         theta = n == k ? eh[k - 1] : INFINITY;
+        // a point within theta has a norm of at most |x| + sqrt(theta)
+        const float yn = sqrtf(nq_) + sqrtf(fmaxf(theta, 0.f));
+        e_hi = fmaxf(fmaxf(err_max, 0.f) + 3.f * (err_max - err_min) + ldexpf(nq_ + fmaxf(nmax, yn * yn), -21),
+                     e_apriori);
         // ---- candidates left that could still enter: d~ <= theta + e_hi
         const float lim = theta + e_hi;
         want_key = lim < INFINITY ? min(order_key(lim) + 1u, kend) : kend;
