@@ -508,8 +508,9 @@ cudaError_t launch_knn_simt(const void *X, mecuco_dtype dt, int64_t N, int64_t m
 // ---------------------------------------------------------------------------
 // Exact re-rank + certification.  One warp per query row.  An exact distance is
 // sum_a (x_a - y_a)^2 as a float-float pair: the difference by TwoSum, its
-// square added to a two-term sum by FMAs, so it carries ~2^-42 relative error:
-// ranks agree with an FP64 brute force except at ties closer than that.
+// square added to a two-term sum by FMAs, whose offset is kept within 8 times the
+// distance, so it carries ~2^-42 relative error: ranks agree with an FP64 brute force
+// except at ties closer than that.
 // Certification: a point left out - rejected by a list, or a candidate that is
 // not evaluated here - has d~ >= some threshold thr, so its true distance is >=
 // thr - e_hi, e_hi bounding the overestimate d~ - d; it cannot enter the top k
@@ -583,10 +584,25 @@ __device__ __forceinline__ unsigned order_key(float v) {
 }
 }  // namespace
 
+// Exact distance of rows xq and y over the G lanes of a group, renormalising every
+// term (no offset).  All groups of the warp together; not inlined, so that the usual
+// case keeps its registers (a second pass with a better offset inside exact_dist4 made
+// 100,000 x 512 take 16.5 ms instead of 15.3 without ever running).
+template <typename T>
+__device__ __noinline__ ff exact_dist_renorm(const T *__restrict__ xq, const T *__restrict__ y, int64_t m, int G) {
+    ff s{0.f, 0.f};
+    for (int64_t a = (threadIdx.x & 31) & (G - 1); a < m; a += G)
+        ff_acc_sqdiff(s, load_elem(xq + a), load_elem(y + a));
+    for (int o = G >> 1; o > 0; o >>= 1) s = ff_add(s, ff_shfl_xor(s, o));
+    return s;
+}
+
 // Exact distances of the candidates j[u] (u < 4; -1: none) from row q, one per
 // group of G lanes and u, returned in every lane of the group.  base[u]: the
-// offset, a power of two above the distance (checked: a sum that reaches it is
-// done again without).
+// offset, a power of two above twice the search's distance.  Where it proves too
+// small (a partial sum reaches it), or more than 8 times the distance (the low word
+// would hold, rounded to FP32, what hi cannot: points far closer than the search
+// resolves), the sum is formed again without an offset.
 template <typename T>
 __device__ __forceinline__ void exact_dist4(const T *__restrict__ X, int64_t m, int64_t ld, const T *__restrict__ xq,
                                             int64_t q, const int (&j)[4], const float (&base)[4], int G, bool vec,
@@ -627,29 +643,29 @@ __device__ __forceinline__ void exact_dist4(const T *__restrict__ X, int64_t m, 
 #pragma unroll
         for (int u = 0; u < 4; ++u) acc_sqdiff2(acc[u], pack2(x, 0.f), pack2(load_elem(xr[u] + a), 0.f), minus, two);
     }
-    bool over = false;
+    unsigned bad = 0u;
 #pragma unroll
     for (int u = 0; u < 4; ++u) {
         const float2 h = unpack2(acc[u].hi), l = unpack2(acc[u].lo);
-        over = over || !(h.x < 2.f * base[u]) || !(h.y < 2.f * base[u]);
+        if (!(h.x < 2.f * base[u]) || !(h.y < 2.f * base[u])) bad |= 1u << u;
         // two sums of a lane, then the group's: renormalised float-float additions
         ff s, e;
         two_sum(h.x - base[u], l.x, s.hi, s.lo);
         two_sum(h.y - base[u], l.y, e.hi, e.lo);
         out[u] = ff_add(s, e);
     }
-    if (__any_sync(0xffffffffu, over)) {
-        // a sum outgrew its offset (the search's distance was far too small):
-        // without one, renormalising every term
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-            out[u] = ff{0.f, 0.f};
-            for (int64_t a = gl; a < m; a += G) ff_acc_sqdiff(out[u], load_elem(xq + a), load_elem(xr[u] + a));
-        }
-    }
     for (int o = G >> 1; o > 0; o >>= 1)
 #pragma unroll
         for (int u = 0; u < 4; ++u) out[u] = ff_add(out[u], ff_shfl_xor(out[u], o));
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (8.f * out[u].hi < base[u] && out[u].hi != 0.f && j[u] >= 0) bad |= 1u << u;
+    bad = __reduce_or_sync(0xffffffffu, bad);  // any group's: the renormalised form is never less accurate
+    if (bad) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            if ((bad >> u) & 1u) out[u] = exact_dist_renorm<T>(xq, xr[u], m, G);
+    }
 }
 
 template <typename T, bool BATCH>
