@@ -132,6 +132,20 @@ __device__ __forceinline__ void atomic_max_u64(unsigned long long *p, unsigned l
     atomicMax(p, v);
 }
 
+// Order of eigenpairs: descending, the lower index first on ties, NaN last.  A total
+// order, so that counting the pairs before gives every pair a place of its own also
+// where the patch was not finite.
+template <typename Real>
+__device__ __forceinline__ bool pair_before(Real a, int ia, Real b, int ib) {
+    return a > b || (a == b && ia < ib) || (b != b && (a == a || ia < ib));
+}
+// max(v, 0), NaN kept
+__device__ __forceinline__ float pos_part(float v) { return v > 0.f || v != v ? v : 0.f; }
+// lambda_l from s_l^2: zero past the rank p; NaN kept
+__device__ __forceinline__ float lambda_of(float sg, int l, int p, int k) {
+    return l < p || sg != sg ? pos_part(sg) / (float)(k - 1) : 0.f;
+}
+
 // ---- rotation of a patch chunk by a per-point orthogonal k x k matrix U0 ----
 // Us[r][l] = U0[r][l] for r, l < k, zero elsewhere (all 64 x 64 entries).
 __device__ __forceinline__ void load_rotation(const float *__restrict__ u, int k, float (*Us)[65]) {

@@ -208,9 +208,9 @@ estimator_kernel(const float *__restrict__ sigma, const float *__restrict__ U, c
     }
     if (lambda_out)
         for (int l = tid; l < k; l += 256)
-            lambda_out[pt * k + l] = (l < p) ? fmaxf(sg[l], 0.f) / (float)(k - 1) : 0.f;
+            lambda_out[pt * k + l] = lambda_of(sg[l], l, p, k);
     if (s_out)
-        for (int l = tid; l < k; l += 256) s_out[pt * k + l] = sqrtf(fmaxf(sg[l], 0.f));
+        for (int l = tid; l < k; l += 256) s_out[pt * k + l] = sqrtf(pos_part(sg[l]));
 }
 
 cudaError_t launch_estimator(const float *sigma, const float *U, const float *M, const float *R,

@@ -170,7 +170,7 @@ jacobi_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restrict__
         int rank = 0;
         for (int j = 0; j < k; ++j) {
             const Real dj = A[j * ld + j];
-            rank += (dj > di) || (dj == di && j < i);
+            rank += pair_before(dj, j, di, i);
         }
         sg[rank] = (float)di;
         for (int r = 0; r < k; ++r) u[r * k + rank] = (float)V[r * ld + i];
@@ -375,7 +375,7 @@ jacobi_warp_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restr
         int rank = 0;
         for (int j = 0; j < k; ++j) {
             const float dj = A[j * ld + j];
-            rank += (dj > di) || (dj == di && j < i);
+            rank += pair_before(dj, j, di, i);
         }
         sg[rank] = di;
         for (int r = 0; r < k; ++r) u[r * k + rank] = Ut[i * kp + r];
@@ -582,7 +582,7 @@ __device__ __forceinline__ void refine_ff_patch(const PatchSeg &seg, int local, 
     float *sg = sigma + pt * (int64_t)k;
     for (int i = tid; i < k; i += NT) {
         int rank = 0;
-        for (int j = 0; j < k; ++j) rank += (lam[j] > lam[i]) || (lam[j] == lam[i] && j < i);
+        for (int j = 0; j < k; ++j) rank += pair_before(lam[j], j, lam[i], i);
         sg[rank] = (float)lam[i];
         for (int r = 0; r < k; ++r) u[r * k + rank] = Xn[r * ld + i];
     }
@@ -817,7 +817,7 @@ __device__ __forceinline__ void refine_res_patch(const PatchSeg &seg, int local,
     if (tid < k) {
         const float li = lam[tid];
         int rank = 0;
-        for (int j = 0; j < k; ++j) rank += (lam[j] > li) || (lam[j] == li && j < tid);
+        for (int j = 0; j < k; ++j) rank += pair_before(lam[j], j, li, tid);
         sg[rank] = li;
         rk[tid] = rank;
     }

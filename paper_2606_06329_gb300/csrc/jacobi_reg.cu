@@ -343,8 +343,8 @@ __device__ __forceinline__ void solve(const PatchSeg &seg, int64_t patch, int np
     int rx = 0, ry = 0;
     for (int c = 0; c < R; ++c) {
         const float v = nu[c];
-        rx += (v > al) || (v == al && c < c0);
-        ry += (v > be) || (v == be && c < c1);
+        rx += pair_before(v, c, al, c0);
+        ry += pair_before(v, c, be, c1);
     }
     if (mine) {
         float *sg = seg.sig + (patch + g) * (int64_t)k;

@@ -515,8 +515,8 @@ patch_m3_kernel(const T *__restrict__ X, int64_t N, int64_t m, int64_t ld, const
     fast_kappa<NT>(k, p, m, out.variant, gsum, sg, out.R + pt * k, diag, ldz, Vs, ldz, Qs, ldz, c_s, red,
                    out.kappa + pt);
     if (out.lambda && tid < k)
-        out.lambda[pt * k + tid] = tid < p ? fmaxf(sg[tid], 0.f) / (float)(k - 1) : 0.f;
-    if (out.s && tid < k) out.s[pt * k + tid] = sqrtf(fmaxf(sg[tid], 0.f));
+        out.lambda[pt * k + tid] = lambda_of(sg[tid], tid, p, k);
+    if (out.s && tid < k) out.s[pt * k + tid] = sqrtf(pos_part(sg[tid]));
 }
 
 namespace {

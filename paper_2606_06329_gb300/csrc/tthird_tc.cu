@@ -426,9 +426,9 @@ tthird_tc_kernel(const __grid_constant__ CUtensorMap map_y, const __grid_constan
     fast_kappa<TT_THREADS>(k, p, m, variant, gsum, sg, R + pt * k, diag, TT_DLD, Us, 65, Qs, 65, c_s, red, kappa + pt);
     if (lambda_out)
         for (int l = tid; l < k; l += TT_THREADS)
-            lambda_out[pt * k + l] = (l < p) ? fmaxf(sg[l], 0.f) / (float)(k - 1) : 0.f;
+            lambda_out[pt * k + l] = lambda_of(sg[l], l, p, k);
     if (s_out)
-        for (int l = tid; l < k; l += TT_THREADS) s_out[pt * k + l] = sqrtf(fmaxf(sg[l], 0.f));
+        for (int l = tid; l < k; l += TT_THREADS) s_out[pt * k + l] = sqrtf(pos_part(sg[l]));
     tc::fence_before();
     __syncthreads();
     if (warp == 0) {
