@@ -268,9 +268,10 @@ __device__ __forceinline__ void solve(const PatchSeg &seg, int64_t patch, int np
     int sweep = 0, seam = H - 1;
     unsigned long long rotations = 0;
     bool converged = false;
+    float mx = 0.f;  // largest squared cosine that this lane met in the sweep
     while (sweep < max_sweeps) {
         float al = dot_cols<NP>(X, X), be = dot_cols<NP>(Y, Y);
-        float mx = 0.f;
+        mx = 0.f;
         unsigned nrot = 0;
         for (int rr = 0; rr < H; ++rr) {
             float t, c, cos2, ga;
@@ -376,11 +377,15 @@ __device__ __forceinline__ void solve(const PatchSeg &seg, int64_t patch, int np
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) rotations += __shfl_xor_sync(FULL, rotations, o);
+    // patches above the bound after the last sweep (the others only shared its warp)
+    const unsigned above = __ballot_sync(FULL, mine && mx >= stop2);
     if (lane == 0) {
         atomicMax(&ctr->jacobi_max_sweeps, (unsigned long long)sweep);
         atomicAdd(&ctr->jacobi_rotations, rotations);
         if (!converged) {
-            atomicAdd(&ctr->jacobi_not_converged, (unsigned long long)np);
+            unsigned missed = 0;
+            for (int p = 0; p < PPW; ++p) missed += ((above >> (p * H)) & (FULL >> (32 - H))) != 0u;
+            atomicAdd(&ctr->jacobi_not_converged, (unsigned long long)missed);
             atomicOr(&ctr->status, (unsigned)DEV_NOT_CONVERGED);
         }
     }
