@@ -136,13 +136,13 @@ typedef enum {
                                         over a device table of all datasets' work items, estimator launches
                                         over segment tables of all datasets' points); 0: one stream lane per
                                         dataset group, as the FP32 form always does.  Results identical */
-    MECUCO_OPT_JACOBI_WARP = 16,     /* FP32 Jacobi sweeps.  2 (default): the register-resident one-sided form
+    MECUCO_OPT_JACOBI_WARP = 16,     /* FP32 Jacobi sweeps.  -1 (default): the register-resident one-sided form
                                         (Cholesky factor, one patch per 8 to 32 lanes) where only the refined
                                         eigenpairs are used (BF16-mixed forward with m >= 128, plain rotation), two
-                                        warps per patch in the fused form elsewhere; 1, 4: that many warps per
-                                        patch in the fused form (a round's rotations applied in one pass over 2 x 2 blocks of A
-                                        and U, two barriers per round, none with 1 warp); 0: one CTA of 128
-                                        threads per patch in three passes (row, column and eigenvector
+                                        warps per patch in the fused form elsewhere; 1, 2, 4: that many warps per
+                                        patch in the fused form (a round's rotations applied in one pass over 2 x 2
+                                        blocks of A and U, two barriers per round, none with 1 warp); 0: one CTA of
+                                        128 threads per patch in three passes (row, column and eigenvector
                                         updates, three barriers per round).  The fused and the CTA form apply the
                                         same rotations and thresholds; all forms agree to rounding.  Measured per
                                         100k patches (k = 64), with the refinement: 230 ms (0), 221 (1), 192 (4),

@@ -100,7 +100,9 @@ struct mecuco_ctx {
     int64_t knn_margin = 32;
     int jacobi_fp64 = -1;
     int jacobi_max_sweeps = 40;
-    int jacobi_warp = 2;  // FP32 sweeps: warps per patch of the fused form (0: the three-pass CTA form)
+    // FP32 sweeps: warps per patch of the fused form (0: the three-pass CTA form); -1: the
+    // register-resident form where only refined pairs are used, else two warps
+    int jacobi_warp = -1;
     int64_t chunk_points = 0;
     int64_t knn_qchunk = 0;
     int profile = 0;
@@ -989,7 +991,7 @@ mecuco_status run_batched_persistent(mecuco_t h, const mecuco_dataset *sets, int
                launch_jacobi_seg(none, tab, ch.nseg, ch.kmax, ch.np, fp64, h->jacobi_max_sweeps, h->ctr, s,
                                  kJacobiPreLoose, h->jacobi_warp, ch.reg));
         if (fp64 == 1 || fp64 == 3) ++h->launches;
-        if (fp64 == 1 && h->jacobi_warp == 2 && ch.reg.np > 0 && ch.reg.np < ch.np) ++h->launches;  // both sweep forms
+        if (fp64 == 1 && h->jacobi_warp < 0 && ch.reg.np > 0 && ch.reg.np < ch.np) ++h->launches;  // both sweep forms
         LAUNCH(h, MECUCO_STAGE_ROTATE, s,
                launch_rotate_tc(dt, none, tab, ch.nseg, ch.np, ch.Y, ch.ldy, h->wait_limit, h->ctr, s));
         LAUNCH(h, MECUCO_STAGE_MOMENTS, s,
@@ -1184,7 +1186,7 @@ mecuco_status mecuco_set_option(mecuco_t h, mecuco_option opt, int64_t v) {
             h->batch_lanes = (int)v;
             break;
         case MECUCO_OPT_JACOBI_WARP:
-            if (v != 0 && v != 1 && v != 2 && v != 4) return MECUCO_ERR_INVALID_ARG;
+            if (v != -1 && v != 0 && v != 1 && v != 2 && v != 4) return MECUCO_ERR_INVALID_ARG;
             h->jacobi_warp = (int)v;
             break;
         case MECUCO_OPT_KNN_SPLIT_BF16:

@@ -854,7 +854,9 @@ cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab
     // FP32 sweeps: one or more warps per patch, or one CTA per patch
     auto sweeps32 = [&](const PatchSeg *t, int nt, int kb, int64_t n, int64_t blk0, float eps) -> cudaError_t {
         if (n <= 0) return cudaSuccess;
-        if (warp_form) return launch_jacobi_warp(one, t, nt, kb, n, (int)blk0, max_sweeps, eps, ctr, s, warp_form);
+        if (warp_form)
+            return launch_jacobi_warp(one, t, nt, kb, n, (int)blk0, max_sweeps, eps, ctr, s,
+                                      warp_form < 0 ? 2 : warp_form);
         const size_t smem = jacobi_smem_bytes(kb, 0);
         cudaError_t r = cudaFuncSetAttribute(jacobi_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                              (int)smem);
@@ -864,7 +866,7 @@ cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab
     };
     if (fp64 == 1 || fp64 == 3) {
         // FP32 sweeps, then one refinement step (3: relative cluster test)
-        const bool fast = reg.np > 0 && fp64 == 1 && warp_form == 2;
+        const bool fast = reg.np > 0 && fp64 == 1 && warp_form < 0;
         if (fast) {
             // |cos| of the last sweep: the step after it squares what is left
             const float stop = pre_eps >= kJacobiPreLoose ? 9.765625e-04f : 1.220703125e-04f;  // 2^-10, 2^-13

@@ -230,7 +230,7 @@ cudaError_t launch_tthird_tc(const PatchSeg &one, const PatchSeg *tab, int ntab,
 // rotated Gram must come out nearly diagonal, take kJacobiPreTight.
 constexpr float kJacobiPreTight = 2.384185791015625e-07f;  // 2^-22
 constexpr float kJacobiPreLoose = 6.103515625e-05f;        // 2^-14
-// reg: the leading points solved, with fp64 = 1 and warp_form = 2 (the default),
+// reg: the leading points solved, with fp64 = 1 and warp_form < 0 (the default),
 // by the register-resident one-sided sweeps (jacobi_reg.cu; 4 to 9 times faster
 // than the fused two-sided form at every k measured) and the refinement through
 // the residual (5 times faster at k = 64).  Callers whose results follow the
@@ -249,9 +249,10 @@ struct JacobiReg {
 // m = 64, k = 52, against 5e-6 at m = 128 and 3e-6 from m = 192 up, and such
 // narrow sets keep the values they had.
 constexpr int64_t JACOBI_REG_MIN_M = 128;
-// warp_form != 0: the FP32 sweeps run one warp per patch (fused 2 x 2 block
-// updates, no block barriers); 0: one CTA of 128 threads per patch.  FP64
-// sweeps (fp64 = 2) always take the CTA form.
+// warp_form 1, 2, 4: the FP32 sweeps run that many warps per patch (fused 2 x 2
+// block updates); 0: one CTA of 128 threads per patch; -1: the register-resident
+// form where reg allows it, else two warps.  FP64 sweeps (fp64 = 2) always take the
+// CTA form.
 cudaError_t launch_jacobi(const float *G, int k, int64_t np, int fp64, int max_sweeps,
                           float *sigma, float *U, DevCounters *ctr, cudaStream_t s,
                           float pre_eps = kJacobiPreTight, int warp_form = 1, bool reg = false);
