@@ -108,6 +108,7 @@ struct mecuco_ctx {
     int profile = 0;
     int64_t profile_mask = -1;  // stages bracketed while profiling (bit = mecuco_stage)
     long long wait_limit = 0;   // clock cycles of the tensor-core kernels' work waits (0: default)
+    int split_cap = 0;          // of the running call's search plan, under a limit (0: none)
     size_t ws_cap = 0;          // cap on the bytes of one device allocation of the context (0: none)
     // per-call bookkeeping
     int64_t launches = 0;
@@ -235,25 +236,19 @@ int candidate_capacity(mecuco_t h, int k) {
 constexpr int64_t KNN_PAIR_MIN_K = 2200;
 
 struct KnnPlan {
-    struct Piece {
-        int64_t rows;  // query rows of one search launch
-        int nsplit;    // candidate-range splits; nsplit x halves lists per row
-    };
-    std::vector<Piece> pieces;
+    // The rows go in launches of qchunk (the first main_rows) and one of the rest;
+    // each row has nsplit x halves lists of kcl candidates.
+    int64_t nrows, main_rows, qchunk;
+    int main_split, tail_split;  // candidate-range splits of the launches
     int kc;
     int halves;     // lists per row and split (the tensor-core kernel's column halves)
     int kcl;        // capacity of each list
     int cap;        // largest number of splits (1024 candidates per row)
-    int64_t qchunk;
-    int64_t max_rows() const {
-        int64_t r = 0;
-        for (const Piece &q : pieces) r = std::max(r, q.rows);
-        return r;
-    }
+    int64_t rows_at(int64_t q) const { return q < main_rows ? std::min(qchunk, main_rows - q) : nrows - q; }
+    int split_at(int64_t q) const { return q < main_rows ? main_split : tail_split; }
+    int64_t max_rows() const { return std::max(std::min(qchunk, main_rows), nrows - main_rows); }
     int64_t max_slots() const {
-        int64_t r = 0;
-        for (const Piece &q : pieces) r = std::max(r, q.rows * q.nsplit * halves * kcl);
-        return r;
+        return std::max(std::min(qchunk, main_rows) * main_split, (nrows - main_rows) * tail_split) * halves * kcl;
     }
     bool tc;        // candidate search on the tensor cores (BF16 operands)
     bool pair;      // tensor-core search as CTA pairs sharing two-SM MMAs
@@ -269,6 +264,7 @@ inline int64_t split_segment(int64_t m) { return (m + 7) / 8 * 8; }
 KnnPlan plan_knn(mecuco_t h, const void *X, mecuco_dtype dt, int64_t N, int64_t m, int64_t ld, int64_t nrows, int k,
                  mecuco_precision prec) {
     KnnPlan p;
+    p.nrows = nrows;
     p.kc = candidate_capacity(h, k);
     p.tc = prec == MECUCO_PREC_BF16_MIXED;
     const bool direct = dt == MECUCO_BF16 && ld % 8 == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
@@ -302,7 +298,8 @@ KnnPlan plan_knn(mecuco_t h, const void *X, mecuco_dtype dt, int64_t N, int64_t 
         sp = std::min(sp, p.cap);
         if (h->knn_splits > 0) sp = std::min(h->knn_splits, p.cap);
         while (sp > 1 && !fits(sp)) --sp;
-        for (int64_t a = 0; a < nrows; a += p.qchunk) p.pieces.push_back({std::min(p.qchunk, nrows - a), sp});
+        p.main_rows = nrows;
+        p.main_split = p.tail_split = sp;
         return p;
     }
     // Launches of whole waves with one list set per row, and the rows of the
@@ -316,22 +313,18 @@ KnnPlan plan_knn(mecuco_t h, const void *X, mecuco_dtype dt, int64_t N, int64_t 
     const double tile = p.tc ? std::max(4000.0, 7.5 * (double)p.mk) : 4500.0 + 122.0 * (double)m;
     const int64_t item_rows = p.tc ? knn_tc_item_rows(p.pair) : 128;
     const double waves1 = (double)((N + 255) / 256) * tile, rr = 3.0 * p.halves * p.kcl / 128;
-    for (int64_t left = nrows; left > 0;) {
-        const int64_t take = left >= wave ? std::min(p.qchunk, left / wave * wave) : left;
-        int best = 1;
-        if (take < wave) {
-            const int64_t items = (take + item_rows - 1) / item_rows, slots = wave / item_rows;
-            double cost = waves1 + rr * (double)take;
-            for (int sp = 2; fits(sp); ++sp) {
-                const double c = (double)((items * sp + slots - 1) / slots) / sp * waves1 + rr * (double)take * sp;
-                if (c < 0.95 * cost) {
-                    cost = c;
-                    best = sp;
-                }
+    p.main_rows = nrows / wave * wave;
+    p.main_split = p.tail_split = 1;
+    if (const int64_t tail = nrows - p.main_rows; tail > 0) {
+        const int64_t items = (tail + item_rows - 1) / item_rows, slots = wave / item_rows;
+        double cost = waves1 + rr * (double)tail;
+        for (int sp = 2; fits(sp) && (h->split_cap == 0 || sp <= h->split_cap); ++sp) {
+            const double c = (double)((items * sp + slots - 1) / slots) / sp * waves1 + rr * (double)tail * sp;
+            if (c < 0.95 * cost) {
+                cost = c;
+                p.tail_split = sp;
             }
         }
-        p.pieces.push_back({take, best});
-        left -= take;
     }
     return p;
 }
@@ -369,33 +362,47 @@ mecuco_status run_knn(mecuco_t h, char *ws, const void *X, mecuco_dtype dt, int6
            launch_row_prep(X, dt, N, m, ld, b.norms, s, b.resid, b.maxima, p.quant, b.xb, b.xb2, split_segment(m),
                            p.ldb));
     const void *Xa = b.xb ? b.xb : X, *Xb = b.xb2 ? b.xb2 : Xa;
-    int64_t q0 = rb;
-    for (const KnnPlan::Piece &piece : p.pieces) {
-        const int64_t nq = piece.rows;
+    for (int64_t q0 = rb; q0 < re;) {
+        const int64_t nq = p.rows_at(q0 - rb);
+        const int nsplit = p.split_at(q0 - rb);
         int32_t *io = idx_out + (q0 - rb) * k;
         float *dout = dist_out ? dist_out + (q0 - rb) * k : nullptr;
         if (p.tc) {
             LAUNCH(h, MECUCO_STAGE_KNN_SEARCH, s,
-                   launch_knn_tc(Xa, Xb, N, p.mk, p.ldb, b.norms, q0, nq, p.kcl, piece.nsplit, include_self, b.cand_d,
+                   launch_knn_tc(Xa, Xb, N, p.mk, p.ldb, b.norms, q0, nq, p.kcl, nsplit, include_self, b.cand_d,
                                  b.cand_i, p.pair ? 1 : 0, h->wait_limit, h->ctr, s));
         } else {
             LAUNCH(h, MECUCO_STAGE_KNN_SEARCH, s,
-                   launch_knn_simt(X, dt, N, m, ld, b.norms, q0, nq, p.kc, piece.nsplit, include_self, b.cand_d,
+                   launch_knn_simt(X, dt, N, m, ld, b.norms, q0, nq, p.kc, nsplit, include_self, b.cand_d,
                                    b.cand_i, s));
         }
         // every row's lists go to the exact re-rank together: a point that a list
         // rejected has d~ >= that list's maximum, so the smallest list maximum
         // bounds every candidate left out
         LAUNCH(h, MECUCO_STAGE_KNN_RERANK, s,
-               launch_knn_rerank(X, dt, N, m, ld, b.norms, q0, nq, p.kcl, piece.nsplit * p.halves, k, b.cand_d,
-                                 b.cand_i, io, dout,
-                                 b.flags, h->ctr, s, b.resid, b.maxima, p.quant));
+               launch_knn_rerank(X, dt, N, m, ld, b.norms, q0, nq, p.kcl, nsplit * p.halves, k, b.cand_d,
+                                 b.cand_i, io, dout, b.flags, h->ctr, s, b.resid, b.maxima, p.quant));
         LAUNCH(h, MECUCO_STAGE_KNN_FALLBACK, s,
                launch_knn_fallback(X, dt, N, m, ld, q0, nq, k, include_self, b.flags, io, dout, h->ctr, s));
         q0 += nq;
     }
     h->knn_rows += re - rb;
     return MECUCO_OK;
+}
+
+// Bytes of a call's workspace, `bytes()` under the present plan: with a limit that does
+// not hold the candidate lists of the fastest split, those of fewer splits, down to
+// one (the plan of the call follows h->split_cap).  have: bytes allocated already.
+template <typename F>
+size_t bytes_within_limit(mecuco_t h, size_t have, F bytes) {
+    h->split_cap = 0;
+    size_t need = bytes();
+    if (h->ws_cap)
+        for (int cap = 1024 / 32 - 1; need > std::max(h->ws_cap, have) && cap > 0; --cap) {
+            h->split_cap = cap;
+            need = bytes();
+        }
+    return need;
 }
 
 size_t knn_bytes(mecuco_t h, const void *X, mecuco_dtype dt, int64_t N, int64_t m, int64_t ld, int64_t nrows, int k,
@@ -410,6 +417,7 @@ size_t knn_bytes(mecuco_t h, const void *X, mecuco_dtype dt, int64_t N, int64_t 
 mecuco_status begin_call(mecuco_t h, cudaStream_t s) {
     h->launches = 0;
     h->knn_rows = 0;
+    h->split_cap = 0;
     CK(cudaSetDevice(h->device));
     CK(cudaMemsetAsync(h->ctr, 0, offsetof(DevCounters, status), s));
     return MECUCO_OK;
@@ -695,16 +703,25 @@ mecuco_status run_batched_lanes(mecuco_t h, const mecuco_dataset *sets, int nset
         const int l = (int)(std::min_element(load.begin(), load.end()) - load.begin());
         load[l] += cost[i];
         lane_of[i] = l;
-        const mecuco_dataset &d = sets[i];
-        set_idx_bytes[i] = d.idx ? 0 : align_up((size_t)d.N * d.k * sizeof(int32_t), 256);
-        const size_t need = set_idx_bytes[i] + std::max(knn_bytes(h, d.X, dt, d.N, d.m, d.ld, d.N, d.k, prec, 0),
-                                                        curvature_bytes(h, d.X, dt, d.N, d.m, d.ld, d.k, true, d.N,
-                                                                        prec));
-        lane_bytes[l] = std::max(lane_bytes[l], align_up(need, 256));
+        set_idx_bytes[i] = sets[i].idx ? 0 : align_up((size_t)sets[i].N * sets[i].k * sizeof(int32_t), 256);
     }
     std::vector<size_t> lane_off(lanes, 0);
-    size_t total = 0;
-    for (int l = 0; l < lanes; ++l) { lane_off[l] = total; total += lane_bytes[l]; }
+    const size_t total = bytes_within_limit(h, h->bws_bytes, [&] {
+        std::fill(lane_bytes.begin(), lane_bytes.end(), 0);
+        for (int i = 0; i < nsets; ++i) {
+            const mecuco_dataset &d = sets[i];
+            const size_t need =
+                set_idx_bytes[i] + std::max(knn_bytes(h, d.X, dt, d.N, d.m, d.ld, d.N, d.k, prec, 0),
+                                            curvature_bytes(h, d.X, dt, d.N, d.m, d.ld, d.k, true, d.N, prec));
+            lane_bytes[lane_of[i]] = std::max(lane_bytes[lane_of[i]], align_up(need, 256));
+        }
+        size_t sum = 0;
+        for (int l = 0; l < lanes; ++l) {
+            lane_off[l] = sum;
+            sum += lane_bytes[l];
+        }
+        return sum;
+    });
     if ((st = ensure(h->bws, h->bws_bytes, total, h->ws_cap)) != MECUCO_OK) return st;
     for (int l = 0; l < lanes; ++l) {
         if (!h->lane_stream[l]) CK(cudaStreamCreateWithFlags(&h->lane_stream[l], cudaStreamNonBlocking));
@@ -1212,9 +1229,9 @@ mecuco_status mecuco_knn_range(mecuco_t h, const void *X, mecuco_dtype dt, int64
     if (prec != MECUCO_PREC_FP32 && prec != MECUCO_PREC_BF16_MIXED) return MECUCO_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     if ((st = begin_call(h, s)) != MECUCO_OK) return st;
-    if ((st = ensure(h->ws, h->ws_bytes, knn_bytes(h, X, dt, N, m, ld, re - rb, k, prec, 0), h->ws_cap)) !=
-        MECUCO_OK)
-        return st;
+    const size_t need =
+        bytes_within_limit(h, h->ws_bytes, [&] { return knn_bytes(h, X, dt, N, m, ld, re - rb, k, prec, 0); });
+    if ((st = ensure(h->ws, h->ws_bytes, need, h->ws_cap)) != MECUCO_OK) return st;
     return run_knn(h, h->ws, X, dt, N, m, ld, k, include_self, prec, rb, re, idx_out, dist_out, s, 0);
 }
 
@@ -1239,9 +1256,9 @@ mecuco_status mecuco_curvature_range(mecuco_t h, const void *X, mecuco_dtype dt,
     if (prec == MECUCO_PREC_BF16_MIXED && ((st = ensure_pairs(h, k)) != MECUCO_OK ||
                                            (st = ensure_rotated(h, k)) != MECUCO_OK))
         return st;
-    if ((st = ensure(h->ws, h->ws_bytes, curvature_bytes(h, X, dt, N, m, ld, k, idx != nullptr, re - rb, prec),
-                     h->ws_cap)) != MECUCO_OK)
-        return st;
+    const size_t need = bytes_within_limit(
+        h, h->ws_bytes, [&] { return curvature_bytes(h, X, dt, N, m, ld, k, idx != nullptr, re - rb, prec); });
+    if ((st = ensure(h->ws, h->ws_bytes, need, h->ws_cap)) != MECUCO_OK) return st;
     return run_curvature(h, h->ws, X, dt, N, m, ld, k, idx, include_self, var, prec, rb, re, kappa_out, lambda_out,
                          U_out, s_out, s);
 }
@@ -1275,7 +1292,9 @@ mecuco_status mecuco_curvature_rsvd(mecuco_t h, const void *X, mecuco_dtype dt, 
     h->rsvd.cols = sketch_cols;
     h->rsvd.power = power_iters;
     h->rsvd.omega = omega;
-    st = ensure(h->ws, h->ws_bytes, curvature_bytes(h, X, dt, N, m, ld, k, idx != nullptr, N, prec), h->ws_cap);
+    const size_t need = bytes_within_limit(
+        h, h->ws_bytes, [&] { return curvature_bytes(h, X, dt, N, m, ld, k, idx != nullptr, N, prec); });
+    st = ensure(h->ws, h->ws_bytes, need, h->ws_cap);
     if (st == MECUCO_OK)
         st = run_curvature(h, h->ws, X, dt, N, m, ld, k, idx, include_self, var, prec, 0, N, kappa_out, nullptr,
                            nullptr, nullptr, s);
@@ -1412,8 +1431,9 @@ mecuco_status mecuco_curvature_exact(mecuco_t h, const void *X, mecuco_dtype dt,
     t.take<float>((size_t)chunk * m * m);
     t.take<float>((size_t)chunk * m);
     t.take<float>((size_t)chunk * m * m);
-    size_t need = t.off;
-    if (!idx) need = std::max(need, knn_bytes(h, X, dt, N, m, ld, nrows, k, prec, idx_bytes));
+    const size_t need = bytes_within_limit(h, h->ws_bytes, [&] {
+        return idx ? t.off : std::max(t.off, knn_bytes(h, X, dt, N, m, ld, nrows, k, prec, idx_bytes));
+    });
     if ((st = ensure(h->ws, h->ws_bytes, need, h->ws_cap)) != MECUCO_OK) return st;
     const int32_t *nbr = idx ? idx + rb * k : nullptr;
     if (!idx) {
@@ -1580,8 +1600,10 @@ mecuco_status mecuco_curvature_host(mecuco_t h, const void *X_host, mecuco_dtype
     if (prec == MECUCO_PREC_BF16_MIXED && ((st = ensure_pairs(h, k)) != MECUCO_OK ||
                                            (st = ensure_rotated(h, k)) != MECUCO_OK))
         return st;
-    const size_t need = std::max(knn_bytes(h, Xd, dt, N, m, ld, N, k, prec, 0),
-                                 curvature_bytes(h, Xd, dt, N, m, ld, k, true, N, prec));
+    const size_t need = bytes_within_limit(h, h->ws_bytes, [&] {
+        return std::max(knn_bytes(h, Xd, dt, N, m, ld, N, k, prec, 0),
+                        curvature_bytes(h, Xd, dt, N, m, ld, k, true, N, prec));
+    });
     if ((st = ensure(h->ws, h->ws_bytes, need, h->ws_cap)) != MECUCO_OK) return st;
     if ((st = run_knn(h, h->ws, Xd, dt, N, m, ld, k, include_self, prec, 0, N, id, nullptr, s, 0)) != MECUCO_OK)
         return st;
