@@ -577,7 +577,7 @@ mecuco_status run_curvature(mecuco_t h, char *ws, const void *X, mecuco_dtype dt
                    launch_rsvd_range(b.G, k, np, h->rsvd.omega, l, h->rsvd.power, b.rQ, b.rB, s));
             LAUNCH(h, MECUCO_STAGE_JACOBI, s,
                    launch_jacobi(b.rB, l, np, 1, h->jacobi_max_sweeps, b.rsig, b.rV, h->ctr, s,
-                                 kJacobiPreTight, h->jacobi_warp));
+                                 h->jacobi_warp));
             ++h->launches;
             LAUNCH(h, MECUCO_STAGE_JACOBI, s,
                    launch_rsvd_compose(b.rQ, b.rsig, b.rV, k, l, h->rsvd.rank, np, b.sig, Ud, s));
@@ -609,8 +609,7 @@ mecuco_status run_curvature(mecuco_t h, char *ws, const void *X, mecuco_dtype dt
             const int haar = var == MECUCO_FAST_HAAR ? 1 : 0;
             LAUNCH(h, MECUCO_STAGE_GRAM, s, launch_gram_tc(dt, sg, nullptr, 0, np, haar, h->wait_limit, h->ctr, s));
             LAUNCH(h, MECUCO_STAGE_JACOBI, s,
-                   launch_jacobi_seg(sg, nullptr, 0, k, np, fp64, h->jacobi_max_sweeps, h->ctr, s, kJacobiPreLoose,
-                                     h->jacobi_warp, m >= JACOBI_REG_MIN_M ? jacobi_reg_all(k, np) : JacobiReg()));
+                   launch_jacobi_seg(sg, nullptr, 0, k, np, fp64, h->jacobi_max_sweeps, h->ctr, s, h->jacobi_warp, m >= JACOBI_REG_MIN_M ? jacobi_reg_all(k, np) : JacobiReg()));
             if (fp64 == 1 || fp64 == 3) ++h->launches;  // the refinement is a second kernel
             LAUNCH(h, MECUCO_STAGE_ROTATE, s,
                    launch_rotate_tc(dt, sg, nullptr, 0, np, b.Y, rot_ld(m), h->wait_limit, h->ctr, s));
@@ -624,14 +623,14 @@ mecuco_status run_curvature(mecuco_t h, char *ws, const void *X, mecuco_dtype dt
             LAUNCH(h, MECUCO_STAGE_GRAM, s,
                    launch_patch_gram(X, dt, N, m, ld, nb, k, 0, np, nullptr, b.G, b.R, nullptr, h->ctr, s));
             LAUNCH(h, MECUCO_STAGE_JACOBI, s, launch_jacobi(b.G, k, np, 1, h->jacobi_max_sweeps, b.sig, b.U0, h->ctr, s,
-                                 kJacobiPreTight, h->jacobi_warp, true));
+                                 h->jacobi_warp, true));
             ++h->launches;
             LAUNCH(h, MECUCO_STAGE_GRAM, s,
                    launch_patch_gram(X, dt, N, m, ld, nb, k, 0, np, b.U0, b.G, b.R, var == MECUCO_FAST_HAAR ? b.Q : nullptr,
                                      h->ctr, s));
             LAUNCH(h, MECUCO_STAGE_JACOBI, s,
                    launch_jacobi(b.G, k, np, fp64, h->jacobi_max_sweeps, b.sig, b.U, h->ctr, s,
-                                 kJacobiPreTight, h->jacobi_warp));
+                                 h->jacobi_warp));
             if (fp64 == 1 || fp64 == 3) ++h->launches;
             LAUNCH(h, MECUCO_STAGE_ESTIMATOR, s,
                    launch_patch_kappa(X, dt, N, m, ld, nb, k, np, b.U0, b.sig, b.U, b.R, Qarg, (int)var,
@@ -1006,7 +1005,7 @@ mecuco_status run_batched_persistent(mecuco_t h, const mecuco_dataset *sets, int
         LAUNCH(h, MECUCO_STAGE_GRAM, s, launch_gram_tc(dt, none, tab, ch.nseg, ch.np, haar, h->wait_limit, h->ctr, s));
         LAUNCH(h, MECUCO_STAGE_JACOBI, s,
                launch_jacobi_seg(none, tab, ch.nseg, ch.kmax, ch.np, fp64, h->jacobi_max_sweeps, h->ctr, s,
-                                 kJacobiPreLoose, h->jacobi_warp, ch.reg));
+                                 h->jacobi_warp, ch.reg));
         if (fp64 == 1 || fp64 == 3) ++h->launches;
         if (fp64 == 1 && h->jacobi_warp < 0 && ch.reg.np > 0 && ch.reg.np < ch.np) ++h->launches;  // both sweep forms
         LAUNCH(h, MECUCO_STAGE_ROTATE, s,
@@ -1358,7 +1357,7 @@ mecuco_status mecuco_curvature_backward(mecuco_t h, const void *X, mecuco_dtype 
         LAUNCH(h, MECUCO_STAGE_GRAM, s,
                launch_patch_gram(X, dt, N, m, ld, nb, k, 0, np, nullptr, b.G, b.R, nullptr, h->ctr, s));
         LAUNCH(h, MECUCO_STAGE_JACOBI, s, launch_jacobi(b.G, k, np, 1, h->jacobi_max_sweeps, b.sig, U0, h->ctr, s,
-                                 kJacobiPreTight, h->jacobi_warp));
+                                 h->jacobi_warp));
         ++h->launches;  // the refinement kernel
         // moments of Z = U0^T X_c and the refined eigenpairs of its Gram
         LAUNCH(h, MECUCO_STAGE_GRAM, s,
@@ -1367,7 +1366,7 @@ mecuco_status mecuco_curvature_backward(mecuco_t h, const void *X, mecuco_dtype 
                launch_patch_m3(X, dt, N, m, ld, nb, k, 0, np, U0, b.M, h->m3_items[k], h->ctr, s));
         LAUNCH(h, MECUCO_STAGE_JACOBI, s,
                launch_jacobi(b.G, k, np, rot_mode, h->jacobi_max_sweeps, b.sig, b.U, h->ctr, s,
-                                 kJacobiPreTight, h->jacobi_warp));
+                                 h->jacobi_warp));
         if (rot_mode == 1 || rot_mode == 3) ++h->launches;  // the refinement kernel
         LAUNCH(h, MECUCO_STAGE_ADJOINT, s,
                launch_adjoint(X, dt, N, m, ld, nb, k, np, (int)var, rank_eps_rotated(k, m), U0, b.sig, b.U, b.M, b.R,
@@ -1405,7 +1404,7 @@ mecuco_status mecuco_tangent_basis(mecuco_t h, const void *X, mecuco_dtype dt, i
         LAUNCH(h, MECUCO_STAGE_GRAM, s,
                launch_patch_gram(X, dt, N, m, ld, nb, k, 0, np, nullptr, G, R, nullptr, h->ctr, s));
         LAUNCH(h, MECUCO_STAGE_JACOBI, s, launch_jacobi(G, k, np, mode, h->jacobi_max_sweeps, sig, U, h->ctr, s,
-                                 kJacobiPreTight, h->jacobi_warp));
+                                 h->jacobi_warp));
         if (mode == 1 || mode == 3) ++h->launches;
         LAUNCH(h, MECUCO_STAGE_BASIS, s,
                launch_tangent_basis(X, dt, N, m, ld, nb, k, np, sig, U, d_out, rank_eps_gram32(m),
@@ -1455,7 +1454,7 @@ mecuco_status mecuco_curvature_exact(mecuco_t h, const void *X, mecuco_dtype dt,
         float *Wd = W_out ? W_out + p0 * m * m : Wb;
         LAUNCH(h, MECUCO_STAGE_EXACT, s, launch_exact_cov(X, dt, N, m, ld, nbr + p0 * k, k, np, S, h->ctr, s));
         LAUNCH(h, MECUCO_STAGE_JACOBI, s, launch_jacobi(S, mm, np, mode, h->jacobi_max_sweeps, vd, Wd, h->ctr, s,
-                                 kJacobiPreTight, h->jacobi_warp));
+                                 h->jacobi_warp));
         if (mode == 1 || mode == 3) ++h->launches;
         LAUNCH(h, MECUCO_STAGE_EXACT, s, launch_exact_kappa(vd, Wd, mm, np, kappa_out + p0, s));
     }

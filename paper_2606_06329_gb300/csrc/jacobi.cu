@@ -9,8 +9,7 @@
 //      block: tau = (a_qq - a_pp) / (2 a_pq), t = sign(tau) / (|tau| +
 //      sqrt(1 + tau^2)), c = 1/sqrt(1 + t^2), s = t c (the rotation zeroing
 //      a_pq); pairs with |a_pq| <= eps sqrt(|a_pp a_qq|) are skipped (eps =
-//      2^-22 in FP32, 2^-50 in FP64; before a refinement step the caller's
-//      pre_eps), and the
+//      2^-22 in FP32, 2^-50 in FP64), and the
 //      rotating pairs are compacted into the round's table (late sweeps are
 //      cheap because few pairs still rotate);
 //   2. A <- A J (each thread walks one row over its share of the pairs),
@@ -425,7 +424,13 @@ cudaError_t launch_jacobi_warp(const PatchSeg &one, const PatchSeg *tab, int nta
 // the FP32 estimate resolves as a cluster (only orthogonalised); with rel != 0
 // the test is relative to the pair, |lam_i - lam_j| <= 2^-18 max(|lam_i|,
 // |lam_j|), for Grams whose FP32 eigenpairs are accurate relative to each
-// eigenvalue (a nearly diagonal Gram, as in the adjoint's rotated basis).
+// eigenvalue (a nearly diagonal Gram, as in the adjoint's rotated basis).  With rel =
+// 0 a pair whose correction would exceed REFINE_MAX_E is taken as one of a cluster
+// too (the relative test leaves 2^-22 / 2^-18 at most), and from REFINE_FIRST_ORDER
+// on the second order is added, X' = X + X E + X E^2 / 2.
+// (With delta alone and the first order, 64 eigenvalues 2^-12 or 2^-16 apart came out
+// with U^T U - I up to 700: what the sweeps leave off the diagonal is not small beside
+// such gaps.)
 // The O(k^3) products R, S and T = A X need more than FP32.  They are carried
 // in two-term FP32 arithmetic ("double-float": a value is hi + lo, |lo| <=
 // ulp(hi) / 2) because GB300 issues FP32 at ~60x its FP64 rate: A and X are
@@ -458,6 +463,11 @@ __device__ __forceinline__ int tri(int a, int b, int k) { return a * k - (a * (a
 }  // namespace
 
 constexpr int FT_REFINE = 256;
+// Largest correction E_ij of a pair, and the largest up to which X (I + E) will do: the
+// step is of first order and leaves E^2 of U^T U - I; beyond, E^2 / 2 is added, which
+// leaves E^4 / 4 (the skew part's exponential to second order).
+constexpr float REFINE_MAX_E = 0.0078125f;              // 2^-7
+constexpr float REFINE_FIRST_ORDER = 2.44140625e-04f;   // 2^-12
 
 template <int NT>
 __device__ __forceinline__ void refine_ff_patch(const PatchSeg &seg, int local, int rel, unsigned char *fsm) {
@@ -558,27 +568,42 @@ __device__ __forceinline__ void refine_ff_patch(const PatchSeg &seg, int local, 
     __syncthreads();
     const double delta = 3.814697265625e-06 * s_lmax;  // 2^-18 max|lam|
     float *Ef = A;  // A is no longer needed
+    bool large = false;
     for (int e = tid; e < kk; e += NT) {
         const int i = e / k, j = e - i * k;
         const int a = i < j ? i : j, b = i < j ? j : i;
         const double rij = Rd(a, b);
         const double sij = Sd(a, b);
         const double dij = rel ? 3.814697265625e-06 * fmax(fabs(lam[i]), fabs(lam[j])) : delta;
+        const double gap = lam[j] - lam[i];
+        // the mean of E_ij's numerator and E_ji's, so that both take the same branch
+        const double num = fabs(sij + 0.5 * (lam[i] + lam[j]) * rij);
         double v;
-        if (i == j || fabs(lam[i] - lam[j]) <= dij) v = 0.5 * rij;
-        else v = (sij + lam[j] * rij) / (lam[j] - lam[i]);
+        if (i == j || fabs(gap) <= dij || (!rel && num > (double)REFINE_MAX_E * fabs(gap))) v = 0.5 * rij;
+        else v = (sij + lam[j] * rij) / gap;  // (a NaN stays one)
+        large = large || fabs(v) > (double)REFINE_FIRST_ORDER;
         Ef[i * ld + j] = (float)v;
     }
-    __syncthreads();
-    // X' = X + X E (FP32), into Th
-    float *Xn = Th;
+    const bool second = __syncthreads_or(large);
+    // X' = X + X E (FP32), into Th; X E kept for the second order
+    float *Xn = Th, *Y = Tl;
     for (int e = tid; e < kk; e += NT) {
         const int r = e / k, c = e - r * k;
         float t = 0.f;
         for (int j = 0; j < k; ++j) t = fmaf(X[r * ld + j], Ef[j * ld + c], t);
         Xn[r * ld + c] = X[r * ld + c] + t;
+        Y[r * ld + c] = t;
     }
     __syncthreads();
+    if (second) {
+        for (int e = tid; e < kk; e += NT) {
+            const int r = e / k, c = e - r * k;
+            float t = 0.f;
+            for (int j = 0; j < k; ++j) t = fmaf(Y[r * ld + j], Ef[j * ld + c], t);
+            Xn[r * ld + c] = fmaf(0.5f, t, Xn[r * ld + c]);
+        }
+        __syncthreads();
+    }
     float *sg = sigma + pt * (int64_t)k;
     for (int i = tid; i < k; i += NT) {
         int rank = 0;
@@ -607,7 +632,8 @@ size_t refine_ff_smem_bytes(int k) {
 // The same refinement step through the residual T = A X - X diag(l), l the
 // sweeps' eigenvalues, for callers that use only the refined eigenpairs:
 //   N = X^T T = S + R diag(l) - diag(l)      (R = I - X^T X, S = X^T A X),
-// so N_ij is the numerator of E_ij for i != j, and lam_i = l_i + N_ii / (1 -
+// so N_ij is the numerator of E_ij for i != j (it decides, with N_ji, whether the pair
+// is one of a cluster), and lam_i = l_i + N_ii / (1 -
 // R_ii).  Only T needs more than FP32: it is small (the sweeps' residual, 1e-6
 // to 1e-4 of lam_1), so N from FP32 products carries 2^-24 of a small matrix,
 // which is a relative error of the correction E, not of the eigenvectors.  R is
@@ -767,50 +793,89 @@ __device__ __forceinline__ void refine_res_patch(const PatchSeg &seg, int local,
     float lmax = 0.f;
     for (int i = 0; i < k; ++i) lmax = fmaxf(lmax, fabsf(lam[i]));
     const float delta = 3.814697265625e-06f * lmax;  // 2^-18 max|lam|
-    // E over T (every thread is past its reads of T)
+    // N over T (every thread is past its reads of T): E_ij needs N_ji too
+    float v[4][4];
+    bool large = false;
     if (mine) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const float2 p = unpack2(n[i][0]), q = unpack2(n[i][1]);
-            float v[4] = {p.x, p.y, q.x, q.y};
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-                const int ii = i0 + i, jj = c0 + c;
-                const float d = (l0[jj] - l0[ii]) + (dl[jj] - dl[ii]);
-                if (ii == jj) {
-                    v[c] = 0.5f * rd[ii];
-                } else if (!(fabsf(d) > delta)) {
-                    v[c] = ii < k && jj < k ? -0.5f * off_dot(X + ii, X + jj, ld, k, 0.f) : 0.f;
-                } else {
-                    v[c] = v[c] / d;
-                }
-            }
-            *reinterpret_cast<float4 *>(T + (i0 + i) * ld + c0) = make_float4(v[0], v[1], v[2], v[3]);
+            v[i][0] = p.x, v[i][1] = p.y, v[i][2] = q.x, v[i][3] = q.y;
+            *reinterpret_cast<float4 *>(T + (i0 + i) * ld + c0) = make_float4(p.x, p.y, q.x, q.y);
         }
     }
     __syncthreads();
-    // X' = X + X E
     if (mine) {
-        f2 acc[4][2] = {};
-        for (int j = 0; j < k; ++j) {
-            const float4 x = *reinterpret_cast<const float4 *>(A + j * ld + i0);
-            const float4 e = *reinterpret_cast<const float4 *>(T + j * ld + c0);
-            const f2 e0 = pack2(e.x, e.y), e1 = pack2(e.z, e.w);
-            const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const float4 t4 = *reinterpret_cast<const float4 *>(T + (c0 + c) * ld + i0);  // N_ji
+            const float nt[4] = {t4.x, t4.y, t4.z, t4.w};
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
-                const f2 x2 = pack2(xv[i], xv[i]);
-                acc[i][0] = fma2(x2, e0, acc[i][0]);
-                acc[i][1] = fma2(x2, e1, acc[i][1]);
+                const int ii = i0 + i, jj = c0 + c;
+                const float d = (l0[jj] - l0[ii]) + (dl[jj] - dl[ii]);
+                // the mean of both numerators, so that E_ij and E_ji take the same branch
+                const float num = 0.5f * fabsf(v[i][c] + nt[i]);
+                if (ii == jj) {
+                    v[i][c] = 0.5f * rd[ii];
+                } else if (!(fabsf(d) > delta) || !(num <= REFINE_MAX_E * fabsf(d))) {
+                    v[i][c] = ii < k && jj < k ? -0.5f * off_dot(X + ii, X + jj, ld, k, 0.f) : 0.f;
+                } else {
+                    v[i][c] = v[i][c] / d;
+                    large = large || fabsf(v[i][c]) > REFINE_FIRST_ORDER;
+                }
             }
         }
+    }
+    const bool second = __syncthreads_or(large);
+    // E over N
+    if (mine) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            float4 *xr = reinterpret_cast<float4 *>(X + (i0 + i) * ld + c0);
-            const float4 x = *xr;
-            const float2 p = unpack2(add2(acc[i][0], pack2(x.x, x.y))), q = unpack2(add2(acc[i][1], pack2(x.z, x.w)));
-            *xr = make_float4(p.x, p.y, q.x, q.y);
+        for (int i = 0; i < 4; ++i)
+            *reinterpret_cast<float4 *>(T + (i0 + i) * ld + c0) = make_float4(v[i][0], v[i][1], v[i][2], v[i][3]);
+    }
+    __syncthreads();
+    // X' = X + X E, and with corrections beyond the first order + (X E) E / 2
+    for (int order = 1;; ++order) {
+        f2 acc[4][2] = {};
+        if (mine) {
+            for (int j = 0; j < k; ++j) {
+                const float4 x = *reinterpret_cast<const float4 *>(A + j * ld + i0);
+                const float4 e = *reinterpret_cast<const float4 *>(T + j * ld + c0);
+                const f2 e0 = pack2(e.x, e.y), e1 = pack2(e.z, e.w);
+                const float xv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const f2 x2 = pack2(xv[i], xv[i]);
+                    acc[i][0] = fma2(x2, e0, acc[i][0]);
+                    acc[i][1] = fma2(x2, e1, acc[i][1]);
+                }
+            }
+            const f2 part = order == 1 ? pack2(1.f, 1.f) : pack2(0.5f, 0.5f);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                float4 *xr = reinterpret_cast<float4 *>(X + (i0 + i) * ld + c0);
+                const float4 x = *xr;
+                const float2 p = unpack2(fma2(part, acc[i][0], pack2(x.x, x.y))),
+                             q = unpack2(fma2(part, acc[i][1], pack2(x.z, x.w)));
+                *xr = make_float4(p.x, p.y, q.x, q.y);
+            }
         }
+        if (order == 2 || !second) break;
+        __syncthreads();  // every thread is past its reads of A
+        if (mine) {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {  // (X E)^T over X^T
+                float t[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 a = unpack2(acc[i][c >> 1]);
+                    t[i] = c & 1 ? a.y : a.x;
+                }
+                *reinterpret_cast<float4 *>(A + (c0 + c) * ld + i0) = make_float4(t[0], t[1], t[2], t[3]);
+            }
+        }
+        __syncthreads();
     }
     // ranks (descending, lowest index first on ties), over dl
     int *rk = reinterpret_cast<int *>(dl);
@@ -846,13 +911,13 @@ size_t jacobi_smem_bytes(int k, int fp64) {
 }
 
 cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t np, int fp64,
-                              int max_sweeps, DevCounters *ctr, cudaStream_t s, float pre_eps, int warp_form,
-                              const JacobiReg &reg) {
+                              int max_sweeps, DevCounters *ctr, cudaStream_t s, int warp_form, const JacobiReg &reg) {
     if (np <= 0) return cudaSuccess;
     if (kmax > 64 || kmax < 1) return cudaErrorInvalidValue;
     cudaError_t e;
     // FP32 sweeps: one or more warps per patch, or one CTA per patch
-    auto sweeps32 = [&](const PatchSeg *t, int nt, int kb, int64_t n, int64_t blk0, float eps) -> cudaError_t {
+    auto sweeps32 = [&](const PatchSeg *t, int nt, int kb, int64_t n, int64_t blk0) -> cudaError_t {
+        const float eps = JacobiEps<float>::rel();
         if (n <= 0) return cudaSuccess;
         if (warp_form)
             return launch_jacobi_warp(one, t, nt, kb, n, (int)blk0, max_sweeps, eps, ctr, s,
@@ -868,16 +933,14 @@ cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab
         // FP32 sweeps, then one refinement step (3: relative cluster test)
         const bool fast = reg.np > 0 && fp64 == 1 && warp_form < 0;
         if (fast) {
-            // |cos| of the last sweep: the step after it squares what is left
-            const float stop = pre_eps >= kJacobiPreLoose ? 9.765625e-04f : 1.220703125e-04f;  // 2^-10, 2^-13
             PatchSeg seg = one;
             seg.npts = (int)np;
             seg.jfirst = 0;
-            e = launch_jacobi_reg(seg, tab, ntab ? reg.nseg : 0, reg.kmax, reg.warps, max_sweeps, stop, ctr, s);
+            e = launch_jacobi_reg(seg, tab, ntab ? reg.nseg : 0, reg.kmax, reg.warps, max_sweeps, ctr, s);
             if (e != cudaSuccess) return e;
-            e = sweeps32(tab + reg.nseg, ntab - reg.nseg, reg.kmax_rest, np - reg.np, reg.np, pre_eps);
+            e = sweeps32(tab + reg.nseg, ntab - reg.nseg, reg.kmax_rest, np - reg.np, reg.np);
         } else {
-            e = sweeps32(tab, ntab, kmax, np, 0, pre_eps);
+            e = sweeps32(tab, ntab, kmax, np, 0);
         }
         if (e != cudaSuccess) return e;
         if (fast) {
@@ -915,17 +978,17 @@ cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab
         jacobi_kernel<double><<<(unsigned)np, JT, smem, s>>>(one, tab, ntab, 0, max_sweeps, JacobiEps<double>::rel(), ctr);
         return cudaGetLastError();
     }
-    return sweeps32(tab, ntab, kmax, np, 0, JacobiEps<float>::rel());
+    return sweeps32(tab, ntab, kmax, np, 0);
 }
 
 cudaError_t launch_jacobi(const float *G, int k, int64_t np, int fp64, int max_sweeps, float *sigma, float *U,
-                          DevCounters *ctr, cudaStream_t s, float pre_eps, int warp_form, bool reg) {
+                          DevCounters *ctr, cudaStream_t s, int warp_form, bool reg) {
     PatchSeg one{};
     one.k = k;
     one.G = const_cast<float *>(G);
     one.sig = sigma;
     one.U = U;
-    return launch_jacobi_seg(one, nullptr, 0, k, np, fp64, max_sweeps, ctr, s, pre_eps, warp_form,
+    return launch_jacobi_seg(one, nullptr, 0, k, np, fp64, max_sweeps, ctr, s, warp_form,
                              reg ? jacobi_reg_all(k, np) : JacobiReg());
 }
 

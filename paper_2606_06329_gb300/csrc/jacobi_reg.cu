@@ -20,10 +20,13 @@
 // Rounds come in twos: the first applies the unscaled rotation x - t y,
 // y + t x (two FMAs per row) and leaves the common factor c to the second,
 // whose four coefficients absorb it.  Squared norms follow the rotations'
-// exact updates and are recomputed every sweep.  The solve ends after a sweep
-// whose largest |cos(x, y)| stayed below the caller's bound (convergence is
-// quadratic: 2^-10 left off-diagonals of at most 2^-15 relative on patches of
-// the curved-patch and MLP workloads).
+// exact updates and are recomputed every sweep.  The solve ends after a sweep whose
+// largest |cos(x, y)| stayed below 2^-17.  Where all gaps are wide the next sweep would
+// square that, but inside a cluster of eigenvalues a tiny inner product still turns
+// two columns by any angle, which undoes earlier rotations to the size of the bound:
+// with a bound of 2^-10, 64 eigenvalues 2^-12 apart kept residuals of 1e-3 lambda_1.
+// (2^-17 costs a sweep on many patches: 30,000 of 301 columns at k = 37 11.1 to 11.3
+// ms in all, a batch of 12 sets 54.2 to 55.3.)
 //
 // The factor is that of G + eps I, eps = 2^-13 of the largest diagonal entry,
 // which has the same eigenvectors: the Gram of a centred patch is singular (its
@@ -77,6 +80,7 @@ __device__ __forceinline__ f2 mul2(f2 a, f2 b) {
 }
 
 constexpr float JR_SHIFT = 1.220703125e-04f;  // 2^-13: the shift eps, on the scaled Gram
+constexpr float JR_STOP2 = 5.820766091346741e-11f;  // 2^-34: the last sweep's squared cosines stay below it
 
 __host__ __device__ constexpr int jr_rows(int k) { return k <= 16 ? 16 : (k + 7) / 8 * 8; }
 // patches per warp
@@ -129,7 +133,7 @@ __device__ __forceinline__ void rotation(float al, float be, float ga, float &t,
 // (np of them); sm: the warp's jr_floats_r(R) shared floats.
 template <int R>
 __device__ __forceinline__ void solve(const PatchSeg &seg, int64_t patch, int np, float *sm, int max_sweeps,
-                                      float stop2, DevCounters *ctr) {
+                                      DevCounters *ctr) {
     constexpr int H = R / 2, PPW = 32 / H, NP = R / 2, LD = R + 4, LDU = R + 1;
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -327,7 +331,7 @@ __device__ __forceinline__ void solve(const PatchSeg &seg, int64_t patch, int np
         }
         ++sweep;
         rotations += nrot;
-        if (__all_sync(FULL, !(mx >= stop2))) {
+        if (__all_sync(FULL, !(mx >= JR_STOP2))) {
             converged = true;
             break;
         }
@@ -378,7 +382,7 @@ __device__ __forceinline__ void solve(const PatchSeg &seg, int64_t patch, int np
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) rotations += __shfl_xor_sync(FULL, rotations, o);
     // patches above the bound after the last sweep (the others only shared its warp)
-    const unsigned above = __ballot_sync(FULL, mine && mx >= stop2);
+    const unsigned above = __ballot_sync(FULL, mine && mx >= JR_STOP2);
     if (lane == 0) {
         atomicMax(&ctr->jacobi_max_sweeps, (unsigned long long)sweep);
         atomicAdd(&ctr->jacobi_rotations, rotations);
@@ -396,7 +400,7 @@ __device__ __forceinline__ void solve(const PatchSeg &seg, int64_t patch, int np
 template <int RMAX>
 __global__ void __launch_bounds__(jr_warps(RMAX) * 32, jr_blocks(RMAX))
 jacobi_reg_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restrict__ tab, int ntab, int64_t nwarps,
-                  int smem_floats, int max_sweeps, float stop2, DevCounters *ctr) {
+                  int smem_floats, int max_sweeps, DevCounters *ctr) {
     extern __shared__ __align__(16) float jr_sm[];
     const int64_t w = (int64_t)blockIdx.x * jr_warps(RMAX) + (threadIdx.x >> 5);
     if (w >= nwarps) return;
@@ -418,22 +422,22 @@ jacobi_reg_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restri
     float *sm = jr_sm + (threadIdx.x >> 5) * smem_floats;
     if (np <= 0) return;
     switch (R) {
-        case 16: solve<16>(seg, patch, np, sm, max_sweeps, stop2, ctr); break;
-        case 24: solve<24>(seg, patch, np, sm, max_sweeps, stop2, ctr); break;
-        case 32: solve<32>(seg, patch, np, sm, max_sweeps, stop2, ctr); break;
+        case 16: solve<16>(seg, patch, np, sm, max_sweeps, ctr); break;
+        case 24: solve<24>(seg, patch, np, sm, max_sweeps, ctr); break;
+        case 32: solve<32>(seg, patch, np, sm, max_sweeps, ctr); break;
         default:
             if constexpr (RMAX > 32) {
-                if (R == 40) solve<40>(seg, patch, np, sm, max_sweeps, stop2, ctr);
-                else if (R == 48) solve<48>(seg, patch, np, sm, max_sweeps, stop2, ctr);
-                else if (RMAX == 56 || R == 56) solve<56>(seg, patch, np, sm, max_sweeps, stop2, ctr);
-                else if constexpr (RMAX > 56) solve<64>(seg, patch, np, sm, max_sweeps, stop2, ctr);
+                if (R == 40) solve<40>(seg, patch, np, sm, max_sweeps, ctr);
+                else if (R == 48) solve<48>(seg, patch, np, sm, max_sweeps, ctr);
+                else if (RMAX == 56 || R == 56) solve<56>(seg, patch, np, sm, max_sweeps, ctr);
+                else if constexpr (RMAX > 56) solve<64>(seg, patch, np, sm, max_sweeps, ctr);
             }
     }
 }
 
 template <int RMAX>
 cudaError_t launch(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t nwarps, int max_sweeps,
-                   float stop2, DevCounters *ctr, cudaStream_t s) {
+                   DevCounters *ctr, cudaStream_t s) {
     int fl = 0;
     for (int R = 16; R <= jr_rows(kmax); R += 8) fl = fl > jr_floats_r(R) ? fl : jr_floats_r(R);
     constexpr int W = jr_warps(RMAX);
@@ -442,7 +446,7 @@ cudaError_t launch(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax,
                                          (int)smem);
     if (e != cudaSuccess) return e;
     jacobi_reg_kernel<RMAX><<<(unsigned)((nwarps + W - 1) / W), W * 32, smem, s>>>(
-        one, tab, ntab, nwarps, fl, max_sweeps, stop2, ctr);
+        one, tab, ntab, nwarps, fl, max_sweeps, ctr);
     return cudaGetLastError();
 }
 }  // namespace
@@ -450,13 +454,12 @@ cudaError_t launch(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax,
 int64_t jacobi_reg_warps(int k, int64_t np) { return (np + jr_ppw(k) - 1) / jr_ppw(k); }
 
 cudaError_t launch_jacobi_reg(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t nwarps,
-                              int max_sweeps, float stop_cos, DevCounters *ctr, cudaStream_t s) {
+                              int max_sweeps, DevCounters *ctr, cudaStream_t s) {
     if (nwarps <= 0) return cudaSuccess;
     if (kmax > 64 || kmax < 1) return cudaErrorInvalidValue;
-    const float stop2 = stop_cos * stop_cos;
-    if (kmax <= 32) return launch<32>(one, tab, ntab, kmax, nwarps, max_sweeps, stop2, ctr, s);
-    if (kmax <= 56) return launch<56>(one, tab, ntab, kmax, nwarps, max_sweeps, stop2, ctr, s);
-    return launch<64>(one, tab, ntab, kmax, nwarps, max_sweeps, stop2, ctr, s);
+    if (kmax <= 32) return launch<32>(one, tab, ntab, kmax, nwarps, max_sweeps, ctr, s);
+    if (kmax <= 56) return launch<56>(one, tab, ntab, kmax, nwarps, max_sweeps, ctr, s);
+    return launch<64>(one, tab, ntab, kmax, nwarps, max_sweeps, ctr, s);
 }
 
 }  // namespace mecuco

@@ -222,14 +222,6 @@ cudaError_t launch_tthird_tc(const PatchSeg &one, const PatchSeg *tab, int ntab,
 // in two-term FP32, ~2^-48 relative);
 // 2 = every sweep in FP64; 3 = as 1 with the refinement's cluster test
 // relative to each eigenvalue pair (for nearly diagonal Grams).
-// pre_eps is the rotation threshold of the FP32 sweeps of modes 1 and 3: the
-// refinement squares the eigenvector error, so kJacobiPreLoose suffices where
-// the eigenpairs feed the estimator directly (on 100k curved patches, m = 4096,
-// k = 64, kappa moved by <= 3.6e-7 relative and the stage took 8% less time;
-// 2^-11 moved it by 1.4e-4).  Eigenvectors that later rotate a patch, whose
-// rotated Gram must come out nearly diagonal, take kJacobiPreTight.
-constexpr float kJacobiPreTight = 2.384185791015625e-07f;  // 2^-22
-constexpr float kJacobiPreLoose = 6.103515625e-05f;        // 2^-14
 // reg: the leading points solved, with fp64 = 1 and warp_form < 0 (the default),
 // by the register-resident one-sided sweeps (jacobi_reg.cu; 4 to 9 times faster
 // than the fused two-sided form at every k measured) and the refinement through
@@ -255,15 +247,15 @@ constexpr int64_t JACOBI_REG_MIN_M = 128;
 // CTA form.
 cudaError_t launch_jacobi(const float *G, int k, int64_t np, int fp64, int max_sweeps,
                           float *sigma, float *U, DevCounters *ctr, cudaStream_t s,
-                          float pre_eps = kJacobiPreTight, int warp_form = 1, bool reg = false);
+                          int warp_form = 1, bool reg = false);
 // The same over a segment table (PatchSeg: G, k, sig, U of each segment);
 // kmax bounds every segment's k.
 cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t np, int fp64,
-                              int max_sweeps, DevCounters *ctr, cudaStream_t s, float pre_eps, int warp_form = 1,
+                              int max_sweeps, DevCounters *ctr, cudaStream_t s, int warp_form = 1,
                               const JacobiReg &reg = JacobiReg());
 // Register-resident one-sided sweeps: nwarps warps in all, each on
 // jacobi_reg_warps()'s share of one segment's patches (PatchSeg: k, npts,
-// jfirst, G, sig, U); stop_cos bounds |cos| between columns in the last sweep.
+// jfirst, G, sig, U).
 int64_t jacobi_reg_warps(int k, int64_t np);
 inline JacobiReg jacobi_reg_all(int k, int64_t np) {  // every point of a single segment
     JacobiReg r;
@@ -273,7 +265,7 @@ inline JacobiReg jacobi_reg_all(int k, int64_t np) {  // every point of a single
     return r;
 }
 cudaError_t launch_jacobi_reg(const PatchSeg &one, const PatchSeg *tab, int ntab, int kmax, int64_t nwarps,
-                              int max_sweeps, float stop_cos, DevCounters *ctr, cudaStream_t s);
+                              int max_sweeps, DevCounters *ctr, cudaStream_t s);
 
 // ---- Step 4: k-space estimator (randomised SVD) ------------------------------
 // For Ritz pairs (the randomised SVD): sigma/U from launch_rsvd_compose, M
