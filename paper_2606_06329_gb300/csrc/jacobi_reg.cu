@@ -129,6 +129,27 @@ __device__ __forceinline__ void rotation(float al, float be, float ga, float &t,
     }
 }
 
+// The counters of a warp's solve of np patches, H lanes each; above: lanes above the
+// bound in the last sweep.  A patch counts as not converged for itself, not for its
+// warp.  Out of line: inlined, it made the R <= 56 kernel spill three times as much.
+__device__ __noinline__ void report(unsigned long long rotations, unsigned above, int np, int H, int sweep,
+                                    DevCounters *ctr) {
+    constexpr unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, g = lane / H;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) rotations += __shfl_xor_sync(FULL, rotations, o);
+    const unsigned missed =
+        __ballot_sync(FULL, g < np && lane == g * H && ((above >> lane) & (FULL >> (32 - H))) != 0u);
+    if (lane == 0) {
+        atomicMax(&ctr->jacobi_max_sweeps, (unsigned long long)sweep);
+        atomicAdd(&ctr->jacobi_rotations, rotations);
+        if (missed) {
+            atomicAdd(&ctr->jacobi_not_converged, (unsigned long long)__popc(missed));
+            atomicOr(&ctr->status, (unsigned)DEV_NOT_CONVERGED);
+        }
+    }
+}
+
 // Eigenvectors of up to 32 / (R / 2) patches of one warp, starting at `patch`
 // (np of them); sm: the warp's jr_floats_r(R) shared floats.
 template <int R>
@@ -271,11 +292,10 @@ __device__ __forceinline__ void solve(const PatchSeg &seg, int64_t patch, int np
     };
     int sweep = 0, seam = H - 1;
     unsigned long long rotations = 0;
-    bool converged = false;
-    float mx = 0.f;  // largest squared cosine that this lane met in the sweep
+    unsigned above = FULL;  // lanes whose patch was above the bound in the last sweep
     while (sweep < max_sweeps) {
         float al = dot_cols<NP>(X, X), be = dot_cols<NP>(Y, Y);
-        mx = 0.f;
+        float mx = 0.f;
         unsigned nrot = 0;
         for (int rr = 0; rr < H; ++rr) {
             float t, c, cos2, ga;
@@ -332,9 +352,10 @@ __device__ __forceinline__ void solve(const PatchSeg &seg, int64_t patch, int np
         ++sweep;
         rotations += nrot;
         if (__all_sync(FULL, !(mx >= JR_STOP2))) {
-            converged = true;
+            above = 0u;
             break;
         }
+        if (sweep == max_sweeps) above = __ballot_sync(FULL, mx >= JR_STOP2);
     }
     // ---- eigenpairs sorted descending
     const float al = dot_cols<NP>(X, X), be = dot_cols<NP>(Y, Y);
@@ -379,20 +400,7 @@ __device__ __forceinline__ void solve(const PatchSeg &seg, int64_t patch, int np
         for (int r = 0; r < k; ++r)
             for (int c = li; c < k; c += H) u[r * k + c] = S[c * LDU + r];
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) rotations += __shfl_xor_sync(FULL, rotations, o);
-    // patches above the bound after the last sweep (the others only shared its warp)
-    const unsigned above = __ballot_sync(FULL, mine && mx >= JR_STOP2);
-    if (lane == 0) {
-        atomicMax(&ctr->jacobi_max_sweeps, (unsigned long long)sweep);
-        atomicAdd(&ctr->jacobi_rotations, rotations);
-        if (!converged) {
-            unsigned missed = 0;
-            for (int p = 0; p < PPW; ++p) missed += ((above >> (p * H)) & (FULL >> (32 - H))) != 0u;
-            atomicAdd(&ctr->jacobi_not_converged, (unsigned long long)missed);
-            atomicOr(&ctr->status, (unsigned)DEV_NOT_CONVERGED);
-        }
-    }
+    report(rotations, above, np, H, sweep, ctr);
 }
 
 // One warp per group of patches; RMAX bounds every patch's R.  The bodies with
