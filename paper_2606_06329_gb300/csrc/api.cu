@@ -70,9 +70,10 @@ struct mecuco_ctx {
     int chunk_share = 1;  // concurrent lanes sharing the chunk budget (batched calls)
     int tc_slots = 4;
     // third-moment pass: TMEM slots of the A operand and CTAs per SM; two CTAs
-    // of 256 columns (2 tiles per pass, 9 passes at k = 64) interleave their
-    // hand-over pipelines: 177 against 251 ms for one CTA of 512 columns at
-    // 100k x 4096 (6 or 8 slots in one CTA: 275 / 261 ms; 2 slots in two: 289 ms)
+    // of 256 columns (2 tiles per pass, 5 passes at k = 64, 9 with every pair)
+    // interleave their hand-over pipelines: with every pair 177 against 251 ms for
+    // one CTA of 512 columns at 100k x 4096 (6 or 8 slots in one CTA: 275 / 261 ms; 2
+    // slots in two: 289 ms)
     int tt_slots = 4;
     int tt_ctas = 2;
     // randomised low-rank SVD (mecuco_curvature_rsvd), set for the duration of a call
@@ -230,9 +231,10 @@ int candidate_capacity(mecuco_t h, int k) {
 }
 
 // CTA pairs (256 x 256 two-SM MMAs, two thirds of the operand bytes per MMA) from
-// this row length of the BF16 operands on: single / pair search time 1.10 at K =
-// 4096, 1.17 at 2352, 0.97 at 2048, 0.92 at 1024, 0.87 at 512 (100,000 points;
-// 0.92 at 200,000 x 1024, 1.05 at 20,000 x 4096).
+// this row length of the BF16 operands on, which lies between two measured ones:
+// single / pair search time 1.14 at K = 4096, 1.21 at 2352, 0.97 at 2048, 0.92 at 1024,
+// 0.88 at 512 (100,000 points, 70,000 at 2352; 0.94 at 200,000 x 1024, 1.08 at 20,000 x
+// 4096).
 constexpr int64_t KNN_PAIR_MIN_K = 2200;
 
 struct KnnPlan {
@@ -308,8 +310,9 @@ KnnPlan plan_knn(mecuco_t h, const void *X, mecuco_dtype dt, int64_t N, int64_t 
     // instead of 4 waves).  A split shortens the search but gives every row
     // another set of lists to re-rank; the model weighs the two, in ns.  A wave
     // costs, per tile of 256 candidates, max(4000, 7.5 K) on the tensor cores (the
-    // drain, or the operands' way from L2) and 4500 + 122 m on the CUDA cores; a row's set of lists 3 per 128 entries in the re-rank (reading
-    // and selecting: it evaluates k + 16 candidates however many there are).
+    // drain, or the operands' way from L2) and 4500 + 122 m on the CUDA cores; a row's
+    // set of lists 3 per 128 entries in the re-rank (reading and selecting: it
+    // evaluates k + 33 candidates however many there are).
     const double tile = p.tc ? std::max(4000.0, 7.5 * (double)p.mk) : 4500.0 + 122.0 * (double)m;
     const int64_t item_rows = p.tc ? knn_tc_item_rows(p.pair) : 128;
     const double waves1 = (double)((N + 255) / 256) * tile, rr = 3.0 * p.halves * p.kcl / 128;

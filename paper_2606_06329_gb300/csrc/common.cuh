@@ -70,9 +70,6 @@ __device__ __forceinline__ float load_elem(const __nv_bfloat16 *p) {
     return __bfloat162float(__ldg(reinterpret_cast<const __nv_bfloat16 *>(p)));
 }
 
-__device__ __forceinline__ float to_f32(float v) { return v; }
-__device__ __forceinline__ float to_f32(__nv_bfloat16 v) { return __bfloat162float(v); }
-
 // --- error-free transformations (Knuth TwoSum, FMA-based TwoProd) ----------
 // A value is carried as an unevaluated sum hi + lo with |lo| <= ulp(hi)/2.
 struct ff {
@@ -126,10 +123,6 @@ __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
     return v;
-}
-
-__device__ __forceinline__ void atomic_max_u64(unsigned long long *p, unsigned long long v) {
-    atomicMax(p, v);
 }
 
 // Order of eigenpairs: descending, the lower index first on ties, NaN last.  A total

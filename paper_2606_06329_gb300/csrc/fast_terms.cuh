@@ -46,8 +46,9 @@ __device__ __forceinline__ int fast_rank(const float *__restrict__ sg, int k, in
 // the Haar variant only), R and the eigenvalues sg in global memory; c_s (64) and
 // red (a row per warp): scratch in shared memory.  Called by all THREADS threads (k <=
 // 64 <= THREADS), Us, Qs and diag visible to all.
-// The sums are two-term FP32 (2^-44 and better): FP64 runs at 1/64 of the FP32
-// rate.  A CTA has nothing else to do meanwhile, so what counts is the length of
+// The sums of squares, the quadratic forms' sums over the rows of Q and tau are
+// two-term FP32 (2^-44 and better); c_l, the entries of U c and the products Q u are
+// FP32 chains of at most 64 terms.  FP64 runs at 1/64 of the FP32 rate.  A CTA has nothing else to do meanwhile, so what counts is the length of
 // the dependent chains: the sums of squares and the k quadratic forms of Q are
 // spread over all threads, eight lanes to a form, and the two reciprocals in FP64
 // are computed beside them (one thread per form: 44,000 of the 95,000 cycles that a

@@ -647,9 +647,10 @@ size_t refine_ff_smem_bytes(int k) {
 // One k^3 two-term product and two FP32 ones, no FP64, against two and a half
 // two-term products at ten operations a term, one FP32 product and k^2 FP64
 // divisions (GB300 has 1/64 of the FP32 rate in FP64).
-// Measured on GB300 per 100k patches: k = 64 9.4 ms (two-term products: 52),
-// k = 37 3.3 (12), k = 32 1.6 (6.7); U^T U - I and the off-diagonals of U^T A U
-// as with the two-term products (5e-7, 1.3e-8 lam_1).  FMA-issue bound.
+// Measured on GB300 per 100k patches, first order alone: k = 64 9.4 ms (two-term
+// products: 52), k = 37 3.3 (12), k = 32 1.6 (6.7); the exchange of the numerators and
+// the second order add 0.5% to a forward pass.  U^T U - I and the off-diagonals of U^T
+// A U as with the two-term products (5e-7, 1.3e-8 lam_1).  FMA-issue bound.
 // Every thread forms 4 x 4 blocks from 16-byte shared loads, two columns per
 // packed FP32 instruction.
 // ---------------------------------------------------------------------------

@@ -39,17 +39,18 @@
 // to 2^-24 of the column norms, i.e. G to 2^-24 (lambda + eps), and G carries
 // noise of 2^-24 lambda_1 anyway.
 //
-// Measured (GB300, 2.07 GHz, per 100k patches of the curved-patch spectrum):
-// k = 64 28 ms, k = 50 21 ms, k = 37 10.2 ms, k = 32 3.3 ms, k = 24 2.1 ms,
-// against 127, 68, 40, 31 and 20 ms for the fused two-sided sweeps; after the
+// Measured (GB300, 2.07 GHz, per 100k patches of the curved-patch spectrum at 1,024
+// columns, with the refinement): k = 64 42.2 ms, k = 50 31.2, k = 37 14.9, k = 32 5.4, k =
+// 24 3.8 (37.7, 27.7, 13.5, 5.0 and 3.4 with the bound 2^-10 and the refinement of first
+// order alone; the fused two-sided sweeps alone 127, 68, 40, 31 and 20); after the
 // refinement U^T U - I is at most 1e-6, against 4e-5 to 2e-4.
-// What bounds it: latency at the warps that fit (252 registers a thread at
-// R = 64, no spills, two warps per scheduler, issue 41% busy, 150k warp
-// instructions per patch; three warps at 168 registers spill and take 10%
-// longer, R <= 56 fits three and R <= 32 four).  The floor per round and warp at
-// R = 64 is 64 shuffles (one warp instruction per clock per SM) and 32 + 96
-// packed FMAs: about 8 warp instructions per rotation, against about 96 and 8
-// to 16 shared-memory words per row pair in jacobi_warp_kernel.
+// What bounds it: latency at the warps that fit (254 registers a thread at R = 64, no
+// spills, two warps per scheduler, 150k warp instructions per patch; three warps at 168
+// registers spill more than they hide and take 10% longer).  R <= 56 runs three warps
+// per scheduler at 168 registers and spills 480 bytes a thread, R <= 32 four.  The floor
+// per round and warp at R = 64 is 64 shuffles (one warp instruction per clock per SM)
+// and 32 + 96 packed FMAs: about 8 warp instructions per rotation, against about 96 and
+// 8 to 16 shared-memory words per row pair in jacobi_warp_kernel.
 #include <math.h>
 
 #include "common.cuh"

@@ -50,7 +50,7 @@ cudaError_t launch_knn_simt(const void *X, mecuco_dtype dt, int64_t N, int64_t m
 // and Xb (candidate operand) are BF16 row-major with K = m columns, ldb % 8 ==
 // 0 and 16-byte aligned bases: both X itself when it is stored that way, both
 // the copy of launch_row_prep, or its two copies of the split (then
-// m is their K = 3 ms).  kc is 32 or 64; lists come out in ascending order.
+// m is their K = 3 ms).  kc <= 64; a list's entries come in no order.
 // pair != 0 (and nq >= 256): CTA pairs sharing 256 x 256 cta_group::2 MMAs;
 // the lists are the same.  wait_limit: clock cycles after which a wait of the
 // work loops gives up (MECUCO_ERR_TIMEOUT); <= 0 selects the default (~0.5 s).
@@ -59,7 +59,6 @@ cudaError_t launch_knn_tc(const void *Xa, const void *Xb, int64_t N, int64_t m, 
                           int64_t q0, int64_t nq, int kc, int nsplit, int include_self,
                           float *cand_d, int32_t *cand_i, int pair, long long wait_limit, DevCounters *ctr,
                           cudaStream_t s);
-size_t knn_tc_smem_bytes();
 // Candidate lists the tensor-core search leaves per row and split (the epilogue's
 // column halves); list h of row r, split s starts at ((r nsplit + s) halves + h) kc.
 int knn_tc_halves();

@@ -533,11 +533,11 @@ cudaError_t launch_knn_simt(const void *X, mecuco_dtype dt, int64_t N, int64_t m
 // whose lists' own threshold (the smallest maximum of the full lists) does not
 // pass the test are re-solved exactly by the full scan.
 // Measured per 100k queries against the form that evaluated and ranked every
-// candidate: 512 columns BF16, k = 32, 128 candidates 6.4 to 2.5 ms; per 70k of
-// 784 FP32 columns, k = 50 6.7 to 3.6 ms; 2,000 x 32 with 1,024 candidates a row
-// 2.98 to 0.04 ms.  Bound by the FP32 pipe (12 operations a term, in packed
-// pairs, 22 before) up to about 1,000 columns, then by the candidate rows' DRAM
-// reads.
+// candidate: 512 columns BF16, k = 32, 128 candidates 6.4 to 3.0 ms (2.6 without the
+// sample); per 70k of 784 FP32 columns, k = 50 6.7 to 4.1 ms (3.7); 2,000 x 32 with
+// several hundred candidates a row 2.98 to 0.03 ms.  Bound by the FP32 pipe (12
+// operations a term, in packed pairs, 22 before) up to about 1,000 columns, then by
+// the candidate rows' DRAM reads.
 // ---------------------------------------------------------------------------
 constexpr int RR_WARPS = 4;
 constexpr int RR_MAXL = 1024;

@@ -34,7 +34,7 @@
 // them cancels in the re-rank's certificate, which estimates the error from the row's
 // own candidates.  Running the blocks backward on every second tile reads a third
 // less from DRAM (89 against 133 GB for 19,456 queries and 210,000 points of 4,096;
-// 4% of the search) but leaves two errors per row, by the parity of the candidate's
+// 62,500 queries against 1,000,000 points of 4,096 417 instead of 391 ms) but leaves two errors per row, by the parity of the candidate's
 // tile: on clusters off the origin (2,048 BF16 rows of 4,096 columns, noise 1 to 2% of
 // the centre) up to 2,048 of 2,048 rows came out certified and wrong.
 // CTA pairs (optional, for 256 or more query rows): two CTAs of a
@@ -47,8 +47,8 @@
 // epilogue warps of both CTAs release an accumulator at the even CTA.  The
 // lists are those of the single-CTA form.  It moves 2/3 of the operand bytes
 // per MMA and so wins where those bound the search, at long rows: 100,000 points
-// 62.4 against 68.8 ms at K = 4096, 70,000 x 784 FP32 rows (K = 2352) 19.4
-// against 22.7 ms, but 32.3 against 31.2 ms at K = 2048 and 15.6 against 13.7 ms
+// 64.0 against 73.1 ms at K = 4096, 70,000 x 784 FP32 rows (K = 2352) 17.8
+// against 21.6 ms, but 31.1 against 30.3 ms at K = 2048 and 13.8 against 12.1 ms
 // at K = 512, where the drain bounds it.
 // Every mbarrier wait is bounded; a timeout sets MECUCO_ERR_TIMEOUT in the
 // device status word, raises a CTA-wide abort flag, drains the copies and MMAs
@@ -647,7 +647,7 @@ bool make_map(CUtensorMap *map, const void *Xb, int64_t N, int64_t m, int64_t ld
 }
 }  // namespace
 
-size_t knn_tc_smem_bytes(int kc) {
+static size_t knn_tc_smem_bytes(int kc) {
     return 1024 + (size_t)NSTAGE * STAGE_BYTES + (size_t)TC_HALVES * kc * TBM * (sizeof(float) + 1) + sizeof(TcShared) +
            64;
 }

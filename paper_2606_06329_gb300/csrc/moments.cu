@@ -20,11 +20,11 @@
 // adjoint uses this.
 //
 // A chunk is MCH columns: gathered row by row (a warp per row, a lane per
-// column, the next chunk's values on their way in registers), centred (a lane per column, the rows shared between the warps: in
-// two-term FP32 for the rotated form, whose small directions would show the
-// rounding of the means), then rotated, or copied, into column-major order, which
-// is what 16-byte operand loads want.  Every sum of a result runs in ascending
-// order of the column in one thread.
+// column, the next chunk's values on their way in registers), centred (a lane per
+// column, the rows shared between the warps: in two-term FP32 for the rotated form,
+// whose small directions would show the rounding of the means), then rotated, or
+// copied, into column-major order, which is what 16-byte operand loads want.  Every
+// sum of a result runs in ascending order of the column in one thread.
 #include <math.h>
 
 #include "common.cuh"

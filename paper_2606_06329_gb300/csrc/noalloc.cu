@@ -116,7 +116,9 @@ extern "C" MECUCO_API mecuco_status mecuco_knn_noalloc(const void *X, mecuco_dty
     if (cudaGetDevice(&dev) != cudaSuccess) return MECUCO_ERR_CUDA;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return MECUCO_ERR_CUDA;
 
-    // candidate capacity and work split as mecuco_knn's plain form (margin 32)
+    // candidate capacity as mecuco_knn's plain form (margin 32); the candidate range
+    // split for two blocks per SM as far as the fixed scratch allows (one fits, so that
+    // is twice the splits that fill the SMs)
     int kc = (k + 32 + 31) / 32 * 32;
     if (kc > 128) kc = 128;
     // layout: counters | norms (N) | flags (qchunk) | cand_d, cand_i (qchunk * nsplit * kc)
