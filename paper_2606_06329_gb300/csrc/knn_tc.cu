@@ -34,9 +34,10 @@
 // them cancels in the re-rank's certificate, which estimates the error from the row's
 // own candidates.  Running the blocks backward on every second tile reads a third
 // less from DRAM (89 against 133 GB for 19,456 queries and 210,000 points of 4,096;
-// 62,500 queries against 1,000,000 points of 4,096 417 instead of 391 ms) but leaves two errors per row, by the parity of the candidate's
-// tile: on clusters off the origin (2,048 BF16 rows of 4,096 columns, noise 1 to 2% of
-// the centre) up to 2,048 of 2,048 rows came out certified and wrong.
+// 62,500 queries against 1,000,000 points 391 instead of 417 ms) but leaves two errors
+// per row, by the parity of the candidate's tile: on clusters off the origin (2,048
+// BF16 rows of 4,096 columns, noise 1 to 2% of the centre) up to 2,048 of 2,048 rows
+// came out certified and wrong.
 // CTA pairs (optional, for 256 or more query rows): two CTAs of a
 // thread-block cluster share one 256 x 256 tcgen05.mma (cta_group::2, M = 256)
 // per K step.  Each CTA loads its own 128 query rows and one 128-row half of
