@@ -308,7 +308,7 @@ def _stage_fracs(stages, steps, shapes, prec, rotations, peaks, elt=2):
     (CUDA events around every launch).  shapes: the (N, m, k) of every dataset
     of the step; the algorithmic work per stage is summed over them:
       knn_search  2 N^2 m FLOP (tensor, BF16; FP32 lanes in the plain form)
-      knn_rerank  N x (k + 16) candidate rows x m x elt bytes read, against HBM
+      knn_rerank  N x (k + 32) candidate rows x m x elt bytes read, against HBM
       gram        the gathered patches, N k m elements, against HBM
       rotate      the gathered patches plus the rotated patches written
                   (N x k rows x m BF16), against HBM
@@ -327,7 +327,7 @@ def _stage_fracs(stages, steps, shapes, prec, rotations, peaks, elt=2):
     for N, m, k in shapes:
         N, m, k = float(N), float(m), float(k)
         tot["knn_search"] += 2.0 * N * N * m
-        tot["knn_rerank"] += N * (k + 16.0) * m * elt
+        tot["knn_rerank"] += N * (k + 32.0) * m * elt  # the k + 16 nearest and the sample
         tot["gram"] += N * k * m * elt
         tot["rotate"] += N * k * m * elt + N * k * m * 2.0
         tot["moments"] += 2.0 * k * (k + 1) * (k + 2) / 6.0 * m * N
