@@ -1359,7 +1359,7 @@ mecuco_status mecuco_curvature_backward(mecuco_t h, const void *X, mecuco_dtype 
         // which ill-conditioned patches amplify)
         LAUNCH(h, MECUCO_STAGE_GRAM, s,
                launch_patch_gram(X, dt, N, m, ld, nb, k, 0, np, nullptr, b.G, b.R, nullptr, h->ctr, s));
-        LAUNCH(h, MECUCO_STAGE_JACOBI, s, launch_jacobi(b.G, k, np, 1, h->jacobi_max_sweeps, b.sig, U0, h->ctr, s,
+        LAUNCH(h, MECUCO_STAGE_JACOBI, s, launch_jacobi(b.G, k, np, 4, h->jacobi_max_sweeps, b.sig, U0, h->ctr, s,
                                  h->jacobi_warp));
         ++h->launches;  // the refinement kernel
         // moments of Z = U0^T X_c and the refined eigenpairs of its Gram

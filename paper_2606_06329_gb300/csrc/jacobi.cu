@@ -426,8 +426,10 @@ cudaError_t launch_jacobi_warp(const PatchSeg &one, const PatchSeg *tab, int nta
 // |lam_j|), for Grams whose FP32 eigenpairs are accurate relative to each
 // eigenvalue (a nearly diagonal Gram, as in the adjoint's rotated basis).  With rel =
 // 0 a pair whose correction would exceed REFINE_MAX_E is taken as one of a cluster
-// too (the relative test leaves 2^-22 / 2^-18 at most), and from REFINE_FIRST_ORDER
-// on the second order is added, X' = X + X E + X E^2 / 2.
+// too, and from REFINE_FIRST_ORDER on the second order is added, X' = X + X E + X E^2 /
+// 2.  With rel = 1 neither: among the null vectors of a rank-deficient patch any
+// noise is a gap relative to the pair, their corrections are as large as they like, and
+// a second order would square them (nothing that the adjoint uses reads them).
 // (With delta alone and the first order, 64 eigenvalues 2^-12 or 2^-16 apart came out
 // with U^T U - I up to 700: what the sweeps leave off the diagonal is not small beside
 // such gaps.)
@@ -465,12 +467,17 @@ __device__ __forceinline__ int tri(int a, int b, int k) { return a * k - (a * (a
 constexpr int FT_REFINE = 256;
 // Largest correction E_ij of a pair, and the largest up to which X (I + E) will do: the
 // step is of first order and leaves E^2 of U^T U - I; beyond, E^2 / 2 is added, which
-// leaves E^4 / 4 (the skew part's exponential to second order).
+// leaves E^4 / 4 (the skew part's exponential to second order).  Eigenvectors that only
+// rotate a patch (the adjoint's U0) take the second order from REFINE_ROTATION on: it
+// moves the last bits of U0, and the gradient with them, for what 2^-16 of
+// orthogonality in a near-degenerate pair is worth.
 constexpr float REFINE_MAX_E = 0.0078125f;              // 2^-7
 constexpr float REFINE_FIRST_ORDER = 2.44140625e-04f;   // 2^-12
+constexpr float REFINE_ROTATION = 0.00390625f;          // 2^-8
 
 template <int NT>
-__device__ __forceinline__ void refine_ff_patch(const PatchSeg &seg, int local, int rel, unsigned char *fsm) {
+__device__ __forceinline__ void refine_ff_patch(const PatchSeg &seg, int local, int rel, float first_order,
+                                                unsigned char *fsm) {
     const int k = seg.k;
     const float *G = seg.G;
     float *sigma = seg.sig, *U = seg.U;
@@ -581,7 +588,7 @@ __device__ __forceinline__ void refine_ff_patch(const PatchSeg &seg, int local, 
         double v;
         if (i == j || fabs(gap) <= dij || (!rel && num > (double)REFINE_MAX_E * fabs(gap))) v = 0.5 * rij;
         else v = (sij + lam[j] * rij) / gap;  // (a NaN stays one)
-        large = large || fabs(v) > (double)REFINE_FIRST_ORDER;
+        large = large || fabs(v) > (double)first_order;
         Ef[i * ld + j] = (float)v;
     }
     const bool second = __syncthreads_or(large);
@@ -615,11 +622,12 @@ __device__ __forceinline__ void refine_ff_patch(const PatchSeg &seg, int local, 
 
 template <int NT>
 __global__ void __launch_bounds__(NT, 512 / NT)
-jacobi_refine_ff_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restrict__ tab, int ntab, int rel) {
+jacobi_refine_ff_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restrict__ tab, int ntab, int rel,
+                        float first_order) {
     extern __shared__ __align__(16) unsigned char fsm[];
     int local;
     const PatchSeg &seg = find_seg(one, tab, ntab, (int)blockIdx.x, local);
-    refine_ff_patch<NT>(seg, local, rel, fsm);
+    refine_ff_patch<NT>(seg, local, rel, first_order, fsm);
 }
 
 size_t refine_ff_smem_bytes(int k) {
@@ -901,7 +909,7 @@ jacobi_refine_res_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *_
     int local;
     const PatchSeg &seg = find_seg(one, tab, ntab, (int)blockIdx.x, local);
     if (ntab == 0 || (int)(&seg - tab) < nres) refine_res_patch<NT>(seg, local, rsm);
-    else refine_ff_patch<NT>(seg, local, 0, reinterpret_cast<unsigned char *>(rsm));
+    else refine_ff_patch<NT>(seg, local, 0, REFINE_FIRST_ORDER, reinterpret_cast<unsigned char *>(rsm));
 }
 
 size_t jacobi_smem_bytes(int k, int fp64) {
@@ -930,8 +938,8 @@ cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab
         jacobi_kernel<float><<<(unsigned)n, JT, smem, s>>>(one, t, nt, (int)blk0, max_sweeps, eps, ctr);
         return cudaGetLastError();
     };
-    if (fp64 == 1 || fp64 == 3) {
-        // FP32 sweeps, then one refinement step (3: relative cluster test)
+    if (fp64 == 1 || fp64 == 3 || fp64 == 4) {
+        // FP32 sweeps, then one refinement step (3: relative cluster test; 4: a rotation)
         const bool fast = reg.np > 0 && fp64 == 1 && warp_form < 0;
         if (fast) {
             PatchSeg seg = one;
@@ -965,7 +973,8 @@ cudaError_t launch_jacobi_seg(const PatchSeg &one, const PatchSeg *tab, int ntab
         auto refine = [&](auto kern, int nt) -> cudaError_t {
             cudaError_t r = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rs);
             if (r != cudaSuccess) return r;
-            kern<<<(unsigned)np, nt, rs, s>>>(one, tab, ntab, fp64 == 3);
+            const float first = fp64 == 3 ? INFINITY : fp64 == 4 ? REFINE_ROTATION : REFINE_FIRST_ORDER;
+            kern<<<(unsigned)np, nt, rs, s>>>(one, tab, ntab, fp64 == 3, first);
             return cudaGetLastError();
         };
         if (kmax <= 16) return refine(jacobi_refine_ff_kernel<64>, 64);

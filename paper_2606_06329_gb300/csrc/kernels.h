@@ -220,7 +220,8 @@ cudaError_t launch_tthird_tc(const PatchSeg &one, const PatchSeg *tab, int ntab,
 // fp64: 0 = FP32 sweeps; 1 = FP32 sweeps then one refinement step (products
 // in two-term FP32, ~2^-48 relative);
 // 2 = every sweep in FP64; 3 = as 1 with the refinement's cluster test
-// relative to each eigenvalue pair (for nearly diagonal Grams).
+// relative to each eigenvalue pair (for nearly diagonal Grams); 4 = as 1 for
+// eigenvectors that only rotate the patch (the adjoint).
 // reg: the leading points solved, with fp64 = 1 and warp_form < 0 (the default),
 // by the register-resident one-sided sweeps (jacobi_reg.cu; 4 to 9 times faster
 // than the fused two-sided form at every k measured) and the refinement through
