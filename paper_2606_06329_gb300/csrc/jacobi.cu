@@ -42,6 +42,15 @@ struct JacobiEps<double> {
     static __host__ __device__ __forceinline__ double rel() { return 8.8817841970012523e-16; }  // 2^-50
 };
 
+// sqrt(|a b|); by the factors' roots where the product leaves FP32's normal range
+// (entries beyond 2^64 and below 2^-63: the Grams of points beyond 1e9 or below 1e-9),
+// where the sweeps would not rotate at all, or by anything.
+__device__ __forceinline__ float geometric_mean(float a, float b) {
+    const float p = fabsf(a * b);
+    return p < INFINITY && p > 1.17549435e-38f ? sqrtf(p) : sqrtf(fabsf(a)) * sqrtf(fabsf(b));
+}
+__device__ __forceinline__ double geometric_mean(double a, double b) { return sqrt(fabs(a * b)); }
+
 constexpr int JT = 128;  // threads per patch
 
 // One rotation of a round's table, read by every walker as one 16-byte (FP32)
@@ -102,7 +111,7 @@ jacobi_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restrict__
                 else { a = (round + tid) % (kp - 1); b = (round + kp - 1 - tid) % (kp - 1); }
                 const int p = a < b ? a : b, q = a < b ? b : a;
                 const Real app = A[p * ld + p], aqq = A[q * ld + q], apq = A[p * ld + q];
-                if (fabs(apq) > eps * sqrt(fabs(app * aqq)) && apq != (Real)0) {
+                if (fabs(apq) > eps * geometric_mean(app, aqq) && apq != (Real)0) {
                     const Real tau = (aqq - app) / (2 * apq);
                     const Real t = (tau >= 0 ? (Real)1 : (Real)-1) / (fabs(tau) + sqrt((Real)1 + tau * tau));
                     const Real c = (Real)1 / sqrt((Real)1 + t * t);
@@ -276,7 +285,7 @@ jacobi_warp_kernel(const __grid_constant__ PatchSeg one, const PatchSeg *__restr
                     const int p = a < b ? a : b, q = a < b ? b : a;
                     float c = 1.f, sn = 0.f;
                     const float app = A[p * ld + p], aqq = A[q * ld + q], apq = A[p * ld + q];
-                    if (fabsf(apq) > eps * sqrtf(fabsf(app * aqq)) && fabsf(apq) > thr && apq != 0.f) {
+                    if (fabsf(apq) > eps * geometric_mean(app, aqq) && fabsf(apq) > thr && apq != 0.f) {
                         const float tau = (aqq - app) / (2 * apq);
                         const float t = (tau >= 0 ? 1.f : -1.f) / (fabsf(tau) + sqrtf(1.f + tau * tau));
                         c = 1.f / sqrtf(1.f + t * t);
